@@ -299,11 +299,11 @@ def run_sweep(args):
 def run_walls(args, peak):
     """Walled channel (no-slip walls on rows 0 and ny-1, body force): FP32 step throughput of
     both models (periodic strip kernel on the whole lattice, then the wall bands recomputed by
-    the wall kernel; two launches per step) on a size x size plate channel (vapour below, liquid above, sine-perturbed
+    the tile kernel; two launches per step) on a size x size plate channel (vapour below, liquid above, sine-perturbed
     interface, F_x = 1e-6), CUDA events around 500 steps on the launching stream; and the
     wall-clock rate of the 101 x 50 FP64 channel of Sec. 5.3 (steps/s over 2e4 steps); and the
-    droplet-collision drive of Sec. 5.4: steps/s of the 200 x 100 FP64 pair (a domain-mean
-    reduction plus a direct step per step), and FP32 throughput of a size x size pair (the
+    droplet-collision drive of Sec. 5.4: steps/s of the 200 x 100 FP64 pair (the tile kernel,
+    rho_ave from the masses the previous step stored), and FP32 throughput of a size x size pair (the
     driven strip kernels, rho_ave from the masses the previous step stored; one reduction per
     64-step graph)."""
     import numpy as np
@@ -333,8 +333,8 @@ def run_walls(args, peak):
             out[key] = {"mlups": size * size / s / 1e6, "us_per_launch": s * 1e6,
                         "algorithmic_bytes_per_cell": BYTES_PER_CELL[model], "gbs": gbs,
                         "frac_of_hbm": gbs / peak,
-                        "kernels": ("pp_step_pair + pp_step_ext (wall bands, 2 rows)",
-                                    "fe_step_pair + fe_step_ext (wall bands, 3 rows)")[model]}
+                        "kernels": ("pp_step_pair + tile_step (wall bands, 2 rows)",
+                                    "fe_step_pair + tile_step (wall bands, 3 rows)")[model]}
             ctx.close()
         rates = {}
         for model, key in ((0, "pseudopotential"), (1, "free_energy")):
@@ -352,7 +352,7 @@ def run_walls(args, peak):
             rates[key] = 20000 / (time.perf_counter() - t)
             ctx.close()
         out["sec53_channel_f64_steps_per_s"] = rates
-        # Sec. 5.4: droplet pair driven together (FP64: reduction + direct step; FP32: driven strip kernels)
+        # Sec. 5.4: droplet pair driven together (FP64: driven tile kernel; FP32: driven strip kernels)
         col = {}
         for model, key in ((0, "pseudopotential"), (1, "free_energy")):
             kw = dict(a=0.25, Tr=0.8, tau_nu=1.0)

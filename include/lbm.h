@@ -82,7 +82,7 @@ typedef enum { LBM_GEOMETRY_FLAT = 0, LBM_GEOMETRY_DROPLET = 1 } lbm_geometry;
  *   A           viscosity-tuning term of the free-energy equilibrium, Eq. (20) (the strain-
  *               rate terms); nu = c_s^2 (tau_nu - 1/2 - A) must be positive (Eq. 23).  Free
  *               energy only (A != 0 with the pseudopotential model: LBM_ERR_UNSUPPORTED).
- *               A != 0 runs the full free-energy kernel (direct loads, one more ring level).
+ *               A != 0 runs the full free-energy kernels (one more level: u at the neighbours).
  *   body_fx/fy  constant body force added to the total force of either model. */
 typedef struct {
     int model;       /* lbm_model */
@@ -151,7 +151,7 @@ int lbm_resolve_params_many(int n, const lbm_params* in, lbm_params* out, lbm_th
 /* Bytes of device workspace a context of this size and precision needs: two population
  * buffers (nine planes, plus the rest-population extension plane for FP32), four fields for
  * the observables, reduction partials, the one-sided walls' row solve (14 nx reals) and one
- * double per strip warp for the droplet-collision drive's stored mass (Sec. 5.4). */
+ * double per strip warp or tile row for the droplet-collision drive's stored mass (Sec. 5.4). */
 size_t lbm_workspace_bytes(int precision, int nx, int ny);
 
 /* Create a context for an nx x ny lattice (nx, ny >= 1).  Boundaries: bc_x must be
@@ -206,11 +206,9 @@ int lbm_set_gravity(lbm_ctx* ctx, double g, double rho_ref, double y_ref);
  * rho_ave the mean density of that state.  The force is external: it enters the total force
  * (velocity, forcing moments) but not the interaction force of the sigma^Li term (Eq. 32).
  * Sec. 5.4 uses ax_lo = 5e-6, ax_hi = -5e-6, x_split = 100, t_on = 2000 on a 200 x 100 lattice.
- * FP32 lattices on the strip kernels run their driven instantiation: each step also sums the
- * populations it stores, which is the next state's mass, and the block-sum reduction runs
- * only at the first step of each captured 64-step graph and at single steps.  FP64 and other
- * shapes reduce every step and run the direct kernels.  The two differ only in the summation
- * order of rho_ave.  Errors: LBM_ERR_ARG for a non-finite value, LBM_ERR_UNSUPPORTED with walls (the
+ * Driven steps also sum the populations they store, which is the next state's mass; the
+ * reduction over the populations runs only at the first step of each captured 64-step graph and
+ * at single steps.  The step kernels differ only in the summation order of rho_ave.  Errors: LBM_ERR_ARG for a non-finite value, LBM_ERR_UNSUPPORTED with walls (the
  * reduction sums the stored populations of a periodic lattice).  Synchronises the stream. */
 int lbm_set_drive(lbm_ctx* ctx, double ax_lo, double ax_hi, double x_split, long long t_on);
 

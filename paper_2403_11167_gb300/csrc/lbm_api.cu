@@ -19,6 +19,7 @@
 #include "step_pair.cuh"
 #include "step_ext.cuh"
 #include "step_iwb_pair.cuh"
+#include "tile.h"
 #include "rest_host.h"
 #include "thermo.h"
 
@@ -37,8 +38,6 @@ int cuda_fail(cudaError_t e, const char* what) {
         if (e_ != cudaSuccess) return cuda_fail(e_, #call);   \
     } while (0)
 
-constexpr int kTXf = 256;  // columns per CTA of the FP32 direct-load kernels
-constexpr int kTXd = 64;   // columns per CTA, FP64
 constexpr int kWallBandPP = 2;  // rows next to each wall that a periodic step gets wrong
 constexpr int kWallBandFE = 3;
 constexpr int kGraphSteps = 64;
@@ -92,10 +91,10 @@ struct lbm_ctx {
     double* d_obs;       // 8 doubles
     int* d_err;          // device error word of the TMA kernels (bounded waits)
     bool use_tma;
-    bool walls;          // no-slip walls on rows 0 and ny-1 (direct wall kernels)
+    bool walls;          // no-slip walls on rows 0 and ny-1 (mirrored or one-sided)
     bool onesided;       // free-energy walls with the one-sided normal mu gradient (LBM_BC_WALL_ZOUHE_ONESIDED)
     void* wall;          // 14 nx reals: the wall rows' J_y and solve scratch (fe_wall_solve_kernel)
-    double* dmass;       // per-warp stored mass of the driven FP32 strip steps (drive_mass_slots)
+    double* dmass;       // stored mass of the driven steps by warp (drive_mass_slots)
     bool drive;          // droplet-collision drive configured (lbm_set_drive)
     bool grav;           // gravity configured (lbm_set_gravity; free-energy model)
     double g, rho_g, y_ref;
@@ -108,7 +107,7 @@ struct lbm_ctx {
     long long step;
     int status;
     bool ready;
-    int rows;
+    int rows;            // rows per strip of the strip kernels
     lbmk::StepParams<float> spf;
     lbmk::StepParams<double> spd;
 };
@@ -318,12 +317,17 @@ static size_t buffer_bytes(int precision, int nx, int ny) {
     return align256((precision == LBM_F64 ? 9 : 10) * (size_t)plane_pitch(nx, ny) * esz);
 }
 
-// Slots of the driven FP32 strip steps' per-warp stored mass: one per consumer warp of every
-// strip CTA of either model's strip kernel (strips of at least one row).
+// Narrowest tile of the tile kernel (full model, FP64): the most tiles across a lattice.
+constexpr int kTileMinCols = lbmk::Tile<double, 2>::kCols;
+
+// Slots of the driven steps' stored mass: strip kernels, one per consumer warp of every strip CTA
+// (strips of at least one row); FP64 tile kernel, one per tile row, for the state that is read and
+// for the one that is written; FP32 tile kernel, three sets of accumulators.
 static size_t drive_mass_slots(int nx, int ny) {
     const size_t pp = (size_t)((nx + kPPPTX - 1) / kPPPTX) * kPPPWarps;
     const size_t fe = (size_t)((nx + kFEPTX - 1) / kFEPTX) * kFEPWarps;
-    return std::max(pp, fe) * (size_t)ny;
+    const size_t tile = 2 * (size_t)((nx + kTileMinCols - 1) / kTileMinCols);
+    return std::max(std::max(std::max(pp, fe), tile) * (size_t)ny, (size_t)3 * lbmk::kDriveParts);
 }
 
 extern "C" size_t lbm_workspace_bytes(int precision, int nx, int ny) {
@@ -379,6 +383,53 @@ static void fill_step_params(lbmk::StepParams<real>& s, const lbm_ctx* c) {
     s.h_nu = (real)(1.0 - 0.5 / p.tau_nu);
     s.h6_e = (real)(6.0 * (1.0 - 0.5 / p.tau_e));
     s.h6_z = (real)(6.0 * (1.0 - 0.5 / p.tau_zeta));
+    const double RT = p.R * c->th.T, kA = G * (C1 - C2 / 3.0), kB = G * (C2 + 0.5 * p.kappa_Li), hn = 1.0 - 0.5 / p.tau_nu;
+    s.m2RT = (real)(-2.0 * RT);
+    s.a2 = (real)(2.0 * p.a);
+    s.k23 = (real)(-2.0 / 3.0 * p.kappa);
+    s.k16 = (real)(-1.0 / 6.0 * p.kappa);
+    s.kc = (real)(10.0 / 3.0 * p.kappa - 2.0 * p.a);
+    s.kA3 = (real)(3.0 * kA);
+    s.kB15 = (real)(1.5 * kB);
+    s.hn2 = (real)(0.5 * hn);
+    s.hn4 = (real)(0.25 * hn);
+    s.sn4 = (real)(0.25 / p.tau_nu);
+    s.me3 = (real)(-3.0 / p.tau_e);
+    s.sz3 = (real)(3.0 / p.tau_zeta);
+}
+
+// Rows per tile of the tile kernel.
+// FP64: the height that minimises tiles per SM x the FP64 operations of one tile in sequence, each
+// phase's warps spread over the SM's four sub-partitions (operations per cell of step64.cuh: sum of
+// the populations or psi, mu, u, collision).  It picks the fastest of the measured heights 1..8 on
+// 256 x 4 (6.2 us with 1), 101 x 50 (8.6 us with 2), 200 x 100 (12.8 us with 6), 256 x 128 (12.7
+// and 20.9 us with 8 and 3) and 400 x 300 (41 and 56 us with 4 and 8).
+// FP32: 4 rows (1022 x 770: 13.7 us against 15.8 with 2 and 14.2 with 8), the full model with its
+// three halo rows 8 (1024^2: 29 us against 40 with 4), fewer while that leaves SMs without a tile.
+static int choose_tile_rows(int prec, int model, int nx, int ny) {
+    const int wb = prec == LBM_F64 ? lbmk::tile_columns<double>(model, nx) : lbmk::tile_columns<float>(model, nx);
+    const long long gx = (nx + wb - 1) / wb;
+    if (prec == LBM_F32) {
+        int r = model == 2 ? 8 : 4;
+        while (r > 2 && gx * ((ny + r - 1) / r) < 152) r /= 2;
+        return r;
+    }
+    static const int ops[3][4] = {{28, 0, 0, 125}, {8, 45, 0, 120}, {8, 45, 40, 140}};
+    int best = 1;
+    long long least = -1;
+    for (int r = 1; r <= lbmk::kTileRows; ++r) {
+        long long t = 0;
+        for (int p = 0; p < 4; ++p) {  // phase p works on the rows of the tile and of the halo it needs
+            const int halo = p == 3 ? 0 : model + 1 - p;
+            t += (long long)((r + 2 * halo + 3) / 4) * ops[model][p];
+        }
+        t *= (gx * ((ny + r - 1) / r) + 151) / 152;
+        if (least < 0 || t < least) {
+            least = t;
+            best = r;
+        }
+    }
+    return best;
 }
 
 static int choose_rows(int nx, int ny, int tx, int strips_per_sm) {
@@ -425,13 +476,8 @@ extern "C" int lbm_create(const lbm_params* p, int nx, int ny, int bc_x, int bc_
     c->prec = c->prm.precision;
     c->esz = c->prec == LBM_F64 ? 8 : 4;
     c->pitch = plane_pitch(nx, ny);
-    {
-        const bool ppm = p->model == LBM_PSEUDOPOTENTIAL;
-        const bool fast = c->prec == LBM_F32 && nx % 4 == 0 && nx >= 8 && ny >= 2 * kWallBandFE &&
-                          std::getenv("LBM_NO_TMA") == nullptr;
-        const int tx = c->prec == LBM_F64 ? kTXd : (walls && !fast) ? kTXf : ppm ? kPPPTX : kFEPTX;
-        c->rows = choose_rows(nx, ny, tx, ppm ? 16 : 12);
-    }
+    const bool ppm = p->model == LBM_PSEUDOPOTENTIAL;
+    c->rows = choose_rows(nx, ny, ppm ? kPPPTX : kFEPTX, ppm ? 16 : 12);
     const size_t need = lbm_workspace_bytes(c->prec, nx, ny);
     if (workspace) {
         if (workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255)) {
@@ -540,30 +586,44 @@ extern "C" int lbm_derived(const lbm_ctx* c, lbm_params* resolved, lbm_thermo* t
 // ----------------------------------------------------------------------------
 // Kernel launches
 
-constexpr int kMassBlocks = 608;  // block sums of the drive's domain mean (4 x 152 SMs; < 3 kRedBlocks)
+constexpr int kMassBlocks = 608;  // block sums of the drive's domain mean (4 x 152 SMs)
+static_assert(kMassBlocks + lbmk::kDriveParts <= 3 * kRedBlocks, "the drive's sums share the reduction partials");
+// Most slots that every CTA of a driven FP64 tile step sums itself; above, a reduction launch precedes it.
+constexpr size_t kTileSlots = 1024;
 
 template <typename real>
 static lbmk::Drive<real> no_drive() {
-    lbmk::Drive<real> d{};
-    d.rho_ave = nullptr;
-    return d;
+    return lbmk::Drive<real>{};
 }
 
-// The drive of the state in buffer src: its mean density reduced on the context stream into
-// partials[kMassBlocks] (block sums in partials[0, kMassBlocks)).
+// The drive's constants.
 template <typename real>
-static lbmk::Drive<real> launch_drive(lbm_ctx* c, int src) {
-    const long long n = (long long)c->nx * c->ny;
-    lbmk::mass_partials_kernel<real><<<kMassBlocks, 256, 0, c->stream>>>(static_cast<const real*>(c->f[src]),
-                                                                       c->pitch, n, c->partials);
-    lbmk::mass_final_kernel<<<1, 32, 0, c->stream>>>(c->partials, kMassBlocks, 1.0 / (double)n,
-                                                     c->partials + kMassBlocks);
-    lbmk::Drive<real> d;
-    d.rho_ave = c->partials + kMassBlocks;
+static lbmk::Drive<real> drive_terms(const lbm_ctx* c) {
+    lbmk::Drive<real> d{};
+    d.inv_cells = 1.0 / ((double)c->nx * c->ny);
     d.x_split = (int)std::floor(std::min(std::max(c->drive_split, -1.0), (double)c->nx));
     d.ax_lo = (real)c->drive_lo;
     d.ax_hi = (real)c->drive_hi;
     return d;
+}
+
+// The drive of a state whose mass is the sum of n doubles at parts: reduced on the context stream to
+// the kDriveParts sums that every warp of a driven kernel adds up.
+template <typename real>
+static lbmk::Drive<real> sum_drive(lbm_ctx* c, const double* parts, int n) {
+    double* sums = c->partials + kMassBlocks;
+    lbmk::mass_sums_kernel<<<lbmk::kDriveParts, 256, 0, c->stream>>>(parts, n, sums);
+    lbmk::Drive<real> d = drive_terms<real>(c);
+    d.parts = sums;
+    return d;
+}
+
+// The same from the populations in buffer src (block sums in partials[0, kMassBlocks)).
+template <typename real>
+static lbmk::Drive<real> launch_drive(lbm_ctx* c, int src) {
+    lbmk::mass_partials_kernel<real><<<kMassBlocks, 256, 0, c->stream>>>(
+        static_cast<const real*>(c->f[src]), c->pitch, (long long)c->nx * c->ny, c->partials);
+    return sum_drive<real>(c, c->partials, kMassBlocks);
 }
 
 // Jacobi sweeps of the one-sided walls' density solve (the oracle's fixed point reaches
@@ -575,66 +635,7 @@ constexpr int kWallIters = 32;
 template <typename real>
 static const real* launch_wall_solve(lbm_ctx* c, int src, const lbmk::StepParams<real>& sp);
 
-// The drive of a state whose mass the previous driven strip step left in c->dmass (its
-// per-warp sums of the populations it stored): rho_ave = their fixed-order sum / cells.
-static lbmk::Drive<float> chained_drive(lbm_ctx* c, dim3 grid, int nwarps) {
-    const long long n = (long long)c->nx * c->ny;
-    lbmk::mass_final_kernel<<<1, 32, 0, c->stream>>>(c->dmass, (int)(grid.x * grid.y) * nwarps, 1.0 / (double)n,
-                                                     c->partials + kMassBlocks);
-    lbmk::Drive<float> d;
-    d.rho_ave = c->partials + kMassBlocks;
-    d.x_split = (int)std::floor(std::min(std::max(c->drive_split, -1.0), (double)c->nx));
-    d.ax_lo = (float)c->drive_lo;
-    d.ax_hi = (float)c->drive_hi;
-    return d;
-}
-
-// One step with the droplet-collision drive acting (periodic lattice).  FP32 lattices that
-// run the strip kernels run their DRIVE instantiation: rho_ave of the state comes from the
-// masses the previous driven step stored (chained: the step before, in the same graph) or,
-// for the first step of a sequence, from the block-sum reduction; FP64 and other shapes run
-// the direct kernels after the reduction.
-static int launch_step_driven(lbm_ctx* c, int src, bool chained) {
-    const void* fin = c->f[src];
-    void* fout = c->f[src ^ 1];
-    const bool pp = c->prm.model == LBM_PSEUDOPOTENTIAL;
-    if (c->prec == LBM_F32 && c->use_tma) {
-        const int tx = pp ? kPPPTX : kFEPTX;
-        dim3 grid((c->nx + tx - 1) / tx, (c->ny + c->rows - 1) / c->rows);
-        const lbmk::Drive<float> d =
-            chained ? chained_drive(c, grid, pp ? kPPPWarps : kFEPWarps) : launch_drive<float>(c, src);
-        if (pp)
-            lbmk::pp_step_pair<kPPPWarps, kPPPStages, true>
-                <<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>((const float*)fin, (float*)fout, c->spf,
-                                                                             c->d_err, d, c->dmass);
-        else
-            lbmk::fe_step_pair<kFEPWarps, kFEPStages, true>
-                <<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>((const float*)fin, (float*)fout, c->spf,
-                                                                             c->d_err, d, c->dmass);
-    } else if (c->prec == LBM_F32) {
-        const lbmk::Drive<float> d = launch_drive<float>(c, src);
-        dim3 grid((c->nx + kTXf - 1) / kTXf, (c->ny + c->rows - 1) / c->rows);
-        if (pp)
-            lbmk::pp_step_ext<float, kTXf, false>
-                <<<grid, kTXf + 32, 0, c->stream>>>((const float*)fin, (float*)fout, c->spf, 0, d);
-        else
-            lbmk::fe_step_ext<float, kTXf, false>
-                <<<grid, kTXf + 32, 0, c->stream>>>((const float*)fin, (float*)fout, c->spf, 0, d, nullptr);
-    } else {
-        const lbmk::Drive<double> d = launch_drive<double>(c, src);
-        dim3 grid((c->nx + kTXd - 1) / kTXd, (c->ny + c->rows - 1) / c->rows);
-        if (pp)
-            lbmk::pp_step_ext<double, kTXd, false>
-                <<<grid, kTXd + 32, 0, c->stream>>>((const double*)fin, (double*)fout, c->spd, 0, d);
-        else
-            lbmk::fe_step_ext<double, kTXd, false>
-                <<<grid, kTXd + 32, 0, c->stream>>>((const double*)fin, (double*)fout, c->spd, 0, d, nullptr);
-    }
-    CK(cudaGetLastError());
-    return LBM_OK;
-}
-
-// Free-energy contexts with A != 0 or gravity run the full model's kernel.
+// Free-energy contexts with A != 0 or gravity run the full model's kernels.
 static bool uses_iwb(const lbm_ctx* c) {
     return c->prm.model == LBM_FREE_ENERGY && (c->prm.A != 0.0 || c->grav);
 }
@@ -650,32 +651,6 @@ static lbmk::Ext<real> ext_terms(const lbm_ctx* c) {
     return e;
 }
 
-template <typename real, int TX>
-static void launch_iwb(lbm_ctx* c, int src, bool driven, const lbmk::StepParams<real>& sp) {
-    if constexpr (std::is_same<real, float>::value) {
-        // FP32 periodic lattices without the drive and with gravity's reference density 0 run the
-        // strip kernel; the rest the direct kernel
-        if (c->use_tma && !c->walls && !driven && (!c->grav || c->rho_g == 0.0)) {
-            dim3 grid((c->nx + IWBSmem::TX - 1) / IWBSmem::TX, (c->ny + c->rows - 1) / c->rows);
-            lbmk::fe_iwb_pair<kIWBWarps, kIWBStages><<<grid, (kIWBWarps + 1) * 32, sizeof(IWBSmem), c->stream>>>(
-                static_cast<const float*>(c->f[src]), static_cast<float*>(c->f[src ^ 1]), sp, ext_terms<float>(c),
-                c->d_err);
-            return;
-        }
-    }
-    const lbmk::Drive<real> d = driven ? launch_drive<real>(c, src) : no_drive<real>();
-    dim3 grid((c->nx + TX - 1) / TX, (c->ny + c->rows - 1) / c->rows);
-    const real* fin = static_cast<const real*>(c->f[src]);
-    real* fout = static_cast<real*>(c->f[src ^ 1]);
-    const real* wjy = launch_wall_solve<real>(c, src, sp);
-    if (c->walls)
-        lbmk::fe_step_iwb<real, TX, true>
-            <<<grid, TX + 32, 0, c->stream>>>(fin, fout, sp, d, ext_terms<real>(c), wjy);
-    else
-        lbmk::fe_step_iwb<real, TX, false>
-            <<<grid, TX + 32, 0, c->stream>>>(fin, fout, sp, d, ext_terms<real>(c), nullptr);
-}
-
 template <typename real>
 static const real* launch_wall_solve(lbm_ctx* c, int src, const lbmk::StepParams<real>& sp) {
     if (!c->onesided) return nullptr;
@@ -685,79 +660,108 @@ static const real* launch_wall_solve(lbm_ctx* c, int src, const lbmk::StepParams
     return w;
 }
 
-// chained: the previous launch on the stream was a driven step of the same sequence (a graph
-// replays its steps in order), so a driven strip step may take rho_ave from its stored masses.
-static int launch_step(lbm_ctx* c, int src, bool driven = false, bool chained = false) {
-    if (uses_iwb(c)) {
-        if (c->prec == LBM_F32)
-            launch_iwb<float, kTXf>(c, src, driven, c->spf);
-        else
-            launch_iwb<double, kTXd>(c, src, driven, c->spd);
-        CK(cudaGetLastError());
-        return LBM_OK;
-    }
-    if (driven) return launch_step_driven(c, src, chained);
-    const void* fin = c->f[src];
-    void* fout = c->f[src ^ 1];
-    const bool pp = c->prm.model == LBM_PSEUDOPOTENTIAL;
-    if (c->walls && c->use_tma) {
-        // periodic fast step over the whole lattice, then the wall bands recomputed
-        const int band = pp ? kWallBandPP : kWallBandFE;
-        if (pp) {
-            dim3 grid((c->nx + kPPPTX - 1) / kPPPTX, (c->ny + c->rows - 1) / c->rows);
-            lbmk::pp_step_pair<kPPPWarps, kPPPStages><<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(
-                (const float*)fin, (float*)fout, c->spf, c->d_err);
-            lbmk::pp_step_ext<float, kTXf, true><<<dim3((c->nx + kTXf - 1) / kTXf, 2), kTXf + 32, 0, c->stream>>>(
-                (const float*)fin, (float*)fout, c->spf, band, no_drive<float>());
-        } else {
-            dim3 grid((c->nx + kFEPTX - 1) / kFEPTX, (c->ny + c->rows - 1) / c->rows);
-            const float* wjy = launch_wall_solve<float>(c, src, c->spf);
-            lbmk::fe_step_pair<kFEPWarps, kFEPStages><<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(
-                (const float*)fin, (float*)fout, c->spf, c->d_err);
-            lbmk::fe_step_ext<float, kTXf, true><<<dim3((c->nx + kTXf - 1) / kTXf, 2), kTXf + 32, 0, c->stream>>>(
-                (const float*)fin, (float*)fout, c->spf, band, no_drive<float>(), wjy);
-        }
-    } else if (c->walls) {
+static int model_index(const lbm_ctx* c) { return uses_iwb(c) ? 2 : c->prm.model == LBM_PSEUDOPOTENTIAL ? 0 : 1; }
+
+// One step of the tile kernel.  band > 0: only the rows next to each wall (after a strip kernel).
+// A driven step takes its state's mass from what the previous driven tile step left (chain > 0: the
+// number of driven steps before it in the same graph) or from a reduction of the populations.
+template <typename real>
+static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int band,
+                            const lbmk::StepParams<real>& sp) {
+    const int m = model_index(c);
+    lbmk::TileArgs<real> T{};
+    T.wb = lbmk::tile_columns<real>(m, c->nx);
+    T.band = band;
+    T.E = ext_terms<real>(c);
+    T.dpg = (real)((double)T.E.rho_g * (double)T.E.g);
+    T.fyg = (real)(c->prm.body_fy + (double)T.E.rho_g * (double)T.E.g);
+    T.wjy = c->walls ? launch_wall_solve<real>(c, src, sp) : nullptr;
+    if (driven) {
+        T.driven = true;
         if (c->prec == LBM_F32) {
-            dim3 grid((c->nx + kTXf - 1) / kTXf, (c->ny + c->rows - 1) / c->rows);
-            if (pp)
-                lbmk::pp_step_ext<float, kTXf, true>
-                    <<<grid, kTXf + 32, 0, c->stream>>>((const float*)fin, (float*)fout, c->spf, 0, no_drive<float>());
-            else
-                lbmk::fe_step_ext<float, kTXf, true><<<grid, kTXf + 32, 0, c->stream>>>(
-                    (const float*)fin, (float*)fout, c->spf, 0, no_drive<float>(), launch_wall_solve<float>(c, src, c->spf));
+            unsigned long long* acc = reinterpret_cast<unsigned long long*>(c->dmass);
+            auto set = [&](int k) { return acc + (k % 3) * lbmk::kDriveParts; };
+            if (chain > 0) {
+                T.D = drive_terms<real>(c);
+                T.acc_in = set(chain - 1);
+            } else {
+                T.D = launch_drive<real>(c, src);
+                CK(cudaMemsetAsync(acc, 0, 3 * lbmk::kDriveParts * sizeof(*acc), c->stream));
+            }
+            T.acc_out = set(chain);
+            T.acc_zero = set(chain + 1);
         } else {
-            dim3 grid((c->nx + kTXd - 1) / kTXd, (c->ny + c->rows - 1) / c->rows);
-            if (pp)
-                lbmk::pp_step_ext<double, kTXd, true>
-                    <<<grid, kTXd + 32, 0, c->stream>>>((const double*)fin, (double*)fout, c->spd, 0, no_drive<double>());
-            else
-                lbmk::fe_step_ext<double, kTXd, true><<<grid, kTXd + 32, 0, c->stream>>>(
-                    (const double*)fin, (double*)fout, c->spd, 0, no_drive<double>(),
-                    launch_wall_solve<double>(c, src, c->spd));
+            const size_t half = (size_t)((c->nx + T.wb - 1) / T.wb) * c->ny;
+            const double* slots = c->dmass + src * half;
+            if (chain > 0 && half <= kTileSlots) {
+                T.D = drive_terms<real>(c);
+                T.slots = slots;
+                T.nslots = (int)half;
+            } else {
+                T.D = chain > 0 ? sum_drive<real>(c, slots, (int)half) : launch_drive<real>(c, src);
+            }
+            T.mass = c->dmass + (src ^ 1) * half;
         }
-    } else if (c->use_tma && pp) {
-        dim3 grid((c->nx + kPPPTX - 1) / kPPPTX, (c->ny + c->rows - 1) / c->rows);
-        lbmk::pp_step_pair<kPPPWarps, kPPPStages><<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(
-            (const float*)fin, (float*)fout, c->spf, c->d_err);
-    } else if (c->use_tma) {
-        dim3 grid((c->nx + kFEPTX - 1) / kFEPTX, (c->ny + c->rows - 1) / c->rows);
-        lbmk::fe_step_pair<kFEPWarps, kFEPStages><<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(
-            (const float*)fin, (float*)fout, c->spf, c->d_err);
-    } else if (c->prec == LBM_F32) {
-        dim3 grid((c->nx + kTXf - 1) / kTXf, (c->ny + c->rows - 1) / c->rows);
-        if (pp)
-            lbmk::pp_step_kernel<float, kTXf><<<grid, kTXf + 32, 0, c->stream>>>((const float*)fin, (float*)fout, c->spf);
+    }
+    CK(lbmk::launch_tile<real>(m, c->walls, static_cast<const real*>(c->f[src]), static_cast<real*>(c->f[src ^ 1]), sp,
+                               T, band > 0 ? band : choose_tile_rows(c->prec, m, c->nx, c->ny), c->stream));
+    return LBM_OK;
+}
+
+// Whether a step runs the strip kernels: FP32 lattices of TMA-copyable rows, and for the full
+// free-energy model neither walls nor the drive nor a reference density; above the size where the
+// strips' streaming beats the tiles' short chains (us per step, tile and strip):
+//   pseudopotential        1792^2  51.9, 59.0   2048^2  67.9, 69.9   2560^2 102.9, 98.5
+//   free energy            1536^2  50.8, 52.8   1792^2  67.2, 63.0   2048^2  87.9, 81.8
+//   full free energy       1536^2  66.4, 67.0   1792^2  87.7, 80.1
+//   walls (P; FE)          1536^2  44.0, 51.1; 57.2, 56.0   2048^2  76.0, 72.8; 99.2, 85.0
+//   drive (P; FE)          1024^2  20.9, 30.9; 29.9, 35.1   1536^2  47.6, 52.1; 66.5, 56.9
+//                          2048^2  82.4, 74.5; 115.5, 86.0
+static bool strip_step(const lbm_ctx* c, bool driven) {
+    if (!c->use_tma) return false;
+    const long long cells = (long long)c->nx * c->ny;
+    if (uses_iwb(c)) return cells >= 2800000 && !c->walls && !driven && (!c->grav || c->rho_g == 0.0);
+    const bool pp = c->prm.model == LBM_PSEUDOPOTENTIAL;
+    if (driven) return cells >= (pp ? 3000000 : 1500000);
+    if (c->walls) return cells >= (pp ? 3400000 : 2100000);
+    return cells >= (pp ? 4500000 : 2800000);
+}
+
+// chain: how many driven steps of the same sequence precede this one on the stream (a graph replays
+// its steps in order); a driven step with one before it takes rho_ave from its stored masses.
+static int launch_step(lbm_ctx* c, int src, bool driven = false, int chain = 0) {
+    if (!strip_step(c, driven))
+        return c->prec == LBM_F32 ? launch_tile_step<float>(c, src, driven, chain, 0, c->spf)
+                                  : launch_tile_step<double>(c, src, driven, chain, 0, c->spd);
+    const float* fin = static_cast<const float*>(c->f[src]);
+    float* fout = static_cast<float*>(c->f[src ^ 1]);
+    const int m = model_index(c);
+    const int tx = m == 0 ? kPPPTX : m == 1 ? kFEPTX : IWBSmem::TX;
+    const dim3 grid((c->nx + tx - 1) / tx, (c->ny + c->rows - 1) / c->rows);
+    if (m == 2) {
+        lbmk::fe_iwb_pair<kIWBWarps, kIWBStages>
+            <<<grid, (kIWBWarps + 1) * 32, sizeof(IWBSmem), c->stream>>>(fin, fout, c->spf, ext_terms<float>(c), c->d_err);
+    } else if (driven) {
+        // the state's mass: what the previous driven strip step stored, by warp, or a reduction
+        const lbmk::Drive<float> d =
+            chain > 0 ? sum_drive<float>(c, c->dmass, (int)(grid.x * grid.y) * (m == 0 ? kPPPWarps : kFEPWarps))
+                    : launch_drive<float>(c, src);
+        if (m == 0)
+            lbmk::pp_step_pair<kPPPWarps, kPPPStages, true><<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(
+                fin, fout, c->spf, c->d_err, d, c->dmass);
         else
-            lbmk::fe_step_kernel<float, kTXf><<<grid, kTXf + 32, 0, c->stream>>>((const float*)fin, (float*)fout, c->spf);
+            lbmk::fe_step_pair<kFEPWarps, kFEPStages, true><<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(
+                fin, fout, c->spf, c->d_err, d, c->dmass);
+    } else if (m == 0) {
+        lbmk::pp_step_pair<kPPPWarps, kPPPStages>
+            <<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
     } else {
-        dim3 grid((c->nx + kTXd - 1) / kTXd, (c->ny + c->rows - 1) / c->rows);
-        if (pp)
-            lbmk::pp_step_kernel<double, kTXd><<<grid, kTXd + 32, 0, c->stream>>>((const double*)fin, (double*)fout, c->spd);
-        else
-            lbmk::fe_step_kernel<double, kTXd><<<grid, kTXd + 32, 0, c->stream>>>((const double*)fin, (double*)fout, c->spd);
+        lbmk::fe_step_pair<kFEPWarps, kFEPStages>
+            <<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
     }
     CK(cudaGetLastError());
+    // walls: the periodic step is right except on the rows next to them
+    if (c->walls) return launch_tile_step<float>(c, src, false, 0, m == 0 ? kWallBandPP : kWallBandFE, c->spf);
     return LBM_OK;
 }
 
@@ -767,7 +771,7 @@ static int build_graph(lbm_ctx* c, int parity, int driven) {
     int rc = LBM_OK;
     int src = parity;
     for (int k = 0; k < kGraphSteps && rc == LBM_OK; ++k) {
-        rc = launch_step(c, src, driven != 0, k > 0);
+        rc = launch_step(c, src, driven != 0, k);
         src ^= 1;
     }
     cudaError_t e = cudaStreamEndCapture(c->stream, &g);

@@ -9,9 +9,10 @@
 // Fusion: every quantity needed at neighbours (psi for the pseudopotential model,
 // rho and mu for the free-energy model) is recomputed from the pulled populations
 // inside the CTA that needs it, so the step moves only 9 loads + 9 stores of
-// populations per cell through HBM.  A CTA owns a strip of TX columns and walks
-// down `rows` rows; the per-row neighbour fields live in small shared-memory
-// rings (sliding window), and one extra warp computes the x-halo columns.
+// populations per cell through HBM.  The step kernels are the strip kernels
+// (step_pair.cuh, step_iwb_pair.cuh: large FP32 lattices) and the tile kernel
+// (step_tile.cuh: the rest); this file holds their per-cell FP32 arithmetic, the
+// initial state and the observables.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -42,6 +43,9 @@ struct StepParams {
     // once on the host: computed in the kernels, a compiler may fuse them differently in two
     // kernels and the same cell would then differ by an ulp of the increments between routes
     real h_e, h_z, h_q, h_nu, h6_e, h6_z;
+    // folded factors of the FP64 arithmetic (step64.cuh): -2 RT, 2 a; -2 kappa/3, -kappa/6,
+    // 10 kappa/3 - 2 a; 3 kA, 1.5 kB; h_nu / 2, h_nu / 4, s_nu / 4; -3 s_e, 3 s_z
+    real m2RT, a2, k23, k16, kc, kA3, kB15, hn2, hn4, sn4, me3, sz3;
 };
 
 // Correctly rounded reciprocal (FP32: one hardware-assisted sequence instead of a full division).
@@ -117,135 +121,6 @@ __device__ __forceinline__ real sum9(const real v[9]) {
     return v[0] + (((v[1] + v[3]) + (v[2] + v[4])) + ((v[5] + v[7]) + (v[6] + v[8])));
 }
 
-// f* = f + M^-1 dm for the moment increments dm (rho increment is zero); M^-1 of Eq. (S49).
-// d0: if not null, receives the rest population's increment, and v[0] is left unchanged (the
-// caller applies it to a compensated rest population; see rest_update).
-template <typename real>
-__device__ __forceinline__ void apply_dm(real v[9], real de, real dz, real djx, real dqx, real djy, real dqy,
-                                         real dpxx, real dpxy, real* d0 = nullptr) {
-    const real A = -de * real(1.0 / 36.0) - dz * real(1.0 / 18.0);
-    const real B = de * real(1.0 / 18.0) + dz * real(1.0 / 36.0);
-    const real X1 = (djx - dqx) * real(1.0 / 6.0);
-    const real Y1 = (djy - dqy) * real(1.0 / 6.0);
-    const real X2 = djx * real(1.0 / 6.0) + dqx * real(1.0 / 12.0);
-    const real Y2 = djy * real(1.0 / 6.0) + dqy * real(1.0 / 12.0);
-    const real Pp = dpxx * real(0.25);
-    const real Z = dpxy * real(0.25);
-    if (d0)
-        *d0 = (dz - de) * real(1.0 / 9.0);
-    else
-        v[0] += (dz - de) * real(1.0 / 9.0);
-    v[1] += A + X1 + Pp;
-    v[2] += A + Y1 - Pp;
-    v[3] += A - X1 + Pp;
-    v[4] += A - Y1 - Pp;
-    v[5] += B + X2 + Y2 + Z;
-    v[6] += B - X2 + Y2 - Z;
-    v[7] += B - X2 - Y2 + Z;
-    v[8] += B + X2 - Y2 - Z;
-}
-
-// ---------------------------------------------------------------------------------
-// Modified pseudopotential collision of one cell (Eqs. 1, 4, 6, 10, 13, 30-32).
-//   v  : pulled populations (in: f, out: f*)
-//   pc : psi at the cell; pn[i] : psi at x + c_i (i = 1..8)
-template <typename real>
-__device__ __forceinline__ void pp_collide(real v[9], real rho, real pc, const real pn[9],
-                                           const StepParams<real>& P) {
-    const real w1 = real(1.0 / 3.0), w2 = real(1.0 / 12.0);
-    // Eq. (10): F_int = -G psi sum_i omega_i psi(x + c_i) c_i, G = -1
-    const real Sx = (pn[1] - pn[3]) * w1 + ((pn[5] - pn[7]) + (pn[8] - pn[6])) * w2;
-    const real Sy = (pn[2] - pn[4]) * w1 + ((pn[5] - pn[7]) + (pn[6] - pn[8])) * w2;
-    const real Fix = pc * Sx, Fiy = pc * Sy;
-    const real Fx = Fix + P.fx, Fy = Fiy + P.fy;
-    // Eq. (30): Q_ab = psi sum_i omega_i C_iab (psi_i - psi), C2 term carrying G
-    const real d1 = pn[1] - pc, d2 = pn[2] - pc, d3 = pn[3] - pc, d4 = pn[4] - pc;
-    const real d5 = pn[5] - pc, d6 = pn[6] - pc, d7 = pn[7] - pc, d8 = pn[8] - pc;
-    const real dd = ((d5 + d6) + (d7 + d8)) * w2;
-    const real sxx = (d1 + d3) * w1 + dd;
-    const real syy = (d2 + d4) * w1 + dd;
-    const real sa = sxx + syy - dd;  // sum_i omega_i d_i
-    const real sxy = ((d5 - d6) + (d7 - d8)) * w2;
-    const real Qxx = pc * (P.kA * sa + P.kB * sxx);
-    const real Qyy = pc * (P.kA * sa + P.kB * syy);
-    const real Qxy = pc * (P.kB * sxy);
-    // Eq. (32) consistency term: 12 kappa_P sigma_Li |F_int|^2/psi^2 = li |S|^2 (G^2 = 1)
-    const real L = P.li * (Sx * Sx + Sy * Sy);
-    // Eq. (6b) and the moments m = M f (Eq. S48)
-    const real jx = (v[1] - v[3]) + (v[5] - v[6]) + (v[8] - v[7]);
-    const real jy = (v[2] - v[4]) + (v[5] + v[6]) - (v[7] + v[8]);
-    const real inv_rho = rcp(rho);
-    const real ux = (jx + real(0.5) * Fx) * inv_rho;
-    const real uy = (jy + real(0.5) * Fy) * inv_rho;
-    const real sax = (v[1] + v[2]) + (v[3] + v[4]);
-    const real sdg = (v[5] + v[6]) + (v[7] + v[8]);
-    const real e = -real(4) * v[0] - sax + real(2) * sdg;
-    const real z = real(4) * v[0] - real(2) * sax + sdg;
-    const real qx = real(2) * (v[3] - v[1]) + (v[5] - v[6]) + (v[8] - v[7]);
-    const real qy = real(2) * (v[4] - v[2]) + (v[5] + v[6]) - (v[7] + v[8]);
-    const real pxx = (v[1] + v[3]) - (v[2] + v[4]);
-    const real pxy = (v[5] + v[7]) - (v[6] + v[8]);
-    const real uu = ux * ux + uy * uy;
-    const real uF = ux * Fx + uy * Fy;
-    const real trQ = Qxx + Qyy;
-    // m* - m = -L (m - m^eq) + (I - L/2) MF' + MC  (Eqs. 1, 4/S66, 32, 13)
-    const real de = -P.s_e * (e - rho * (real(3) * uu - real(2))) + (real(1) - real(0.5) * P.s_e) * real(6) * uF +
-                    P.s_e * (L + real(1.5) * trQ);
-    const real dz = -P.s_z * (z - rho * (real(1) - real(3) * uu)) - (real(1) - real(0.5) * P.s_z) * real(6) * uF -
-                    P.s_z * (L + real(1.5) * trQ);
-    const real dqx = -P.s_q * (qx + rho * ux) - (real(1) - real(0.5) * P.s_q) * Fx;
-    const real dqy = -P.s_q * (qy + rho * uy) - (real(1) - real(0.5) * P.s_q) * Fy;
-    const real dpxx = -P.s_nu * (pxx - rho * (ux * ux - uy * uy)) +
-                      (real(1) - real(0.5) * P.s_nu) * real(2) * (ux * Fx - uy * Fy) - P.s_nu * (Qxx - Qyy);
-    const real dpxy = -P.s_nu * (pxy - rho * ux * uy) + (real(1) - real(0.5) * P.s_nu) * (ux * Fy + uy * Fx) -
-                      P.s_nu * Qxy;
-    // j* - j = F exactly (tau_j drops out)
-    apply_dm(v, de, dz, Fx, dqx, Fy, dqy, dpxx, dpxy);
-}
-
-// ---------------------------------------------------------------------------------
-// Improved well-balanced free-energy collision of one cell (Eqs. 1, 6, 20, 21, 24).
-//   mn[i] : mu at x + c_i, rn[i] : rho at x + c_i (i = 1..8)
-template <typename real>
-__device__ __forceinline__ void fe_collide(real v[9], real rho, const real mn[9], const real rn[9],
-                                           const StepParams<real>& P) {
-    const real w1 = real(1.0 / 3.0), w2 = real(1.0 / 12.0);
-    // Eq. (24) gradient with weights: d_a phi = 3 sum_i w_i phi_i c_ia
-    const real gmx = (mn[1] - mn[3]) * w1 + ((mn[5] - mn[7]) + (mn[8] - mn[6])) * w2;
-    const real gmy = (mn[2] - mn[4]) * w1 + ((mn[5] - mn[7]) + (mn[6] - mn[8])) * w2;
-    const real grx = (rn[1] - rn[3]) * w1 + ((rn[5] - rn[7]) + (rn[8] - rn[6])) * w2;
-    const real gry = (rn[2] - rn[4]) * w1 + ((rn[5] - rn[7]) + (rn[6] - rn[8])) * w2;
-    const real Fx = -rho * gmx + P.fx, Fy = -rho * gmy + P.fy;
-    const real jx = (v[1] - v[3]) + (v[5] - v[6]) + (v[8] - v[7]);
-    const real jy = (v[2] - v[4]) + (v[5] + v[6]) - (v[7] + v[8]);
-    const real inv_rho = rcp(rho);
-    const real ux = (jx + real(0.5) * Fx) * inv_rho;
-    const real uy = (jy + real(0.5) * Fy) * inv_rho;
-    const real sax = (v[1] + v[2]) + (v[3] + v[4]);
-    const real sdg = (v[5] + v[6]) + (v[7] + v[8]);
-    const real e = -real(4) * v[0] - sax + real(2) * sdg;
-    const real z = real(4) * v[0] - real(2) * sax + sdg;
-    const real qx = real(2) * (v[3] - v[1]) + (v[5] - v[6]) + (v[8] - v[7]);
-    const real qy = real(2) * (v[4] - v[2]) + (v[5] + v[6]) - (v[7] + v[8]);
-    const real pxx = (v[1] + v[3]) - (v[2] + v[4]);
-    const real pxy = (v[5] + v[7]) - (v[6] + v[8]);
-    const real uu = ux * ux + uy * uy;
-    const real uF = ux * Fx + uy * Fy;
-    const real s = ux * grx + uy * gry;  // u . grad rho
-    const real Gx = Fx + grx * real(1.0 / 3.0), Gy = Fy + gry * real(1.0 / 3.0);  // F + c_s^2 grad rho
-    // M F_i of Eq. (21): (0, 6uF + 4s, -6uF - 4s, Fx, -Fx, Fy, -Fy, 2(uxGx - uyGy), uxGy + uyGx)
-    const real fe = real(6) * uF + real(4) * s;
-    // m^eq of Eq. (20): (rho, rho(-4 + 3uu), rho(4 - 3uu), rho u, -rho u, ..., rho(ux^2-uy^2), rho ux uy)
-    const real de = -P.s_e * (e - rho * (real(3) * uu - real(4))) + (real(1) - real(0.5) * P.s_e) * fe;
-    const real dz = -P.s_z * (z - rho * (real(4) - real(3) * uu)) - (real(1) - real(0.5) * P.s_z) * fe;
-    const real dqx = -P.s_q * (qx + rho * ux) - (real(1) - real(0.5) * P.s_q) * Fx;
-    const real dqy = -P.s_q * (qy + rho * uy) - (real(1) - real(0.5) * P.s_q) * Fy;
-    const real dpxx = -P.s_nu * (pxx - rho * (ux * ux - uy * uy)) +
-                      (real(1) - real(0.5) * P.s_nu) * real(2) * (ux * Gx - uy * Gy);
-    const real dpxy = -P.s_nu * (pxy - rho * ux * uy) + (real(1) - real(0.5) * P.s_nu) * (ux * Gy + uy * Gx);
-    apply_dm(v, de, dz, Fx, dqx, Fy, dqy, dpxx, dpxy);
-}
-
 // Chemical potential (up to the constant mu_b(rho_v)) at one cell from rho at the cell (rc) and
 // its 8 neighbours; Eq. (24) Laplacian summed over differences.
 template <typename real>
@@ -260,8 +135,7 @@ __device__ __forceinline__ real fe_mu(real rc, const real rn[9], const StepParam
 // Blackwell's packed FP32: one instruction computes both lanes).  Every operation is an
 // explicit correctly rounded add / multiply / fused multiply-add, never re-associated or
 // contracted by the compiler, so the single-cell and the two-cell kernels produce bitwise
-// identical cells.  The algebra is that of pp_collide / fe_collide / fe_mu above (Eqs. 10-13,
-// 20, 21, 24, 29-32), arranged for FP32 in three ways:
+// identical cells.  The algebra is Eqs. 10-13, 20, 21, 24, 29-32 in moments (Eqs. S48, S49), arranged for FP32 in three ways:
 //  * Mirror equivariance.  Every sum over velocities is grouped so that reflecting the lattice
 //    in x (1<->3, 5<->6, 7<->8) or in y (2<->4, 5<->8, 6<->7) maps each partial result onto
 //    itself or onto its exact negative (IEEE addition is commutative and a - b = -(b - a)).
@@ -445,16 +319,17 @@ __device__ __forceinline__ void apply_dm_v(F v[9], F de, F dz, F djx, F dqx, F d
 
 // Improved well-balanced free-energy collision (Eqs. 1, 6, 20, 21, 24); mn, rn: mu and rho
 // at x + c_i (i = 1..8).  COMP: the rest population's increment goes to *d0, v[0] unchanged.
-// fx: the x body force of the cell (P.fx, or P.fx plus the droplet-collision drive).
+// fx, fy: the external force of the cell (the body force; fx with the droplet-collision drive, fy
+// at a one-sided wall with the normal force).
 template <class F, bool COMP = false>
-__device__ __forceinline__ void fe_collide_fx_v(F v[9], F rho, const F mn[9], const F rn[9], F fx,
-                                                const StepParams<float>& P, F* d0) {
+__device__ __forceinline__ void fe_collide_f_v(F v[9], F rho, const F mn[9], const F rn[9], F fx, F fy,
+                                               const StepParams<float>& P, F* d0) {
     const F w1 = F::c(1.0f / 3.0f), w2 = F::c(1.0f / 12.0f);
     const F gmx = fmav(mn[1] - mn[3], w1, ((mn[5] - mn[7]) + (mn[8] - mn[6])) * w2);
     const F gmy = fmav(mn[2] - mn[4], w1, ((mn[5] - mn[7]) + (mn[6] - mn[8])) * w2);
     const F grx = fmav(rn[1] - rn[3], w1, ((rn[5] - rn[7]) + (rn[8] - rn[6])) * w2);
     const F gry = fmav(rn[2] - rn[4], w1, ((rn[5] - rn[7]) + (rn[6] - rn[8])) * w2);
-    const F Fx = fmav(-rho, gmx, fx), Fy = fmav(-rho, gmy, F::c(P.fy));
+    const F Fx = fmav(-rho, gmx, fx), Fy = fmav(-rho, gmy, fy);
     const F jx = mom_jx(v);
     const F jy = mom_jy(v);
     const F inv_rho = rcp_v(rho);
@@ -484,6 +359,11 @@ __device__ __forceinline__ void fe_collide_fx_v(F v[9], F rho, const F mn[9], co
     const F dpxx = fmav(F::c(2.0f * hn), fmav(ux, Gx, -(uy * Gy)), F::c(-P.s_nu) * (pxx - rho * fmav(ux, ux, -(uy * uy))));
     const F dpxy = fmav(F::c(hn), fmav(ux, Gy, uy * Gx), F::c(-P.s_nu) * (pxy - rho * ux * uy));
     apply_dm_v<F, COMP>(v, de, dz, Fx, dqx, Fy, dqy, dpxx, dpxy, d0);
+}
+template <class F, bool COMP = false>
+__device__ __forceinline__ void fe_collide_fx_v(F v[9], F rho, const F mn[9], const F rn[9], F fx,
+                                                const StepParams<float>& P, F* d0) {
+    fe_collide_f_v<F, COMP>(v, rho, mn, rn, fx, F::c(P.fy), P, d0);
 }
 template <class F, bool COMP = false>
 __device__ __forceinline__ void fe_collide_v(F v[9], F rho, const F mn[9], const F rn[9],
@@ -523,7 +403,7 @@ __device__ __forceinline__ F pseudo_psi_v(F rho, const StepParams<float>& P) {
     return sqrt_v(F::c(2.0f) * fmav(rho, F::c(kThirdHi), fmav(rho, F::c(kThirdLo), -cs_pressure_v(rho, P))));
 }
 
-// Modified pseudopotential collision (Eqs. 1, 4, 6, 10, 13, 30-32) in the algebra of pp_collide:
+// Modified pseudopotential collision (Eqs. 1, 4, 6, 10, 13, 30-32):
 // pc = psi at the cell, pn[i] = psi at x + c_i (i = 1..8).
 // COMP: compensated rest population with the moving populations' rounding absorbed (the rest
 // increment goes to *d0, v[0] unchanged; see apply_dm_v and rest_update).
@@ -582,13 +462,22 @@ __device__ __forceinline__ void pp_collide_v(F v[9], F rho, F pc, const F pn[9],
 
 // Droplet-collision drive (Sec. 5.4): the force a_x |rho - rho_ave| along x, a_x = ax_lo for
 // x <= x_split and ax_hi beyond, rho_ave the mean density of the state being collided (a device
-// scalar).  rho_ave == nullptr: no drive.
+// scalar), given as the parts of its sum.
+constexpr int kDriveParts = 32;
 template <typename real>
 struct Drive {
-    const double* rho_ave;
+    const double* parts;  // kDriveParts sums whose sum is the mass of the state; nullptr: no drive
+    double inv_cells;
     int x_split;
     real ax_lo, ax_hi;
 };
+// rho_ave: every warp sums the parts in the same order (all lanes of a warp call it)
+template <typename real>
+__device__ __forceinline__ double drive_mean(const Drive<real>& D) {
+    double s = __ldg(D.parts + (threadIdx.x & 31));
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s * D.inv_cells;
+}
 
 // ---------------------------------------------------------------------------------
 // Compensated rest population of the FP32 step (both models).
@@ -680,20 +569,7 @@ __device__ __forceinline__ float sum9_rest(const float v[9], int q, const StepPa
 __device__ __forceinline__ float pseudo_psi(float rho, const StepParams<float>& P) {
     return pseudo_psi_v(F1(rho), P).v;
 }
-__device__ __forceinline__ void pp_collide(float v[9], float rho, float pc, const float pn[9],
-                                           const StepParams<float>& P) {
-    F1 vv[9], n[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        vv[i] = F1(v[i]);
-        n[i] = F1(pn[i]);
-    }
-    pp_collide_v(vv, F1(rho), F1(pc), n, P);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = vv[i].v;
-}
-
-// The same collision with a compensated rest population (v[0] and q updated together).
+// The collision with a compensated rest population (v[0] and q updated together).
 __device__ __forceinline__ void pp_collide_comp(float v[9], int& q, float rho, float pc, const float pn[9],
                                                 const StepParams<float>& P) {
     F1 vv[9], n[9], d0;
@@ -708,42 +584,6 @@ __device__ __forceinline__ void pp_collide_comp(float v[9], int& q, float rho, f
     rest_update(v[0], q, d0.v, P);
 }
 
-// FP32 single-cell entry points used by every FP32 free-energy kernel (the templates above
-// serve FP64).
-__device__ __forceinline__ void fe_collide(float v[9], float rho, const float mn[9], const float rn[9],
-                                           const StepParams<float>& P) {
-    // entry 0 of mn, rn (the cell itself) is not used and callers need not set it
-    F1 vv[9], m[9], r[9];
-    m[0] = r[0] = F1(0.0f);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) vv[i] = F1(v[i]);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        m[i] = F1(mn[i]);
-        r[i] = F1(rn[i]);
-    }
-    fe_collide_v(vv, F1(rho), m, r, P);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = vv[i].v;
-}
-// The same collision with a compensated rest population: v[0] (hi) and q of the cell are
-// updated together (see rest_update).
-__device__ __forceinline__ void fe_collide_comp(float v[9], int& q, float rho, const float mn[9], const float rn[9],
-                                                const StepParams<float>& P) {
-    F1 vv[9], m[9], r[9], d0;
-    m[0] = r[0] = F1(0.0f);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) vv[i] = F1(v[i]);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        m[i] = F1(mn[i]);
-        r[i] = F1(rn[i]);
-    }
-    fe_collide_v<F1, true>(vv, F1(rho), m, r, P, &d0);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) v[i] = vv[i].v;
-    rest_update(v[0], q, d0.v, P);
-}
 __device__ __forceinline__ float fe_mu(float rc, const float rn[9], const StepParams<float>& P) {
     // rn[0] is not used and callers need not set it
     F1 r[9];
@@ -751,207 +591,6 @@ __device__ __forceinline__ float fe_mu(float rc, const float rn[9], const StepPa
 #pragma unroll
     for (int i = 1; i < 9; ++i) r[i] = F1(rn[i]);
     return fe_mu_v(F1(rc), r, P).v;
-}
-
-// ---------------------------------------------------------------------------------
-// Pseudopotential step.  Block = TX main threads (one column each) + one halo warp.
-template <typename real, int TX>
-__global__ void __launch_bounds__(TX + 32) pp_step_kernel(const real* __restrict__ fin, real* __restrict__ fout,
-                                                          const StepParams<real> P) {
-    __shared__ real s_psi[4][TX + 2];
-    const int nx = P.nx, ny = P.ny;
-    const long long pitch = P.pitch;
-    const int x0 = blockIdx.x * TX;
-    const int w = min(TX, nx - x0);
-    const int y0 = blockIdx.y * P.rows;
-    const int y1 = min(y0 + P.rows, ny);
-    const int t = threadIdx.x;
-    const bool is_main = t < TX;
-    bool has_col;
-    int x, sc;
-    if (is_main) {
-        has_col = t < w;
-        x = x0 + (has_col ? t : 0);
-        sc = t + 1;
-    } else {
-        const int lane = t - TX;
-        has_col = lane < 2;
-        x = lane == 0 ? wrap_idx(x0 - 1, nx) : wrap_idx(x0 + w, nx);
-        sc = lane == 0 ? 0 : w + 1;
-    }
-    const int xm = x == 0 ? nx - 1 : x - 1;
-    const int xp = x == nx - 1 ? 0 : x + 1;
-
-    real cur[9], prv[9];
-    auto row_offsets = [&](int r, long long& om, long long& o0, long long& op) {
-        om = (long long)wrap_idx(r - 1, ny) * nx;
-        o0 = (long long)wrap_idx(r, ny) * nx;
-        op = (long long)wrap_idx(r + 1, ny) * nx;
-    };
-    if (has_col) {
-        long long om, o0, op;
-        row_offsets(y0 - 1, om, o0, op);
-        pull9(fin, pitch, x, xm, xp, om, o0, op, cur);
-    }
-#pragma unroll 1
-    for (int r = y0 - 1; r <= y1; ++r) {
-        real nxt[9];
-        const bool more = r < y1;
-        if (has_col && more) {
-            long long om, o0, op;
-            row_offsets(r + 1, om, o0, op);
-            pull9(fin, pitch, x, xm, xp, om, o0, op, nxt);
-        }
-        real rho = real(0);
-        if (has_col) {
-            rho = sum9(cur);
-            s_psi[r & 3][sc] = pseudo_psi(rho, P);
-        }
-        __syncthreads();
-        if (is_main && has_col && r > y0) {
-            // centre row c = r - 1: neighbours in rows c-1 (slot r-2), c (r-1), c+1 (r)
-            const real* sm = s_psi[(r - 2) & 3];
-            const real* s0 = s_psi[(r - 1) & 3];
-            const real* sp = s_psi[r & 3];
-            real pn[9];
-            pn[0] = s0[sc];
-            pn[1] = s0[sc + 1];
-            pn[2] = sp[sc];
-            pn[3] = s0[sc - 1];
-            pn[4] = sm[sc];
-            pn[5] = sp[sc + 1];
-            pn[6] = sp[sc - 1];
-            pn[7] = sm[sc - 1];
-            pn[8] = sm[sc + 1];
-            const real rho_c = sum9(prv);
-            const long long o = (long long)(r - 1) * nx + x;
-            if constexpr (std::is_same<real, float>::value) {
-                int q = rest_lo_plane(fin, pitch)[o];  // compensated rest population
-                pp_collide_comp(prv, q, rho_c, pn[0], pn, P);
-                rest_lo_plane(fout, pitch)[o] = (short)q;
-            } else {
-                pp_collide(prv, rho_c, pn[0], pn, P);
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) fout[i * pitch + o] = prv[i];
-        }
-        if (has_col) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                prv[i] = cur[i];
-                cur[i] = nxt[i];
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------
-// Free-energy step.  rho ring (8 rows, 2 halo columns each side), mu ring (4 rows, 1 halo).
-// Halo warp lanes: 0 -> x0-2, 1 -> x0-1 (also mu), 2 -> x0+w (also mu), 3 -> x0+w+1.
-template <typename real, int TX>
-__global__ void __launch_bounds__(TX + 32) fe_step_kernel(const real* __restrict__ fin, real* __restrict__ fout,
-                                                          const StepParams<real> P) {
-    __shared__ real s_rho[8][TX + 4];
-    __shared__ real s_mu[4][TX + 2];
-    const int nx = P.nx, ny = P.ny;
-    const long long pitch = P.pitch;
-    const int x0 = blockIdx.x * TX;
-    const int w = min(TX, nx - x0);
-    const int y0 = blockIdx.y * P.rows;
-    const int y1 = min(y0 + P.rows, ny);
-    const int t = threadIdx.x;
-    const bool is_main = t < TX;
-    bool has_col, has_mu;
-    int x, rc, mc;  // global column, rho-ring column, mu-ring column
-    if (is_main) {
-        has_col = t < w;
-        has_mu = has_col;
-        x = x0 + (has_col ? t : 0);
-        rc = t + 2;
-        mc = t + 1;
-    } else {
-        const int lane = t - TX;
-        has_col = lane < 4;
-        has_mu = lane == 1 || lane == 2;
-        const int off = lane == 0 ? -2 : lane == 1 ? -1 : lane == 2 ? w : w + 1;
-        x = wrap_idx(x0 + off, nx);
-        rc = lane == 0 ? 0 : lane == 1 ? 1 : lane == 2 ? w + 2 : w + 3;
-        mc = lane == 1 ? 0 : w + 1;
-    }
-    const int xm = x == 0 ? nx - 1 : x - 1;
-    const int xp = x == nx - 1 ? 0 : x + 1;
-    auto row_offsets = [&](int r, long long& om, long long& o0, long long& op) {
-        om = (long long)wrap_idx(r - 1, ny) * nx;
-        o0 = (long long)wrap_idx(r, ny) * nx;
-        op = (long long)wrap_idx(r + 1, ny) * nx;
-    };
-    real p0[9], p1[9], p2[9];  // pulled populations of rows r-2, r-1, r
-    if (has_col) {
-        long long om, o0, op;
-        row_offsets(y0 - 2, om, o0, op);
-        pull9(fin, pitch, x, xm, xp, om, o0, op, p2);
-    }
-#pragma unroll 1
-    for (int r = y0 - 2; r <= y1 + 1; ++r) {
-        real nxt[9];
-        if (has_col && r <= y1) {
-            long long om, o0, op;
-            row_offsets(r + 1, om, o0, op);
-            pull9(fin, pitch, x, xm, xp, om, o0, op, nxt);
-        }
-        if (has_col) s_rho[r & 7][rc] = sum9(p2);
-        __syncthreads();
-        if (has_mu && r >= y0) {
-            // mu at row r - 1 from rho rows r-2, r-1, r
-            const real* rm = s_rho[(r - 2) & 7];
-            const real* r0 = s_rho[(r - 1) & 7];
-            const real* rp = s_rho[r & 7];
-            real rn[9];
-            rn[1] = r0[rc + 1];
-            rn[2] = rp[rc];
-            rn[3] = r0[rc - 1];
-            rn[4] = rm[rc];
-            rn[5] = rp[rc + 1];
-            rn[6] = rp[rc - 1];
-            rn[7] = rm[rc - 1];
-            rn[8] = rm[rc + 1];
-            s_mu[(r - 1) & 3][mc] = fe_mu(r0[rc], rn, P);
-        }
-        __syncthreads();
-        if (is_main && has_col && r >= y0 + 2) {
-            // centre row c = r - 2
-            const real* mm = s_mu[(r - 3) & 3];
-            const real* m0 = s_mu[(r - 2) & 3];
-            const real* mp = s_mu[(r - 1) & 3];
-            const real* rm = s_rho[(r - 3) & 7];
-            const real* r0 = s_rho[(r - 2) & 7];
-            const real* rp = s_rho[(r - 1) & 7];
-            real mn[9], rn[9];
-            mn[1] = m0[mc + 1]; mn[2] = mp[mc]; mn[3] = m0[mc - 1]; mn[4] = mm[mc];
-            mn[5] = mp[mc + 1]; mn[6] = mp[mc - 1]; mn[7] = mm[mc - 1]; mn[8] = mm[mc + 1];
-            rn[1] = r0[rc + 1]; rn[2] = rp[rc]; rn[3] = r0[rc - 1]; rn[4] = rm[rc];
-            rn[5] = rp[rc + 1]; rn[6] = rp[rc - 1]; rn[7] = rm[rc - 1]; rn[8] = rm[rc + 1];
-            const real rho_c = r0[rc];
-            const long long o = (long long)(r - 2) * nx + x;
-            if constexpr (std::is_same<real, float>::value) {
-                int q = rest_lo_plane(fin, pitch)[o];  // compensated rest population
-                fe_collide_comp(p0, q, rho_c, mn, rn, P);
-                rest_lo_plane(fout, pitch)[o] = (short)q;
-            } else {
-                fe_collide(p0, rho_c, mn, rn, P);
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) fout[i * pitch + o] = p0[i];
-        }
-        if (has_col) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                p0[i] = p1[i];
-                p1[i] = p2[i];
-                p2[i] = nxt[i];
-            }
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------------

@@ -12,9 +12,8 @@
 // warp's lanes cover four columns on each side of its 56-column run, and the ring stages eight
 // halo columns on each side of the strip (multiples of 4 keep every bulk copy 16-byte aligned).
 //
-// The direct kernel fe_step_iwb (step_ext.cuh) serves FP64, walls, the drive and gravity with a
-// non-zero reference density; it writes the same equations with plain arithmetic, so the two
-// agree to rounding, not bit for bit.
+// The tile kernel (step_tile.cuh) serves smaller lattices, FP64, walls, the drive and gravity with a
+// non-zero reference density, in FP32 with this arithmetic and to the same bits.
 //
 // Requirements (checked on the host): nx % 4 == 0, nx >= 8, ny >= 4; every wait bounded.
 #pragma once
@@ -28,26 +27,20 @@
 
 namespace lbmk {
 
-// Velocity of Eq. (6b) with the full force F = -rho grad mu + (fx, fy): the same operations, in
-// the same order, as inside fe_collide_iwb_v, so a cell's stored u equals the u of its collision.
+// Velocity of Eq. (6b) with the full force F = -rho grad mu + (fx, fy), and that force.
 template <class F>
-__device__ __forceinline__ void fe_velocity_v(const F v[9], F rho, const F mn[9], F fx, F fy, F& ux, F& uy) {
+__device__ __forceinline__ void fe_velocity_v(const F v[9], F rho, const F mn[9], F fx, F fy, F& ux, F& uy, F& Fx,
+                                              F& Fy) {
     const F w1 = F::c(1.0f / 3.0f), w2 = F::c(1.0f / 12.0f);
     const F gmx = fmav(mn[1] - mn[3], w1, ((mn[5] - mn[7]) + (mn[8] - mn[6])) * w2);
     const F gmy = fmav(mn[2] - mn[4], w1, ((mn[5] - mn[7]) + (mn[6] - mn[8])) * w2);
-    const F Fx = fmav(-rho, gmx, fx), Fy = fmav(-rho, gmy, fy);
+    Fx = fmav(-rho, gmx, fx);
+    Fy = fmav(-rho, gmy, fy);
     const F inv_rho = rcp_v(rho);
     ux = fmav(F::c(0.5f), Fx, mom_jx(v)) * inv_rho;
     uy = fmav(F::c(0.5f), Fy, mom_jy(v)) * inv_rho;
 }
 
-// Full improved well-balanced collision (Eqs. 1, 6, 20, 21, 23, 24) in the FP32 algebra of
-// fe_collide_fx_v: un, wn -- u_x and u_y at x + c_i (i = 0..8, entry 0 the cell's own); fx, fy --
-// the external force (body force and buoyancy); pg, dpg -- p_g at the cell and d_y p_g; A -- the
-// viscosity-tuning coefficient.  With X = uu + c_s^2 A S (S = grad u + grad u^T from the Eq. 24
-// stencil) the equilibrium is the plain one with uu -> X plus p_g: its moments gain
-// e += rho A tr S + 6 p_g, zeta -= rho A tr S + 9 p_g, p_xx += rho A (S_xx - S_yy) / 3,
-// p_xy += rho A S_xy / 3.  COMP: the rest increment goes to *d0, v[0] unchanged.
 // Velocity derivatives of Eq. (24) at the cell from u_x (un) and u_y (wn) at x + c_i.
 template <class F>
 struct Strain {
@@ -64,23 +57,21 @@ __device__ __forceinline__ Strain<F> strain_v(const F un[9], const F wn[9]) {
     return g;
 }
 
-// st: the velocity derivatives of strain_v (taken before the populations are pulled, so that
-// the neighbours' velocities are no longer live during the collision).
+// Full improved well-balanced collision (Eqs. 1, 6, 20, 21, 23, 24) in the FP32 algebra of
+// fe_collide_f_v: st -- the velocity derivatives of strain_v (in the strip kernel taken before the
+// populations are pulled, so that the neighbours' velocities are no longer live during the
+// collision); ux, uy, Fx, Fy -- the cell's velocity and force (fe_velocity_v); pg, dpg -- p_g at the
+// cell and d_y p_g; A -- the viscosity-tuning coefficient.  With X = uu + c_s^2 A S (S = grad u +
+// grad u^T from the Eq. 24 stencil) the equilibrium is the plain one with uu -> X plus p_g: its
+// moments gain e += rho A tr S + 6 p_g, zeta -= rho A tr S + 9 p_g, p_xx += rho A (S_xx - S_yy) / 3,
+// p_xy += rho A S_xy / 3.  COMP: the rest increment goes to *d0, v[0] unchanged.
 template <class F, bool COMP = false>
-__device__ __forceinline__ void fe_collide_iwb_v(F v[9], F rho, const F mn[9], const F rn[9], const Strain<F>& st,
-                                                 F fx, F fy, F pg, float dpg, float A,
-                                                 const StepParams<float>& P, F* d0 = nullptr) {
+__device__ __forceinline__ void fe_collide_iwb_u_v(F v[9], F rho, const F rn[9], const Strain<F>& st, F ux, F uy, F Fx,
+                                                   F Fy, F pg, float dpg, float A, const StepParams<float>& P,
+                                                   F* d0 = nullptr) {
     const F w1 = F::c(1.0f / 3.0f), w2 = F::c(1.0f / 12.0f);
-    const F gmx = fmav(mn[1] - mn[3], w1, ((mn[5] - mn[7]) + (mn[8] - mn[6])) * w2);
-    const F gmy = fmav(mn[2] - mn[4], w1, ((mn[5] - mn[7]) + (mn[6] - mn[8])) * w2);
     const F grx = fmav(rn[1] - rn[3], w1, ((rn[5] - rn[7]) + (rn[8] - rn[6])) * w2);
     const F gry = fmav(rn[2] - rn[4], w1, ((rn[5] - rn[7]) + (rn[6] - rn[8])) * w2);
-    const F Fx = fmav(-rho, gmx, fx), Fy = fmav(-rho, gmy, fy);
-    const F jx = mom_jx(v);
-    const F jy = mom_jy(v);
-    const F inv_rho = rcp_v(rho);
-    const F ux = fmav(F::c(0.5f), Fx, jx) * inv_rho;
-    const F uy = fmav(F::c(0.5f), Fy, jy) * inv_rho;
     // strain rate from the velocity stencil (Eq. 24)
     const F dxux = st.dxux, dyux = st.dyux, dxuy = st.dxuy, dyuy = st.dyuy;
     const F rA = rho * F::c(A);
@@ -113,6 +104,17 @@ __device__ __forceinline__ void fe_collide_iwb_v(F v[9], F rho, const F mn[9], c
     const F dpxx = fmav(F::c(2.0f * hn), fmav(ux, Gx, -(uy * Gy)), F::c(-P.s_nu) * nxx);
     const F dpxy = fmav(F::c(hn), fmav(ux, Gy, uy * Gx), F::c(-P.s_nu) * nxy);
     apply_dm_v<F, COMP>(v, de, dz, Fx, dqx, Fy, dqy, dpxx, dpxy, d0);
+}
+
+// The collision from the neighbours' mu: velocity and force recomputed (the same operations on the
+// same values as in the row pipeline's u, so a cell's stored u equals the u of its collision).
+template <class F, bool COMP = false>
+__device__ __forceinline__ void fe_collide_iwb_v(F v[9], F rho, const F mn[9], const F rn[9], const Strain<F>& st,
+                                                 F fx, F fy, F pg, float dpg, float A,
+                                                 const StepParams<float>& P, F* d0 = nullptr) {
+    F ux, uy, Fx, Fy;
+    fe_velocity_v(v, rho, mn, fx, fy, ux, uy, Fx, Fy);
+    fe_collide_iwb_u_v<F, COMP>(v, rho, rn, st, ux, uy, Fx, Fy, pg, dpg, A, P, d0);
 }
 
 // Shared memory of one CTA: S staged rows of the strip (its columns plus 8 halo columns on each
@@ -269,7 +271,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, 3) fe_iwb_pair(const float* __r
                 F2 v[9], mn[9];
                 pull_pair<WH>(sm.stage[(k - 4) % S], sm.stage[(k - 3) % S], sm.stage[(k - 2) % S], sc, v);
                 neighbours_pair(m3, m2, m1, mn);
-                fe_velocity_v(v, r2.c, mn, fx, fy_of(r2.c), ux, uy);
+                F2 Fx, Fy;
+                fe_velocity_v(v, r2.c, mn, fx, fy_of(r2.c), ux, uy, Fx, Fy);
             }
             ux2 = with_shifted(ux);
             uy2 = with_shifted(uy);

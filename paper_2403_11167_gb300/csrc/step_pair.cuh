@@ -72,7 +72,7 @@ __device__ __forceinline__ void neighbours_pair(const Row2& ym, const Row2& y0, 
 }
 
 // DRIVE: the droplet-collision drive of Sec. 5.4 adds a_x |rho - rho_ave| to each cell's x
-// force (rho_ave from D.rho_ave), and every consumer warp writes the sum of the populations it
+// force (rho_ave from D.parts), and every consumer warp writes the sum of the populations it
 // stored -- the mass of the next state, which on a periodic lattice holds each stored population
 // once -- to mass[((blockIdx.y * gridDim.x) + blockIdx.x) * NW + warp] (0 for idle warps), so
 // that the next step's rho_ave needs no pass over the lattice.
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
     r1.c = r2.c = r3.c = m2.c = m3.c = F2::c(1.0f);
     r1.xm = r1.xp = r2.xm = r2.xp = r3.xm = r3.xp = F2::c(1.0f);
     m2.xm = m2.xp = m3.xm = m3.xp = F2::c(1.0f);
-    const float rave = DRIVE ? (float)*D.rho_ave : 0.0f;
+    const float rave = DRIVE ? (float)drive_mean(D) : 0.0f;
     const F2 ax = DRIVE ? drive_ax(D, x0 + col) : F2::c(0.0f);
     F2 macc = F2::c(0.0f);
     bool ok = mbar_wait_bounded(&sm.full[0], 0) && mbar_wait_bounded(&sm.full[1], 0);
@@ -281,7 +281,7 @@ __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, flo
     p1.c = p2.c = F2::c(0.0f);
     p1.xm = p1.xp = p2.xm = p2.xp = F2::c(0.0f);
     F2 rho1 = F2::c(1.0f);  // rho of row q-1
-    const float rave = DRIVE ? (float)*D->rho_ave : 0.0f;
+    const float rave = DRIVE ? (float)drive_mean(*D) : 0.0f;
     const F2 ax = DRIVE ? drive_ax(*D, x0 + col) : F2::c(0.0f);
     F2 macc = F2::c(0.0f);
     bool ok = mbar_wait_bounded(&sm.full[0], 0) && mbar_wait_bounded(&sm.full[1], 0);

@@ -1,0 +1,431 @@
+// step_tile.cuh -- the step of every lattice that the TMA strip kernels do not serve: FP64, FP32
+// lattices whose width is not a multiple of 4 or that are too small for strips, no-slip walls, the
+// droplet-collision drive and the full free-energy model.
+//
+// A CTA updates a tile of at most kTileRows rows and one warp's columns.  Each warp holds one row
+// of the tile or of its halo; a lane holds two adjacent cells in FP32 (packed, F2) or one in FP64.
+// A warp pulls its row's populations once and keeps them in registers; the neighbour fields (psi;
+// rho and mu; rho, mu and u) go through shared memory between rows and through shuffles within a
+// row, one CTA barrier per field.  So the chain from the first load to the last store is one row's
+// work whatever the lattice, where a CTA that walks down a strip pays it once per row.
+//
+// What bounds it (GB300).  FP64: the FP64 pipe, 64 cycles per warp instruction on each of the 608
+// sub-partitions whatever the number of active lanes, so the arithmetic below is written for few
+// operations (step64.cuh) and the tile height spreads the rows over the sub-partitions
+// (tile_rows_f64 in lbm_api.cu).  FP32 on small lattices: the latency of one row's chain plus a
+// launch; on lattices that fill the GPU: instruction issue.
+//
+// Per-cell FP32 arithmetic is that of the strip kernels (lbm_kernels.cuh, step_iwb_pair.cuh) on
+// the same packed type, so both routes give the same bits.
+//
+// Walls (rows 0 and ny-1; see step_ext.cuh): halo rows beyond a wall are the mirrored rows; a wall
+// row's populations get the first fill when they are pulled and the final fill (J = -F/2) before
+// the collision (full model: before u).  band > 0 updates only the rows next to each wall (grid.y = 2).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "lbm_kernels.cuh"
+#include "step64.cuh"
+#include "step_ext.cuh"
+#include "step_iwb_pair.cuh"
+#include "step_pair.cuh"
+
+namespace lbmk {
+
+constexpr int kTileRows = 8;  // most rows of a tile
+
+// Lane layout of a tile row: V the cells of a lane, kPer of them; HC halo columns on each side of
+// the (at most) kCols columns a warp updates.  MODEL: 0 pseudopotential, 1 free energy, 2 full
+// free energy; LV is its number of halo rows.
+template <typename real, int MODEL>
+struct Tile {
+    using V = typename std::conditional<std::is_same<real, float>::value, F2, double>::type;
+    static constexpr int kPer = std::is_same<real, float>::value ? 2 : 1;
+    static constexpr int LV = MODEL + 1;
+    static constexpr int HC = kPer == 1 ? LV : (MODEL == 2 ? 4 : 2);
+    static constexpr int kCols = 32 * kPer - 2 * HC;
+    static constexpr int kThreads = 32 * (kTileRows + 2 * LV);
+};
+
+// The stored mass of driven steps.  FP64: one slot per tile row, summed by every CTA of the next
+// step.  FP32: fixed-point numbers of unit 2^9 rest_unit (2^-29 of the EOS packing limit, at or below
+// the rounding of the densities they add up), added atomically to kDriveParts accumulators: integer
+// sums are exact in any order, and cost a driven FP32 step no FP64 instructions but the mean's (with
+// FP64 sums per row a 1024^2 step took 38 us, with these 21 us).  Three sets of accumulators take
+// turns: a step reads the set of the step before, adds to its own and zeroes the next one's.
+constexpr double kTileMassUnit = 512.0;  // in units of rest_unit
+
+// What a tile step takes besides StepParams: the full model's terms, the walls' solved J_y, and the
+// drive: the state's mass is the sum of D.parts, of nslots slots (FP64), or of the accumulators acc_in.
+template <typename real>
+struct TileArgs {
+    int wb;    // columns per tile
+    int band;  // > 0: only the rows next to each wall
+    Ext<real> E;
+    real fyg, dpg;  // fy + rho_g g (the force is fyg - rho g) and d_y p_g = rho_g g
+    const real* wjy;
+    bool driven;
+    Drive<real> D;
+    const double* slots;
+    int nslots;
+    double* mass;  // the next state's slots (FP64)
+    const unsigned long long* acc_in;
+    unsigned long long *acc_out, *acc_zero;
+};
+
+template <class V>
+__device__ __forceinline__ V cst(double x) {
+    if constexpr (std::is_same<V, double>::value)
+        return x;
+    else
+        return V::c((float)x);
+}
+__device__ __forceinline__ F2 abs_v(F2 a) { return F2(fabsf(a.v.x), fabsf(a.v.y)); }
+
+// FP32: the strip kernels' arithmetic (step64.cuh has the FP64 overloads)
+__device__ __forceinline__ F2 tile_psi(F2 rho, const StepParams<float>& P) { return pseudo_psi_v(rho, P); }
+__device__ __forceinline__ F2 tile_mu(F2 rho, const F2 n[9], const StepParams<float>& P) { return fe_mu_v(rho, n, P); }
+__device__ __forceinline__ void tile_collide_pp(F2 v[9], F2 rho, const F2 pn[9], F2 fx, F2, unsigned& qw,
+                                                const StepParams<float>& P) {
+    F2 d0;
+    pp_collide_fx_v<F2, true>(v, rho, pn[0], pn, fx, P, &d0);
+    qw = rest_update_pair(v[0], qw, d0, P);
+}
+__device__ __forceinline__ void tile_collide_fe(F2 v[9], F2 rho, const F2 mn[9], const F2 rn[9], F2 fx, F2 fy,
+                                                unsigned& qw, const StepParams<float>& P) {
+    F2 d0;
+    fe_collide_f_v<F2, true>(v, rho, mn, rn, fx, fy, P, &d0);
+    qw = rest_update_pair(v[0], qw, d0, P);
+}
+__device__ __forceinline__ void tile_velocity(const F2 v[9], F2 rho, const F2 mn[9], F2 fx, F2 fy, F2& ux, F2& uy,
+                                              F2& Fx, F2& Fy) {
+    fe_velocity_v(v, rho, mn, fx, fy, ux, uy, Fx, Fy);
+}
+__device__ __forceinline__ void tile_collide_iwb(F2 v[9], F2 rho, const F2 rn[9], const F2 un[9], const F2 wn[9],
+                                                 F2 ux, F2 uy, F2 Fx, F2 Fy, float pg, float dpg, float A,
+                                                 unsigned& qw, const StepParams<float>& P) {
+    F2 d0;
+    fe_collide_iwb_u_v<F2, true>(v, rho, rn, strain_v(un, wn), ux, uy, Fx, Fy, F2::c(pg), dpg, A, P, &d0);
+    qw = rest_update_pair(v[0], qw, d0, P);
+}
+
+// A row of a field with its x-shifted values (Row2 of step_pair.cuh, for either type).
+template <class V>
+struct Row {
+    V c, xm, xp;
+};
+__device__ __forceinline__ Row<F2> shifted(F2 c) {
+    const Row2 r = with_shifted(c);
+    return {r.c, r.xm, r.xp};
+}
+__device__ __forceinline__ Row<double> shifted(double c) {
+    return {c, __shfl_up_sync(0xffffffffu, c, 1), __shfl_down_sync(0xffffffffu, c, 1)};
+}
+template <class V>
+__device__ __forceinline__ void neighbours(const Row<V>& ym, const Row<V>& y0, const Row<V>& yp, V n[9]) {
+    n[0] = y0.c;
+    n[1] = y0.xp;
+    n[2] = yp.c;
+    n[3] = y0.xm;
+    n[4] = ym.c;
+    n[5] = yp.xp;
+    n[6] = yp.xm;
+    n[7] = ym.xm;
+    n[8] = ym.xp;
+}
+
+// Pulled populations of a lane's cells from global memory; om, o0, op: offsets of rows y-1, y, y+1;
+// xl, xa, xb, xr: wrapped columns of the cell before, the lane's cells (one in FP64: xb unused) and
+// the cell after.  EVEN: nx is even, so a lane's two cells are 8-byte aligned.
+template <bool EVEN>
+__device__ __forceinline__ void pull_tile(const float* __restrict__ f, long long pitch, int xl, int xa, int xb, int xr,
+                                          long long om, long long o0, long long op, F2 v[9]) {
+    auto pair = [](const float* p, int a, int b) {
+        if constexpr (EVEN)
+            return F2(__ldg(reinterpret_cast<const float2*>(p + a)));
+        else
+            return F2(__ldg(p + a), __ldg(p + b));
+    };
+    auto two = [](const float* p, int a, int b) { return F2(__ldg(p + a), __ldg(p + b)); };
+    v[0] = pair(f + o0, xa, xb);
+    v[1] = two(f + 1 * pitch + o0, xl, xa);
+    v[2] = pair(f + 2 * pitch + om, xa, xb);
+    v[3] = two(f + 3 * pitch + o0, xb, xr);
+    v[4] = pair(f + 4 * pitch + op, xa, xb);
+    v[5] = two(f + 5 * pitch + om, xl, xa);
+    v[6] = two(f + 6 * pitch + om, xb, xr);
+    v[7] = two(f + 7 * pitch + op, xb, xr);
+    v[8] = two(f + 8 * pitch + op, xl, xa);
+}
+template <bool EVEN>
+__device__ __forceinline__ void pull_tile(const double* __restrict__ f, long long pitch, int xl, int xa, int, int xr,
+                                          long long om, long long o0, long long op, double v[9]) {
+    pull9(f, pitch, xa, xl, xr, om, o0, op, v);
+}
+
+// Zou-He completion of a wall row's cells (wall_fill of step_ext.cuh).
+template <class V>
+__device__ __forceinline__ void tile_wall_fill(V v[9], bool top, V Jx, V Jy) {
+    const V h = cst<V>(0.5) * (v[1] - v[3]);
+    const V hx = cst<V>(0.5) * Jx, sy = Jy * cst<V>(1.0 / 6.0), ty = Jy * cst<V>(2.0 / 3.0);
+    if (!top) {
+        v[2] = v[4] + ty;
+        v[5] = (v[7] - h) + (hx + sy);
+        v[6] = (v[8] + h) - (hx - sy);
+    } else {
+        v[4] = v[2] - ty;
+        v[7] = (v[5] + h) - (hx + sy);
+        v[8] = (v[6] - h) + (hx - sy);
+    }
+}
+// x component of the Eq. (24) gradient
+template <class V>
+__device__ __forceinline__ V tile_grad_x(const V n[9]) {
+    return fmav(n[1] - n[3], cst<V>(1.0 / 3.0), ((n[5] - n[7]) + (n[8] - n[6])) * cst<V>(1.0 / 12.0));
+}
+// wall-normal gradient of the one-sided reading (wall_grad_y_onesided)
+template <class V>
+__device__ __forceinline__ V tile_grad_y_onesided(const V n[9], bool top) {
+    const V a = cst<V>(2.0 / 3.0), d = cst<V>(1.0 / 6.0);
+    if (!top) return fmav(a, n[2] - n[0], d * ((n[5] - n[1]) + (n[6] - n[3])));
+    return -fmav(a, n[4] - n[0], d * ((n[8] - n[1]) + (n[7] - n[3])));
+}
+
+template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN>
+__global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
+    tile_step(const real* __restrict__ fin, real* __restrict__ fout, const StepParams<real> P,
+              const TileArgs<real> T) {
+    using L = Tile<real, MODEL>;
+    using V = typename L::V;
+    constexpr int LV = L::LV, HC = L::HC, KP = L::kPer, RMAX = kTileRows + 2 * LV;
+    __shared__ V s_a[RMAX][32];                        // psi or rho
+    __shared__ V s_mu[MODEL > 0 ? RMAX : 1][32];       // mu
+    __shared__ V s_u[MODEL > 1 ? 2 * RMAX : 1][32];    // u_x, then u_y
+    __shared__ double s_mass[16];
+    __shared__ real s_rave;
+    const int nx = P.nx, ny = P.ny;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nwarps = blockDim.x >> 5, rows = nwarps - 2 * LV;
+    const int by = blockIdx.y + gridDim.y * blockIdx.z;  // more than 65535 tiles in y use z
+    const int y0 = WALLS && T.band > 0 ? (by == 0 ? 0 : ny - T.band) : by * rows;
+    if (y0 >= ny) return;
+    const int y1 = WALLS && T.band > 0 ? y0 + T.band : min(y0 + rows, ny);
+    const int x0 = blockIdx.x * T.wb;
+    const int w = min(T.wb, nx - x0);  // > 0 (the host's grid)
+    const int y = y0 - LV + warp;      // this warp's row (rows beyond the lattice mirrored or wrapped)
+    const int yr = WALLS ? mirror_row(y, ny) : wrap_idx(y, ny);
+    const bool wall = WALLS && (y == 0 || y == ny - 1);      // a wall row of the lattice or its image
+    const bool wall_img = WALLS && (yr == 0 || yr == ny - 1);
+    const bool top = WALLS && yr != 0;
+    const int c = KP * lane - HC;  // first column of the lane, from x0
+    const bool out_row = warp >= LV && y < y1;
+    const bool out_a = out_row && c >= 0 && c < w;
+    const bool out_b = KP == 2 && out_row && c >= 0 && c + 1 < w;
+    const long long oc = (long long)y * nx + x0 + c;  // (out rows and lanes only)
+
+    // the state's mean density: every CTA sums in the same order
+    if constexpr (DRIVE) {
+        if (KP == 1 && T.nslots > 0) {
+            double s = 0.0;
+            for (int k = threadIdx.x; k < T.nslots; k += blockDim.x) s += __ldg(T.slots + k);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) s_mass[warp] = s;
+        } else if (warp == 0) {
+            double m;
+            if (KP == 2 && T.acc_in) {
+                unsigned long long s = T.acc_in[lane];
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                m = (double)(long long)s * (kTileMassUnit * (double)P.rest_unit * T.D.inv_cells);
+            } else {
+                m = drive_mean(T.D);
+            }
+            if (lane == 0) s_rave = (real)m;
+        }
+        if (KP == 2 && blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
+    }
+
+    V v[9], rho = cst<V>(1.0), f0 = cst<V>(0.0);  // f0: psi (MODEL 0)
+    [[maybe_unused]] unsigned qw = 0;              // FP32: the cells' int16 rest extensions
+    if (y < y1 + LV && c < w + HC) {
+        int xl = x0 + c - 1, xa = x0 + c, xb = x0 + c + 1, xr = x0 + c + KP;
+        auto wrap = [nx](int x) {
+            while (x < 0) x += nx;
+            while (x >= nx) x -= nx;
+            return x;
+        };
+        xl = wrap(xl);
+        xa = wrap(xa);
+        xb = wrap(xb);
+        xr = wrap(xr);
+        const long long o0 = (long long)yr * nx, om = yr == 0 ? (long long)(ny - 1) * nx : o0 - nx,
+                        op = yr == ny - 1 ? 0 : o0 + nx;
+        pull_tile<EVEN>(fin, P.pitch, xl, xa, xb, xr, om, o0, op, v);
+        if constexpr (std::is_same<real, float>::value) {
+            const short* q = rest_lo_plane(fin, P.pitch);
+            if constexpr (EVEN) {
+                if (out_a) qw = __ldg(reinterpret_cast<const unsigned*>(q + oc));
+            } else {
+                if (out_a) qw = (unsigned)(unsigned short)__ldg(q + oc);
+                if (out_b) qw |= (unsigned)(unsigned short)__ldg(q + oc + 1) << 16;
+            }
+        }
+        if (wall_img) {
+            // first fill: J = (0, -fy/2), or the solved J_y of the one-sided reading
+            V jy = cst<V>(real(-0.5) * P.fy);
+            if (MODEL > 0 && T.wjy) {
+                if constexpr (KP == 1)
+                    jy = T.wjy[(top ? nx : 0) + xa];
+                else
+                    jy = F2(T.wjy[(top ? nx : 0) + xa], T.wjy[(top ? nx : 0) + xb]);
+            }
+            tile_wall_fill(v, top, cst<V>(0.0), jy);
+            if (MODEL == 2 && !T.wjy && T.E.g != real(0)) {
+                // gravity: the wall node's density solved in closed form (wall_gravity_refill)
+                const real sg = top ? real(-0.5) : real(0.5);
+                const V rw = (sum9_v(v) - cst<V>(sg * T.dpg)) * cst<V>(real(1) / (real(1) - sg * T.E.g));
+                tile_wall_fill(v, top, cst<V>(0.0), cst<V>(-0.5) * fmav(cst<V>(-T.E.g), rw, cst<V>(T.fyg)));
+            }
+        }
+        rho = sum9_v(v);
+        if (MODEL == 0) f0 = tile_psi(rho, P);
+    }
+    s_a[warp][lane] = MODEL == 0 ? f0 : rho;
+    __syncthreads();
+
+    // external force of the lane's cells (body force, drive, buoyancy)
+    V fx = cst<V>(P.fx), fy = cst<V>(P.fy);
+    if constexpr (DRIVE) {
+        real rave;
+        if (KP == 1 && T.nslots > 0) {
+            double s = (lane & 15) < nwarps ? s_mass[lane & 15] : 0.0;
+            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            rave = (real)(s * T.D.inv_cells);
+        } else {
+            rave = s_rave;
+        }
+        const int gx = x0 + c;
+        const real al = gx <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi, ah = gx + 1 <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi;
+        if constexpr (KP == 1)
+            fx = fma(al, fabs(rho - rave), fx);
+        else
+            fx = fmav(F2(al, ah), abs_v(rho - F2::c(rave)), fx);
+    }
+    if (MODEL == 2) fy = fmav(cst<V>(-T.E.g), rho, cst<V>(T.fyg));
+
+    if constexpr (MODEL == 0) {
+        if (!out_row) return;
+        V pn[9];
+        neighbours(shifted(s_a[warp - 1][lane]), shifted(f0), shifted(s_a[warp + 1][lane]), pn);
+        if (wall) {
+            mirror_neighbours(pn, top);
+            const V Fx = fmav(pn[0], tile_grad_x(pn), fx);  // Eq. (10) + external
+            tile_wall_fill(v, top, cst<V>(-0.5) * Fx, cst<V>(-0.5) * fy);
+        }
+        tile_collide_pp(v, rho, pn, fx, fy, qw, P);
+    } else {
+        Row<V> rm, r0 = shifted(rho), rp, m0;
+        V mu = cst<V>(0.0);
+        if (warp >= 1 && warp < nwarps - 1 && y < y1 + LV - 1) {
+            rm = shifted(s_a[warp - 1][lane]);
+            rp = shifted(s_a[warp + 1][lane]);
+            V n[9];
+            neighbours(rm, r0, rp, n);
+            mu = tile_mu(rho, n, P);
+        }
+        s_mu[warp][lane] = mu;
+        __syncthreads();
+        if constexpr (MODEL == 1) {
+            if (!out_row) return;
+            V mn[9], rn[9];
+            neighbours(shifted(s_mu[warp - 1][lane]), shifted(mu), shifted(s_mu[warp + 1][lane]), mn);
+            neighbours(rm, r0, rp, rn);
+            if (wall) {
+                // the one-sided reading's normal force -rho d_y mu enters through fy
+                if (T.wjy) fy = fmav(-rho, tile_grad_y_onesided(mn, top), fy);
+                mirror_neighbours(mn, top);
+                mirror_neighbours(rn, top);
+                const V Fx = fmav(-rho, tile_grad_x(mn), fx);
+                tile_wall_fill(v, top, cst<V>(-0.5) * Fx, cst<V>(-0.5) * fy);
+            }
+            tile_collide_fe(v, rho, mn, rn, fx, fy, qw, P);
+        } else {
+            V ux = cst<V>(0.0), uy = cst<V>(0.0), Fx = cst<V>(0.0), Fy = cst<V>(0.0);
+            if (warp >= 2 && warp < nwarps - 2 && y < y1 + 1) {
+                V mn[9];
+                neighbours(shifted(s_mu[warp - 1][lane]), shifted(mu), shifted(s_mu[warp + 1][lane]), mn);
+                if (wall) {
+                    if (T.wjy) fy = fmav(-rho, tile_grad_y_onesided(mn, top), fy);
+                    mirror_neighbours(mn, top);
+                    const V Gx = fmav(-rho, tile_grad_x(mn), fx);
+                    tile_wall_fill(v, top, cst<V>(-0.5) * Gx, cst<V>(-0.5) * fy);
+                }
+                tile_velocity(v, rho, mn, fx, fy, ux, uy, Fx, Fy);
+            }
+            s_u[warp][lane] = ux;
+            s_u[RMAX + warp][lane] = uy;
+            __syncthreads();
+            if (!out_row) return;
+            V rn[9], un[9], wn[9];
+            neighbours(rm, r0, rp, rn);
+            neighbours(shifted(s_u[warp - 1][lane]), shifted(ux), shifted(s_u[warp + 1][lane]), un);
+            neighbours(shifted(s_u[RMAX + warp - 1][lane]), shifted(uy), shifted(s_u[RMAX + warp + 1][lane]), wn);
+            if (wall) {
+                mirror_neighbours(rn, top);
+                // velocities beyond a no-slip wall: odd extension through u = 0 at the wall node
+                mirror_neighbours(un, top);
+                mirror_neighbours(wn, top);
+                const int i0 = top ? 2 : 4, i1 = top ? 5 : 7, i2 = top ? 6 : 8;
+#pragma unroll
+                for (int i = 1; i < 9; ++i)
+                    if (i == i0 || i == i1 || i == i2) {
+                        un[i] = -un[i];
+                        wn[i] = -wn[i];
+                    }
+            }
+            tile_collide_iwb(v, rho, rn, un, wn, ux, uy, Fx, Fy, T.dpg * ((real)y - T.E.y_ref), T.dpg, T.E.A, qw, P);
+        }
+    }
+
+    if constexpr (DRIVE) {
+        // the mass this warp stored
+        if constexpr (KP == 1) {
+            double s = out_a ? sum9_v(v) : 0.0;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) T.mass[(long long)y * gridDim.x + blockIdx.x] = s;
+        } else {
+            const F2 m = sum9_v(v) * F2::c(P.rest_inv * (float)(1.0 / kTileMassUnit));
+            const int k = out_a ? __float2int_rn(m.v.x) : 0, l = out_b ? __float2int_rn(m.v.y) : 0;
+            // each below 2^30: summed over the warp in two 16-bit halves
+            const int lo = __reduce_add_sync(0xffffffffu, (k & 0xffff) + (l & 0xffff));
+            const int hi = __reduce_add_sync(0xffffffffu, (k >> 16) + (l >> 16));
+            if (lane == 0)
+                atomicAdd(T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts,
+                          (unsigned long long)(((long long)hi << 16) + lo));
+        }
+    }
+    if constexpr (KP == 1) {
+        if (out_a)
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fout[i * P.pitch + oc] = v[i];
+    } else if constexpr (EVEN) {
+        if (out_a) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(fout + i * P.pitch + oc) = v[i].v;
+            *reinterpret_cast<unsigned*>(rest_lo_plane(fout, P.pitch) + oc) = qw;
+        }
+    } else {
+        short* q = rest_lo_plane(fout, P.pitch);
+        if (out_a) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fout[i * P.pitch + oc] = v[i].v.x;
+            q[oc] = (short)(qw & 0xffffu);
+        }
+        if (out_b) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fout[i * P.pitch + oc + 1] = v[i].v.y;
+            q[oc + 1] = (short)(qw >> 16);
+        }
+    }
+}
+
+}  // namespace lbmk

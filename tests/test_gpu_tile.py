@@ -1,0 +1,121 @@
+"""The tile step kernel: tile edges of both precisions and every option against the FP64 oracle, and
+the size rule that takes FP32 lattices to the strip kernels (the same bits on either side)."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2403_11167_gb300 import inputs
+from helpers import gpu_context, oracle_params, pop_err
+
+pytestmark = pytest.mark.gpu
+
+PP, FE = 0, 1
+F32, F64 = 0, 1
+STEPS = 12
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+
+    import __graft_entry__
+
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+# one cell, fewer columns than the halo, one column below / at / above a tile (FP32 60 and 56, FP64
+# 30, 28 and 26 columns), two tiles, rows around the tile heights 1 .. 8
+SHAPES = [(1, 1), (2, 5), (27, 1), (31, 9), (59, 4), (60, 8), (61, 7), (113, 17)]
+
+
+@pytest.mark.parametrize("option", ["plain", "drive", "A", "walls", "onesided"])
+@pytest.mark.parametrize("model", [PP, FE])
+@pytest.mark.parametrize("precision", [F64, F32])
+def test_tile_edges_against_oracle(model, precision, option):
+    """Random densities: every population after 12 steps, FP64 within 1e-11 and FP32 within 5e-6 of
+    its cell's density (12 steps of at most 3 roundings of 2^-24 on sums of up to a few densities)."""
+    from paper_2403_11167_gb300 import lbm
+
+    if model == PP and option in ("A", "onesided"):
+        pytest.skip("free-energy terms")
+    for nx, ny in SHAPES:
+        walls = {"walls": 1, "onesided": 2}.get(option, 0)
+        if walls and ny < 4:
+            continue
+        kw = dict(a=0.25, Tr=0.85, tau_nu=0.9, body_fx=1e-5, body_fy=0.0 if walls == 1 else -2e-5)
+        if model == PP:
+            kw.update(kappa_P=0.7, kappa_Li=-0.2)
+        if option in ("A", "onesided"):
+            kw["A"] = 0.1 if option == "A" or ny % 2 else 0.0
+        ctx, rp, th = gpu_context(model, precision, nx, ny, walls=walls, **kw)
+        rho0 = inputs.random_field(nx, ny, th.rho_v * 1.5, th.rho_l * 0.8, seed=nx + ny)
+        p = oracle_params(rp, th, walls=walls)
+        if option == "onesided":
+            ctx.set_gravity(1e-5, 0.1, 0.5 * ny)
+            p.g, p.rho_g, p.y_ref = 1e-5, 0.1, 0.5 * ny
+        f0 = O.init_iwb(p, rho0) if option == "onesided" else O.init(model, rho0)
+        ctx.set_density(rho0)
+        if option == "drive":
+            ctx.set_drive(5e-4, -3e-4, nx // 2, 2)
+            p.drive_ax_lo, p.drive_ax_hi, p.drive_x_split = 5e-4, -3e-4, nx // 2
+            f_ref = O.run_driven(model, p, f0, STEPS, t0=0, t_on=2)
+        else:
+            f_ref = O.run(model, p, f0, STEPS)
+        ctx.step(STEPS)
+        err = pop_err(ctx.populations(), f_ref)
+        assert err < (1e-11 if precision == F64 else 5e-6), (nx, ny, err)
+        assert ctx.observables(0)["status"] == lbm.LBM_OK
+        ctx.close()
+
+
+def _device_populations(ctx):
+    import torch
+
+    ctx.synchronize()
+    ptr, pitch = ctx.device_populations()
+    off = ptr - ctx.workspace.data_ptr()
+    planes = ctx.workspace[off:off + 40 * pitch].view(torch.int32).view(10, pitch)
+    n = ctx.nx * ctx.ny
+    return planes[:9, :n].clone(), planes[9].view(torch.int16)[:n].clone()
+
+
+@pytest.mark.parametrize("case", [
+    (PP, 2052, 2196, {}), (PP, 8, 563000, {}), (PP, 600004, 8, {}), (PP, 4100, 1101, {}),
+    (FE, 1684, 1680, {}), (FE, 8, 350400, {}), (FE, 300004, 10, {}), (FE, 484, 5801, {}),
+    (FE, 1684, 1680, dict(A=0.15)), (FE, 300004, 10, dict(A=0.1)),
+    (PP, 1848, 1844, dict(walls=1)), (FE, 1452, 1450, dict(walls=1)), (FE, 1452, 1450, dict(walls=2)),
+    (PP, 1740, 1732, dict(drive=5e-4)), (FE, 1228, 1226, dict(drive=5e-4))])
+def test_strips_match_tiles(case, monkeypatch):
+    """Just above the size rule a lattice runs the strip kernels, with LBM_NO_TMA the tile kernel: the
+    same bits, rest extensions included, after one graph of steps and some single ones (square, one
+    narrow strip, few rows, uneven strips, walls, the drive).  The driven routes sum rho_ave in
+    different units, which may change a force of 1e-4 by rounding: within 1e-6."""
+    import torch
+
+    model, nx, ny, opt = case
+    walls = opt.get("walls", 0)
+    kw = dict(a=0.25, Tr=0.85, tau_nu=0.8, body_fx=1e-6 if walls else 0.0, body_fy=-1e-6 if walls == 2 else 0.0)
+    if "A" in opt:
+        kw["A"] = opt["A"]
+    rng = torch.Generator(device="cuda").manual_seed(nx)
+    got = []
+    for tiles in (False, True):
+        if tiles:
+            monkeypatch.setenv("LBM_NO_TMA", "1")
+        ctx, rp, th = gpu_context(model, F32, nx, ny, walls=walls, **kw)
+        if not tiles:
+            rho = 0.5 * (th.rho_l + th.rho_v) * (0.98 + 0.04 * torch.rand((ny, nx), device="cuda", generator=rng))
+            torch.cuda.synchronize()
+        ctx.set_density_device(rho)
+        if "drive" in opt:
+            ctx.set_drive(opt["drive"], -opt["drive"], nx // 2, -1)
+        ctx.step(67)
+        got.append(_device_populations(ctx))
+        ctx.close()
+    (fa, qa), (fb, qb) = got
+    if "drive" in opt:
+        a, b = fa.view(torch.float32), fb.view(torch.float32)
+        assert float((a - b).abs().max()) <= 1e-6 * float(b.abs().max())
+    else:
+        assert torch.equal(fa, fb) and torch.equal(qa, qb)
