@@ -10,11 +10,12 @@
 //                         rho (2 N floats) fit in one CTA's shared
 //                         memory: one CTA per lattice runs every step of that lattice in
 //                         shared memory, in one persistent launch (no HBM traffic per step);
-//   tiled lattices     -- the rest: a work table of (lattice, strip) items; one launch per
-//                         time step runs the two-cells-per-lane TMA strip of the context
-//                         path (pp_pair_strip) over every active lattice,
-//                         replayed as captured 64-step CUDA graphs on a second stream,
-//                         concurrently with the resident launch.
+//   tiled lattices     -- the rest: one launch per time step over a work table, replayed as
+//                         captured 64-step CUDA graphs on a second stream, concurrently with
+//                         the resident launch.  While the unfinished lattices hold many cells
+//                         the table is one of (lattice, strip) items for the two-cells-per-lane
+//                         TMA strip of the context path (pp_pair_strip), then one of tiles for
+//                         CTAs that each take a run of them (pp_batch_tile).
 //
 // An autotuner picks the resident block size and the strip height by timing short trials
 // (cached per shape class for the process), and orders work longest-first.
@@ -36,6 +37,7 @@
 #include "lbm_kernels.cuh"
 #include "ring.cuh"
 #include "step_pair.cuh"
+#include "tile.h"
 #include "rest_host.h"
 
 namespace {
@@ -57,6 +59,12 @@ static_assert(kBPStages >= 4, "the pseudopotential strip ring needs at least 4 s
 using BPSmem = lbmk::WarpStripSmem<kBPWarps, kBPStages, 60>;
 constexpr int kBPTX = BPSmem::TX;  // widest pair strip (240 columns)
 constexpr int kChunk = 64;       // steps per captured graph
+constexpr int kTileCtasPerSM = 4;          // resident CTAs of the tile kernel
+// Unfinished cells from which strips are the faster step (24 lattices of 192^2 .. 512^2, 0.8 million
+// cells: 6.5 ms with tiles, 10.4 with strips; 96 lattices, 3.9 million cells at first, 100 .. 400 steps:
+// 27.2 ms with tiles only, 25.6 with strips only, 24.7 with this rule, 24.9 and 24.6 with 1.5 and 3.5
+// million).
+constexpr long long kStripCells = 2500000;
 constexpr size_t kResidentSmemMax = 200 * 1024;
 
 struct BatchLattice {
@@ -152,21 +160,104 @@ __global__ void __launch_bounds__(1024, 1)
 
 // Tiled lattices, two cells per lane: one strip of one lattice per CTA, one step per launch.
 template <int NW, int S>
-__global__ void __launch_bounds__((NW + 1) * 32, 1)
+__global__ void __launch_bounds__((NW + 1) * 32, 4)
     pp_batch_pair(const BatchLattice* __restrict__ lats, const BatchItem* __restrict__ items,
-                  const int* __restrict__ step_base, int k, int* __restrict__ err) {
+                  const int* __restrict__ state, int k, int* __restrict__ err) {
     using Smem = WarpStripSmem<NW, S, 60>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
     const BatchItem it = items[blockIdx.x];
     const BatchLattice& L = lats[it.lat];
-    const int step = *step_base + k;
+    const int step = state[0] + k;
     if (step >= L.nsteps) return;
-    const StepParams<float> P = L.P;
+    // in shared memory, not in registers: 94 of them allow four CTAs per SM, 110 three (a sweep of 3.9
+    // million cells: 25.6 ms against 29.1)
+    __shared__ StepParams<float> P;
+    if (threadIdx.x < sizeof(P) / 4)
+        reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
+    __syncthreads();
     pp_pair_strip<NW, S>(L.buf[step & 1], L.buf[(step + 1) & 1], P, it.x0, it.w, it.y0, it.y1, sm, err);
 }
 
-__global__ void advance_step(int* step_base, int by) { *step_base += by; }
+// The same lattices in tiles of kBatchTileRows rows, one row per warp (step_tile.cuh): CTA b takes its
+// share of the tiles of the unfinished lattices, which head the table (state[1] of them), one after the
+// other.  Neighbouring tiles follow each other, so their common halo rows are still in L1; a lattice's
+// constants are read from shared memory where they are used, because held in registers they would cost
+// CTAs per SM.  (Copying the next tile's rows to shared memory ahead, two cp.async stages per warp, made
+// a sweep that exceeds L2 3% faster and a small one 8% slower; the strips are faster there.)
+constexpr int kBatchTileRows = 4;
+__global__ void __launch_bounds__(32 * (kBatchTileRows + 2))
+    pp_batch_tile(const BatchLattice* __restrict__ lats, const BatchItem* __restrict__ tiles,
+                  const int* __restrict__ state, int k) {
+    constexpr int R = kBatchTileRows;
+    __shared__ F2 s_psi[2][R + 2][32];
+    __shared__ StepParams<float> P;
+    const int step = state[0] + k, count = state[1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, c = 2 * lane - 2;
+    const int i1 = (int)((long long)count * (blockIdx.x + 1) / gridDim.x);
+    int lat = -1, par = 0;
+    bool done = false;
+    const float* fin = nullptr;
+    float* fout = nullptr;
+    for (int i = (int)((long long)count * blockIdx.x / gridDim.x); i < i1; ++i) {
+        const BatchItem it = tiles[i];
+        if (it.lat != lat) {
+            lat = it.lat;
+            const BatchLattice& L = lats[lat];
+            done = step >= L.nsteps;
+            fin = L.buf[step & 1];
+            fout = L.buf[(step + 1) & 1];
+            __syncthreads();  // every warp is done with the previous lattice's constants
+            if (threadIdx.x < sizeof(P) / 4)
+                reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
+            __syncthreads();
+        }
+        if (done) continue;
+        const int nx = P.nx, ny = P.ny, y = it.y0 - 1 + warp;
+        F2 v[9], rho = F2::c(1.0f), psi = F2::c(0.0f);
+        unsigned qw = 0;
+        const bool out_row = warp >= 1 && y < it.y1;
+        const bool out = out_row && c >= 0 && c < it.w;
+        const long long oc = (long long)y * nx + it.x0 + c;
+        if (y < it.y1 + 1 && c < it.w + 2) {
+            // lattices of the table are at least 8 wide and 4 tall: one wrap each way
+            const int yr = wrap_once(y, ny), xa = wrap_once(it.x0 + c, nx);
+            const int xl = xa == 0 ? nx - 1 : xa - 1, xr = wrap_once(xa + 2, nx);
+            const long long o0 = (long long)yr * nx, om = yr == 0 ? (long long)(ny - 1) * nx : o0 - nx,
+                            op = yr == ny - 1 ? 0 : o0 + nx;
+            pull_tile<true>(fin, P.pitch, xl, xa, xa + 1, xr, om, o0, op, v);
+            if (out) qw = __ldg(reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch) + oc));
+            rho = sum9_v(v);
+            psi = pseudo_psi_v(rho, P);
+        }
+        F2(*s)[32] = s_psi[par];  // two buffers: the next tile's psi may be written before this one's is read
+        par ^= 1;
+        s[warp][lane] = psi;
+        __syncthreads();
+        if (!out_row) continue;
+        F2 pn[9];
+        neighbours(shifted(s[warp - 1][lane]), shifted(psi), shifted(s[warp + 1][lane]), pn);
+        tile_collide_pp(v, rho, pn, F2::c(P.fx), F2::c(P.fy), qw, P);
+        if (out) {
+#pragma unroll
+            for (int j = 0; j < 9; ++j) *reinterpret_cast<float2*>(fout + j * P.pitch + oc) = v[j].v;
+            *reinterpret_cast<unsigned*>(rest_lo_plane(fout, P.pitch) + oc) = qw;
+        }
+    }
+}
+
+// Start (by < 0) or advance the tiled lattices' clock: state[0] the steps done, state[1] the tiles of
+// the lattices (order: their step counts and tiles) that are not finished by then.
+__global__ void batch_clock_kernel(int* state, int by, const int2* __restrict__ order, int n) {
+    const int base = by < 0 ? 0 : state[0] + by;
+    int tiles = 0;
+    for (int i = threadIdx.x; i < n; i += 32) tiles += order[i].x > base ? order[i].y : 0;
+    tiles = __reduce_add_sync(0xffffffffu, tiles);
+    if (threadIdx.x == 0) {
+        state[0] = base;
+        state[1] = tiles;
+    }
+}
 
 // Observables of every lattice (one CTA per lattice): rho and psi of the final state into
 // the lattice scratch, then u (Eq. 6b with the Shan-Chen force), mass, u_max, probes,
@@ -273,7 +364,9 @@ struct lbm_batch {
     std::vector<lbm_batch_lattice> spec;
     std::vector<BatchLattice> lat;       // host copy of the device table
     std::vector<int> resident_ids;       // sorted longest-first
-    std::vector<BatchItem> items;        // sorted by lattice nsteps, longest first
+    std::vector<BatchItem> items;        // strips, sorted by lattice nsteps, longest first
+    std::vector<BatchItem> tiles;        // tiles, in the same order of lattices
+    std::vector<int2> order;             // tiled lattices in that order: steps, tiles
     int max_tiled_steps;
     int resident_threads;
     size_t resident_smem;
@@ -281,6 +374,8 @@ struct lbm_batch {
     char* pool;
     BatchLattice* d_lat;
     BatchItem* d_items;
+    BatchItem* d_tiles;
+    int2* d_order;
     int* d_ids;
     int* d_step;
     int* d_err;
@@ -288,7 +383,7 @@ struct lbm_batch {
     std::vector<double> h_obs;
     cudaStream_t s_res, s_tile;
     cudaEvent_t ev_fork, ev_join;
-    cudaGraphExec_t chunk;
+    cudaGraphExec_t chunk[2];            // kChunk steps with strips, with tiles
     bool ran;
     std::vector<std::vector<double>> rho0;  // kept for re-initialisation after autotuning trials
 };
@@ -316,8 +411,8 @@ int batch_init_state(lbm_batch* b) {
             L.P.rest_inv);
     }
     BCK(cudaGetLastError());
-    const int zero = 0;
-    BCK(cudaMemcpyAsync(b->d_step, &zero, sizeof(int), cudaMemcpyHostToDevice, b->s_tile));
+    if (b->d_order) lbmk::batch_clock_kernel<<<1, 32, 0, b->s_tile>>>(b->d_step, -1, b->d_order, (int)b->order.size());
+    BCK(cudaGetLastError());
     BCK(cudaMemsetAsync(b->d_err, 0, sizeof(int) * 16, b->s_tile));
     BCK(cudaStreamSynchronize(b->s_tile));
     return LBM_OK;
@@ -331,11 +426,42 @@ int launch_resident(lbm_batch* b, int step_limit, cudaStream_t s) {
     return LBM_OK;
 }
 
+int launch_tile_step(lbm_batch* b, int k, cudaStream_t s) {
+    const int grid = (int)std::min<size_t>(b->tiles.size(), 152 * kTileCtasPerSM);
+    lbmk::pp_batch_tile<<<grid, 32 * (lbmk::kBatchTileRows + 2), 0, s>>>(b->d_lat, b->d_tiles, b->d_step, k);
+    BCK(cudaGetLastError());
+    return LBM_OK;
+}
+
 int launch_tiled_step(lbm_batch* b, int k, cudaStream_t s) {
     if (b->items.empty()) return LBM_OK;
     lbmk::pp_batch_pair<kBPWarps, kBPStages><<<(unsigned)b->items.size(), (kBPWarps + 1) * 32, sizeof(BPSmem), s>>>(
         b->d_lat, b->d_items, b->d_step, k, b->d_err);
     BCK(cudaGetLastError());
+    return LBM_OK;
+}
+
+// Tiles of every tiled lattice, longest lattice first, and the lattices in that order.
+int build_tiles(lbm_batch* b) {
+    std::vector<int> ids;
+    for (int i = 0; i < b->n; ++i)
+        if (!b->lat[i].resident) ids.push_back(i);
+    if (ids.empty()) return LBM_OK;
+    std::stable_sort(ids.begin(), ids.end(), [&](int x, int y) { return b->lat[x].nsteps > b->lat[y].nsteps; });
+    for (int i : ids) {
+        const int nx = b->lat[i].P.nx, ny = b->lat[i].P.ny, wb = lbmk::tile_columns<float>(0, nx);
+        const size_t first = b->tiles.size();
+        for (int y0 = 0; y0 < ny; y0 += lbmk::kBatchTileRows)
+            for (int x0 = 0; x0 < nx; x0 += wb)
+                b->tiles.push_back(
+                    BatchItem{i, x0, std::min(wb, nx - x0), y0, std::min(y0 + lbmk::kBatchTileRows, ny)});
+        b->order.push_back(make_int2(b->lat[i].nsteps, (int)(b->tiles.size() - first)));
+    }
+    const size_t tb = sizeof(BatchItem) * b->tiles.size(), ob = sizeof(int2) * b->order.size();
+    BCK(cudaMalloc(&b->d_tiles, tb));
+    BCK(cudaMemcpy(b->d_tiles, b->tiles.data(), tb, cudaMemcpyHostToDevice));
+    BCK(cudaMalloc(&b->d_order, ob));
+    BCK(cudaMemcpy(b->d_order, b->order.data(), ob, cudaMemcpyHostToDevice));
     return LBM_OK;
 }
 
@@ -429,6 +555,7 @@ int autotune(lbm_batch* b) {
             if (it != g_tune_cache.end()) choice = it->second;
         }
         if (const char* e = std::getenv("LBM_BATCH_ROWS")) choice = std::max(1, std::atoi(e));  // tuning experiments
+        if (choice < 0 && cells < kStripCells) choice = 32;  // the strips will not run
         if (choice < 0) {
             // two passes in opposite orders, 16 steps per trial, best time per candidate:
             // a single short pass in one order favoured whichever candidate ran last
@@ -471,6 +598,27 @@ int autotune(lbm_batch* b) {
     return batch_init_state(b);  // trials advanced the state: start again from f^eq(rho0)
 }
 
+// kChunk steps of the tiled lattices and the clock step as a graph.
+int capture_chunk(lbm_batch* b, bool strips, cudaGraphExec_t* out) {
+    cudaGraph_t g = nullptr;
+    BCK(cudaStreamBeginCapture(b->s_tile, cudaStreamCaptureModeThreadLocal));
+    int rc = LBM_OK;
+    for (int k = 0; k < kChunk && rc == LBM_OK; ++k)
+        rc = strips ? launch_tiled_step(b, k, b->s_tile) : launch_tile_step(b, k, b->s_tile);
+    if (rc == LBM_OK)
+        lbmk::batch_clock_kernel<<<1, 32, 0, b->s_tile>>>(b->d_step, kChunk, b->d_order, (int)b->order.size());
+    cudaError_t e = cudaStreamEndCapture(b->s_tile, &g);
+    if (rc) {
+        if (g) cudaGraphDestroy(g);
+        return rc;
+    }
+    if (e != cudaSuccess) return bfail(e, "cudaStreamEndCapture(batch)");
+    e = cudaGraphInstantiate(out, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return bfail(e, "cudaGraphInstantiate(batch)");
+    return LBM_OK;
+}
+
 }  // namespace
 
 extern "C" const char* lbm_batch_last_error(void) { return g_batch_msg; }
@@ -479,8 +627,11 @@ extern "C" void lbm_batch_destroy(lbm_batch* b) {
     if (!b) return;
     cudaStreamSynchronize(b->s_res);
     cudaStreamSynchronize(b->s_tile);
-    if (b->chunk) cudaGraphExecDestroy(b->chunk);
+    for (cudaGraphExec_t g : b->chunk)
+        if (g) cudaGraphExecDestroy(g);
     if (b->d_items) cudaFree(b->d_items);
+    if (b->d_tiles) cudaFree(b->d_tiles);
+    if (b->d_order) cudaFree(b->d_order);
     if (b->pool) cudaFree(b->pool);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
     if (b->ev_join) cudaEventDestroy(b->ev_join);
@@ -626,6 +777,7 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     if ((e = cudaFuncSetAttribute(lbmk::pp_batch_pair<kBPWarps, kBPStages>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BPSmem))) != cudaSuccess)
         return fail(bfail(e, "cudaFuncSetAttribute(batch strip smem)"));
+    if ((rc = build_tiles(b))) return fail(rc);
     build_items(b, 32);
     if ((rc = upload_tables(b))) return fail(rc);
     if ((rc = batch_init_state(b))) return fail(rc);
@@ -641,27 +793,19 @@ extern "C" int lbm_batch_run(lbm_batch* b) {
         if (rc) return rc;
     }
     b->ran = true;
-    // tiled lattices: replays of a captured chunk of 64 single-step launches + step advance
-    if (!b->items.empty() && !b->chunk) {
-        cudaGraph_t g = nullptr;
-        BCK(cudaStreamBeginCapture(b->s_tile, cudaStreamCaptureModeThreadLocal));
-        int rc = LBM_OK;
-        for (int k = 0; k < kChunk && rc == LBM_OK; ++k) rc = launch_tiled_step(b, k, b->s_tile);
-        if (rc == LBM_OK) lbmk::advance_step<<<1, 1, 0, b->s_tile>>>(b->d_step, kChunk);
-        cudaError_t e = cudaStreamEndCapture(b->s_tile, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
-        }
-        if (e != cudaSuccess) return bfail(e, "cudaStreamEndCapture(batch)");
-        e = cudaGraphInstantiate(&b->chunk, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return bfail(e, "cudaGraphInstantiate(batch)");
-    }
     // resident lattices: one persistent launch, concurrent with the tiled replays
     int rc = launch_resident(b, -1, b->s_res);
     if (rc) return rc;
-    for (int s = 0; s < b->max_tiled_steps; s += kChunk) BCK(cudaGraphLaunch(b->chunk, b->s_tile));
+    // tiled lattices: replays of a captured chunk of single-step launches and a clock step; strips
+    // while the unfinished lattices hold enough cells for them, then tiles
+    for (int s = 0; s < b->max_tiled_steps; s += kChunk) {
+        long long cells = 0;
+        for (int i = 0; i < b->n; ++i)
+            if (!b->lat[i].resident && b->lat[i].nsteps > s) cells += (long long)b->lat[i].P.nx * b->lat[i].P.ny;
+        cudaGraphExec_t& g = b->chunk[cells >= kStripCells ? 0 : 1];
+        if (!g && (rc = capture_chunk(b, cells >= kStripCells, &g))) return rc;
+        BCK(cudaGraphLaunch(g, b->s_tile));
+    }
     BCK(cudaEventRecord(b->ev_join, b->s_res));
     BCK(cudaStreamWaitEvent(b->s_tile, b->ev_join, 0));
     return LBM_OK;

@@ -119,3 +119,32 @@ def test_strips_match_tiles(case, monkeypatch):
         assert float((a - b).abs().max()) <= 1e-6 * float(b.abs().max())
     else:
         assert torch.equal(fa, fb) and torch.equal(qa, qb)
+
+
+def test_batch_strips_and_tiles_match_single_lattices():
+    """A batch that starts above the batch's size rule (strips) and falls below it when the short lattices
+    finish (tiles), some in the middle of a 64-step graph, with lattices narrower than a tile, of several
+    tiles and of one: the same bits as single-lattice runs."""
+    from paper_2403_11167_gb300 import lbm
+
+    sizes = [(512, 512, 64), (512, 512, 70), (512, 512, 100), (512, 512, 130), (512, 512, 3), (512, 512, 64),
+             (512, 512, 61), (512, 512, 129), (512, 512, 1), (512, 512, 0), (60, 76, 140), (64, 130, 131),
+             (1200, 4, 66), (124, 37, 128), (8, 600, 65)]
+    assert sum(nx * ny for nx, ny, _ in sizes) > 2500000
+    specs, rhos = [], []
+    for k, (nx, ny, steps) in enumerate(sizes):
+        p = lbm.lbm_params_default(PP, precision=F32, a=0.25, Tr=0.8 + 0.005 * k, tau_nu=0.8, kappa_P=0.7, kappa_Li=-0.1)
+        _, th = lbm.lbm_resolve_params(p)
+        specs.append(dict(nx=nx, ny=ny, geometry=0, nsteps=steps, params=p))
+        rhos.append(inputs.spinodal_noise(nx, ny, 0.5 * (th.rho_l + th.rho_v), 0.01, seed=k))
+    b = lbm.Batch(specs, rhos)
+    assert b.info()["n_resident"] == 0
+    for _ in range(2):  # the second run starts again from the initial densities
+        b.run()
+        for i, (s, r) in enumerate(zip(specs, rhos)):
+            ctx = lbm.Context(s["params"], s["nx"], s["ny"])
+            ctx.set_density(r)
+            ctx.step(s["nsteps"])
+            assert np.array_equal(b.populations(i), ctx.populations()), (i, sizes[i])
+            ctx.close()
+    b.close()
