@@ -6,10 +6,9 @@
 // lattices of uneven sizes and step counts.  Run one at a time, the small ones are
 // launch-latency bound and the large ones leave most SMs idle.  Here they run together:
 //
-//   resident lattices  -- populations (9 N floats, the rest extensions N int16) + psi and
-//                         rho (2 N floats) fit in one CTA's shared
-//                         memory: one CTA per lattice runs every step of that lattice in
-//                         shared memory, in one persistent launch (no HBM traffic per step);
+//   resident lattices  -- those of at most 4452 cells: one CTA per lattice runs every step of
+//                         that lattice in shared memory and registers, in one persistent launch
+//                         per size class (no HBM traffic per step);
 //   tiled lattices     -- the rest: one launch per time step over a work table, replayed as
 //                         captured 64-step CUDA graphs on a second stream, concurrently with
 //                         the resident launch.  While the unfinished lattices hold many cells
@@ -17,7 +16,7 @@
 //                         TMA strip of the context path (pp_pair_strip), then one of tiles for
 //                         CTAs that each take a run of them (pp_batch_tile).
 //
-// An autotuner picks the resident block size and the strip height by timing short trials
+// An autotuner picks the resident cells per thread and the strip height by timing short trials
 // (cached per shape class for the process), and orders work longest-first.
 #include <cuda_runtime.h>
 
@@ -84,8 +83,8 @@ struct BatchItem {
 
 size_t a256(size_t n) { return (n + 255) & ~size_t(255); }
 
-// Shared memory of a resident lattice of N cells: 9 population planes, psi and rho (FP32), and
-// the int16 extensions of the rest population.
+// The size rule of resident lattices: 11 floats and an int16 per cell within kResidentSmemMax (the kernel
+// keeps 9 floats per cell in shared memory).
 size_t resident_bytes(size_t N) { return 11 * N * sizeof(float) + ((2 * N + 15) & ~size_t(15)); }
 
 // One population buffer of a lattice: 9 FP32 planes plus the int16 rest plane (plane 9).
@@ -96,66 +95,148 @@ size_t buffer_bytes(long long pitch) { return a256(10 * (size_t)pitch * 4); }
 namespace lbmk {
 
 // ------------------------------------------------------------------------------------
-// Resident lattice: all steps in shared memory.  Stored layout S_i(x) (post-collision at
-// the source cell, as in the tiled kernels).  Per step: (A) rho and psi of every cell into
-// shared arrays; barrier; (B) collision of every cell from the pulled populations and the
-// psi neighbours, f* written to the lattice's spare global buffer (L2-resident at these
-// sizes); barrier; (C) each thread copies its own cells' f* back into S; barrier.  Nothing
-// is held in registers across a barrier, so the block can be 1024 threads wide.
-__global__ void __launch_bounds__(1024, 1)
+// Resident lattice: all steps on one SM.  A thread keeps PAIRS pairs of cells for the whole run: their
+// rest populations and extensions stay in its registers, the eight moving populations in shared memory
+// in the stored layout S_i(x) (post-collision at the source cell).  Per step: (A) pull every cell's
+// populations into registers and write psi; barrier; (B) collide from the neighbours' psi and write f*
+// over S, which every thread has read by then; barrier.  So no population moves through global memory
+// and each step has two barriers.  A pair is two cells of one row when nx is even, so that reads of
+// unshifted columns and all writes are 8 bytes; otherwise the cells c and c + ceil(N/2).
+//
+// What bounds it: issue and the latency of the two phases at 16 warps per SM (128 registers a thread).
+// The earlier kernel (one cell at a time, f* through a global buffer, three barriers) took 11.4 us per
+// step for 64 x 64 cells on each of 152 SMs (54.8 GLUPS) and 12.5 us for 608 lattices of 256 x 4 (49.6);
+// this one 6.8 us (91.5) and 7.4 us (84.4).
+struct CellOff {  // steps to the wrapped neighbours of a cell, two 16-bit numbers each: columns, rows
+    int lr, mp;
+    __device__ __forceinline__ int dl() const { return (short)lr; }
+    __device__ __forceinline__ int dr() const { return lr >> 16; }
+    __device__ __forceinline__ int dm() const { return (short)mp; }
+    __device__ __forceinline__ int dp() const { return mp >> 16; }
+};
+// left of cell c and right of cell d of the same row
+__device__ __forceinline__ CellOff cell_off(int c, int d, int nx, int ny) {
+    const int x = c % nx, y = c / nx;
+    const int l = x == 0 ? nx - 1 : -1, r = d % nx == nx - 1 ? 1 - nx : 1;
+    const int m = y == 0 ? (ny - 1) * nx : -nx, p = y == ny - 1 ? -(ny - 1) * nx : nx;
+    return {(l & 0xffff) | r << 16, (m & 0xffff) | p << 16};
+}
+
+template <int PAIRS, int THREADS, bool EVEN>
+__global__ void __launch_bounds__(THREADS, 1)
     pp_resident_kernel(const BatchLattice* __restrict__ lats, const int* __restrict__ ids, int step_limit) {
     extern __shared__ __align__(16) float rsm[];
+    __shared__ StepParams<float> P;  // (read where they are used: registers are short)
     const BatchLattice& L = lats[ids[blockIdx.x]];
-    const StepParams<float> P = L.P;
-    const int nx = P.nx, ny = P.ny, N = nx * ny;
-    const long long pitch = P.pitch;
-    float* S = rsm;            // 9 planes of N
-    float* psi = rsm + 9 * N;  // N
-    float* rho = psi + N;      // N
-    short* Q = reinterpret_cast<short*>(rho + N);  // N: rest-population extensions
+    if (threadIdx.x < sizeof(P) / 4)
+        reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
+    const int nx = L.P.nx, ny = L.P.ny, N = nx * ny, H = (N + 1) / 2;
+    const int Ns = (N + 3) & ~3;  // plane stride
+    const long long pitch = L.P.pitch;
+    auto S = [&](int i) { return rsm + (i - 1) * Ns; };  // planes 1..8
+    float* psi = rsm + 8 * Ns;
     const float* g0 = L.buf[0];
-    float* G = L.buf[1];
-    for (int idx = threadIdx.x; idx < 9 * N; idx += blockDim.x) {
-        const int i = idx / N, c = idx - i * N;
-        S[idx] = g0[i * pitch + c];
+    for (int i = 1; i < 9; ++i)
+        for (int c = threadIdx.x; c < N; c += blockDim.x) S(i)[c] = g0[i * pitch + c];
+    // this thread's pairs (pair p: cells a(p), b(p); b may not exist when N is odd)
+    auto cell_a = [&](int p) { return EVEN ? 2 * p : p; };
+    auto cell_b = [&](int p) { return EVEN ? 2 * p + 1 : p + H; };
+    F2 v[PAIRS][9];
+    unsigned q[PAIRS];
+    CellOff oa[PAIRS], ob[EVEN ? 1 : PAIRS];
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) {
+        const int p = threadIdx.x + j * blockDim.x, a = cell_a(p), b = cell_b(p);
+        v[j][0] = F2::c(1.0f);
+        q[j] = 0;
+        if (p < H) {
+            const short* ql = rest_lo_plane(g0, pitch);
+            oa[j] = cell_off(a, EVEN ? b : a, nx, ny);
+            if (!EVEN) ob[EVEN ? 0 : j] = cell_off(b < N ? b : a, b < N ? b : a, nx, ny);
+            v[j][0] = F2(g0[a], g0[b < N ? b : a]);
+            q[j] = (unsigned)(unsigned short)ql[a] | (unsigned)(unsigned short)ql[b < N ? b : a] << 16;
+        }
     }
-    for (int c = threadIdx.x; c < N; c += blockDim.x) Q[c] = rest_lo_plane(g0, pitch)[c];
     __syncthreads();
+    // both cells' values of a plane, dx columns and dy rows away
+    auto at = [&](const float* f, int j, int p, int dx, int dy) {
+        const CellOff A = oa[j];
+        if constexpr (EVEN) {
+            const int c = 2 * p + (dy < 0 ? A.dm() : dy > 0 ? A.dp() : 0);
+            if (dx == 0) return F2(*reinterpret_cast<const float2*>(f + c));
+            if (dx < 0) return F2(f[c + A.dl()], f[c]);
+            return F2(f[c + 1], f[c + 1 + A.dr()]);
+        } else {
+            const CellOff B = ob[j];
+            const int a = p + (dx < 0 ? A.dl() : dx > 0 ? A.dr() : 0) + (dy < 0 ? A.dm() : dy > 0 ? A.dp() : 0);
+            const int b0 = p + H < N ? p + H : p;
+            const int b = b0 + (dx < 0 ? B.dl() : dx > 0 ? B.dr() : 0) + (dy < 0 ? B.dm() : dy > 0 ? B.dp() : 0);
+            return F2(f[a], f[b]);
+        }
+    };
+    auto put = [&](float* f, int p, F2 w) {
+        if constexpr (EVEN) {
+            *reinterpret_cast<float2*>(f + 2 * p) = w.v;
+        } else {
+            f[p] = w.v.x;
+            if (p + H < N) f[p + H] = w.v.y;
+        }
+    };
     const int nsteps = step_limit >= 0 ? min(step_limit, L.nsteps) : L.nsteps;
     for (int s = 0; s < nsteps; ++s) {
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            float v[9];
-            pull_cell_shared(S, N, c % nx, c / nx, nx, ny, v);
-            const float r = sum9(v);
-            rho[c] = r;
-            psi[c] = pseudo_psi(r, P);
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {
+            const int p = threadIdx.x + j * blockDim.x;
+            if (p >= H) continue;
+            F2* w = v[j];
+            w[1] = at(S(1), j, p, -1, 0);
+            w[2] = at(S(2), j, p, 0, -1);
+            w[3] = at(S(3), j, p, 1, 0);
+            w[4] = at(S(4), j, p, 0, 1);
+            w[5] = at(S(5), j, p, -1, -1);
+            w[6] = at(S(6), j, p, 1, -1);
+            w[7] = at(S(7), j, p, 1, 1);
+            w[8] = at(S(8), j, p, -1, 1);
+            put(psi, p, pseudo_psi_v(sum9_v(w), P));
         }
         __syncthreads();
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            const int x = c % nx, y = c / nx;
-            float v[9], pn[9];
-            pull_cell_shared(S, N, x, y, nx, ny, v);
-            gather8(psi, x, y, nx, ny, pn);
-            int q = Q[c];  // compensated rest population (only this thread touches Q[c])
-            pp_collide_comp(v, q, rho[c], pn[0], pn, P);
-            Q[c] = (short)q;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) G[i * pitch + c] = v[i];
-        }
-        __syncthreads();
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
+        for (int j = 0; j < PAIRS; ++j) {
+            const int p = threadIdx.x + j * blockDim.x;
+            if (p >= H) continue;
+            F2 pn[9], d0;
+            pn[0] = at(psi, j, p, 0, 0);
+            pn[1] = at(psi, j, p, 1, 0);
+            pn[2] = at(psi, j, p, 0, 1);
+            pn[3] = at(psi, j, p, -1, 0);
+            pn[4] = at(psi, j, p, 0, -1);
+            pn[5] = at(psi, j, p, 1, 1);
+            pn[6] = at(psi, j, p, -1, 1);
+            pn[7] = at(psi, j, p, -1, -1);
+            pn[8] = at(psi, j, p, 1, -1);
+            pp_collide_v<F2, true>(v[j], sum9_v(v[j]), pn[0], pn, P, &d0);
+            q[j] = rest_update_pair(v[j][0], q[j], d0, P);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) S[i * N + c] = G[i * pitch + c];
+            for (int i = 1; i < 9; ++i) put(S(i), p, v[j][i]);
         }
         __syncthreads();
     }
     // final state to the buffer the tiled convention uses after nsteps steps
     float* g = L.buf[nsteps & 1];
-    for (int idx = threadIdx.x; idx < 9 * N; idx += blockDim.x) {
-        const int i = idx / N, c = idx - i * N;
-        g[i * pitch + c] = S[idx];
+    short* ql = rest_lo_plane(g, pitch);
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) {
+        const int p = threadIdx.x + j * blockDim.x, a = cell_a(p), b = cell_b(p);
+        if (p >= H) continue;
+        g[a] = v[j][0].v.x;
+        ql[a] = (short)(q[j] & 0xffffu);
+        if (b < N) {
+            g[b] = v[j][0].v.y;
+            ql[b] = (short)(q[j] >> 16);
+        }
     }
-    for (int c = threadIdx.x; c < N; c += blockDim.x) rest_lo_plane(g, pitch)[c] = Q[c];
+    for (int i = 1; i < 9; ++i)
+        for (int c = threadIdx.x; c < N; c += blockDim.x) g[i * pitch + c] = S(i)[c];
 }
 
 // Tiled lattices, two cells per lane: one strip of one lattice per CTA, one step per launch.
@@ -359,30 +440,39 @@ __global__ void batch_obs_kernel(const BatchLattice* __restrict__ lats, double* 
 // --------------------------------------------------------------------------------------
 // Host side
 
+namespace {
+// Resident lattices that run as one launch on a stream of its own: CTAs of threads x pairs cells.
+struct ResidentGroup {
+    std::vector<int> ids;  // longest first
+    int max_cells;
+    bool even;             // even widths
+    int pairs, threads;    // chosen by the autotuner
+    int* d_ids;
+    cudaStream_t stream;
+    cudaEvent_t done;
+};
+}  // namespace
+
 struct lbm_batch {
     int n;
     std::vector<lbm_batch_lattice> spec;
     std::vector<BatchLattice> lat;       // host copy of the device table
-    std::vector<int> resident_ids;       // sorted longest-first
+    std::vector<ResidentGroup> groups;   // resident lattices by size and parity of the width
     std::vector<BatchItem> items;        // strips, sorted by lattice nsteps, longest first
     std::vector<BatchItem> tiles;        // tiles, in the same order of lattices
     std::vector<int2> order;             // tiled lattices in that order: steps, tiles
     int max_tiled_steps;
-    int resident_threads;
-    size_t resident_smem;
     int strip_rows;
     char* pool;
     BatchLattice* d_lat;
     BatchItem* d_items;
     BatchItem* d_tiles;
     int2* d_order;
-    int* d_ids;
     int* d_step;
     int* d_err;
     double* d_obs;
     std::vector<double> h_obs;
-    cudaStream_t s_res, s_tile;
-    cudaEvent_t ev_fork, ev_join;
+    cudaStream_t s_tile;
     cudaGraphExec_t chunk[2];            // kChunk steps with strips, with tiles
     bool ran;
     std::vector<std::vector<double>> rho0;  // kept for re-initialisation after autotuning trials
@@ -400,7 +490,7 @@ std::map<TuneKey, int> g_tune_cache;
 std::mutex g_tune_mu;
 
 int batch_init_state(lbm_batch* b) {
-    BCK(cudaStreamSynchronize(b->s_res));
+    for (const ResidentGroup& g : b->groups) BCK(cudaStreamSynchronize(g.stream));
     BCK(cudaStreamSynchronize(b->s_tile));
     for (int i = 0; i < b->n; ++i) {
         const BatchLattice& L = b->lat[i];
@@ -418,11 +508,53 @@ int batch_init_state(lbm_batch* b) {
     return LBM_OK;
 }
 
-int launch_resident(lbm_batch* b, int step_limit, cudaStream_t s) {
-    if (b->resident_ids.empty()) return LBM_OK;
-    const int nb = (int)b->resident_ids.size();
-    lbmk::pp_resident_kernel<<<nb, b->resident_threads, b->resident_smem, s>>>(b->d_lat, b->d_ids, step_limit);
+// The resident kernel's forms by pairs per thread; the widest block holds the largest resident lattice.
+using ResidentKernel = void (*)(const BatchLattice*, const int*, int);
+ResidentKernel resident_kernel(int pairs, bool even, int threads) {
+    if (pairs == 1) return even ? lbmk::pp_resident_kernel<1, 512, true> : lbmk::pp_resident_kernel<1, 512, false>;
+    if (pairs == 2) return even ? lbmk::pp_resident_kernel<2, 512, true> : lbmk::pp_resident_kernel<2, 512, false>;
+    if (threads <= 512)
+        return even ? lbmk::pp_resident_kernel<4, 512, true> : lbmk::pp_resident_kernel<4, 512, false>;
+    return even ? lbmk::pp_resident_kernel<4, 576, true> : lbmk::pp_resident_kernel<4, 576, false>;
+}
+// Threads of a CTA whose threads hold `pairs` pairs of a lattice of `cells` cells.
+int resident_threads(int cells, int pairs) { return ((cells + 1) / 2 + 32 * pairs - 1) / (32 * pairs) * 32; }
+
+int launch_resident(const lbm_batch* b, const ResidentGroup& g, int step_limit) {
+    const size_t smem = 9 * sizeof(float) * (size_t)((g.max_cells + 3) & ~3);
+    const ResidentKernel k = resident_kernel(g.pairs, g.even, g.threads);
+    BCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k<<<(unsigned)g.ids.size(), g.threads, smem, g.stream>>>(b->d_lat, g.d_ids, step_limit);
     BCK(cudaGetLastError());
+    return LBM_OK;
+}
+
+// Groups of the resident lattices: CTAs of one launch have the same shared memory and threads, so
+// lattices of up to 1152, 2304 and 4608 cells run as separate launches, and odd widths apart.
+int build_groups(lbm_batch* b) {
+    for (int cls = 0; cls < 6; ++cls) {
+        ResidentGroup g{};
+        g.even = cls % 2 == 0;
+        const int hi = 1152 << cls / 2, lo = cls < 2 ? 0 : hi / 2;
+        for (int i = 0; i < b->n; ++i) {
+            const int nx = b->lat[i].P.nx, cells = nx * b->lat[i].P.ny;
+            if (b->lat[i].resident && (nx % 2 == 0) == g.even && cells > lo && cells <= hi) {
+                g.ids.push_back(i);
+                g.max_cells = std::max(g.max_cells, cells);
+            }
+        }
+        if (g.ids.empty()) continue;
+        std::stable_sort(g.ids.begin(), g.ids.end(), [&](int x, int y) {
+            return (long long)b->lat[x].nsteps * b->lat[x].P.nx * b->lat[x].P.ny >
+                   (long long)b->lat[y].nsteps * b->lat[y].P.nx * b->lat[y].P.ny;
+        });
+        b->groups.push_back(g);  // (owned by the batch from here on, whatever fails below)
+        ResidentGroup& o = b->groups.back();
+        BCK(cudaStreamCreateWithFlags(&o.stream, cudaStreamNonBlocking));
+        BCK(cudaEventCreateWithFlags(&o.done, cudaEventDisableTiming));
+        BCK(cudaMalloc(&o.d_ids, sizeof(int) * o.ids.size()));
+        BCK(cudaMemcpy(o.d_ids, o.ids.data(), sizeof(int) * o.ids.size(), cudaMemcpyHostToDevice));
+    }
     return LBM_OK;
 }
 
@@ -511,37 +643,39 @@ double time_ms(cudaStream_t s, const std::function<int()>& fn, int* rc) {
     return ms;
 }
 
-// Autotuner: resident block size (cells per thread 1/2/4) and tiled strip height.  Each
+// Autotuner: pairs of cells per thread of each resident group and tiled strip height.  Each
 // candidate runs a short trial on the real initial state (restored afterwards); the choice is
 // cached per shape class for the lifetime of the process.
 int autotune(lbm_batch* b) {
-    int max_res_n = 0;
-    for (int id : b->resident_ids) max_res_n = std::max(max_res_n, b->lat[id].P.nx * b->lat[id].P.ny);
-    if (!b->resident_ids.empty()) {
-        const TuneKey key{0, max_res_n, (int)b->resident_ids.size()};
+    for (ResidentGroup& g : b->groups) {
+        const TuneKey key{g.even ? 0 : 2, g.max_cells, (int)g.ids.size()};
         int choice = -1;
         {
-            std::lock_guard<std::mutex> g(g_tune_mu);
+            std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune_cache.find(key);
             if (it != g_tune_cache.end()) choice = it->second;
         }
         if (choice < 0) {
             double best = 1e30;
-            for (int threads : {256, 512, 1024}) {
-                if (threads > 32 * ((max_res_n + 31) / 32) && threads > 256) continue;
-                b->resident_threads = threads;
-                int rc = LBM_OK;
-                const double ms = time_ms(b->s_res, [&] { return launch_resident(b, 16, b->s_res); }, &rc);
+            for (int pairs : {1, 2, 4}) {
+                const int threads = resident_threads(g.max_cells, pairs);
+                if (threads > (pairs == 4 ? 576 : 512)) continue;
+                g.pairs = pairs;
+                g.threads = threads;
+                int rc = launch_resident(b, g, 1);  // (loads the kernel)
+                if (rc) return rc;
+                const double ms = time_ms(g.stream, [&] { return launch_resident(b, g, 64); }, &rc);
                 if (rc) return rc;
                 if (ms < best) {
                     best = ms;
-                    choice = threads;
+                    choice = pairs;
                 }
             }
-            std::lock_guard<std::mutex> g(g_tune_mu);
+            std::lock_guard<std::mutex> lk(g_tune_mu);
             g_tune_cache[key] = choice;
         }
-        b->resident_threads = choice;
+        g.pairs = choice;
+        g.threads = resident_threads(g.max_cells, choice);
     }
     if (!b->items.empty() || b->max_tiled_steps > 0) {
         long long cells = 0;
@@ -625,7 +759,12 @@ extern "C" const char* lbm_batch_last_error(void) { return g_batch_msg; }
 
 extern "C" void lbm_batch_destroy(lbm_batch* b) {
     if (!b) return;
-    cudaStreamSynchronize(b->s_res);
+    for (ResidentGroup& g : b->groups) {
+        if (g.stream) cudaStreamSynchronize(g.stream);
+        if (g.d_ids) cudaFree(g.d_ids);
+        if (g.done) cudaEventDestroy(g.done);
+        if (g.stream) cudaStreamDestroy(g.stream);
+    }
     cudaStreamSynchronize(b->s_tile);
     for (cudaGraphExec_t g : b->chunk)
         if (g) cudaGraphExecDestroy(g);
@@ -633,9 +772,6 @@ extern "C" void lbm_batch_destroy(lbm_batch* b) {
     if (b->d_tiles) cudaFree(b->d_tiles);
     if (b->d_order) cudaFree(b->d_order);
     if (b->pool) cudaFree(b->pool);
-    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_join) cudaEventDestroy(b->ev_join);
-    if (b->s_res) cudaStreamDestroy(b->s_res);
     if (b->s_tile) cudaStreamDestroy(b->s_tile);
     delete b;
 }
@@ -727,32 +863,21 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         pool_bytes += 2 * buffer_bytes(P.pitch) + a256(2 * N * 4 + 8 * N);
     }
     const size_t tail = pool_bytes;
-    pool_bytes += a256(sizeof(BatchLattice) * n) + a256(sizeof(int) * n) + 256 + 256 + a256(8 * sizeof(double) * n);
+    pool_bytes += a256(sizeof(BatchLattice) * n) + 256 + 256 + a256(8 * sizeof(double) * n);
     cudaError_t e = cudaMalloc(&b->pool, pool_bytes);
     if (e != cudaSuccess) {
         delete b;
         return bfail(e, "cudaMalloc(batch pool)");
     }
-    size_t smax = 0;
     for (int i = 0; i < n; ++i) {
         BatchLattice& L = b->lat[i];
         const size_t fb = buffer_bytes(L.P.pitch);
         L.buf[0] = reinterpret_cast<float*>(b->pool + offs[i]);
         L.buf[1] = reinterpret_cast<float*>(b->pool + offs[i] + fb);
         L.scratch = reinterpret_cast<float*>(b->pool + offs[i] + 2 * fb);
-        if (L.resident) {
-            b->resident_ids.push_back(i);
-            smax = std::max(smax, resident_bytes((size_t)L.P.nx * L.P.ny));
-        }
     }
-    std::stable_sort(b->resident_ids.begin(), b->resident_ids.end(), [&](int x, int y) {
-        return (long long)b->lat[x].nsteps * b->lat[x].P.nx * b->lat[x].P.ny >
-               (long long)b->lat[y].nsteps * b->lat[y].P.nx * b->lat[y].P.ny;
-    });
-    b->resident_smem = smax;
     b->d_lat = reinterpret_cast<BatchLattice*>(b->pool + tail);
-    b->d_ids = reinterpret_cast<int*>(b->pool + tail + a256(sizeof(BatchLattice) * n));
-    b->d_step = reinterpret_cast<int*>(reinterpret_cast<char*>(b->d_ids) + a256(sizeof(int) * n));
+    b->d_step = reinterpret_cast<int*>(b->pool + tail + a256(sizeof(BatchLattice) * n));
     b->d_err = reinterpret_cast<int*>(reinterpret_cast<char*>(b->d_step) + 256);
     b->d_obs = reinterpret_cast<double*>(reinterpret_cast<char*>(b->d_err) + 256);
     b->h_obs.assign(8 * (size_t)n, 0.0);
@@ -761,19 +886,9 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         lbm_batch_destroy(b);
         return code;
     };
-    if ((e = cudaStreamCreateWithFlags(&b->s_res, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&b->s_tile, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming)) != cudaSuccess)
-        return fail(bfail(e, "stream/event create"));
-    if (!b->resident_ids.empty()) {
-        if ((e = cudaMemcpy(b->d_ids, b->resident_ids.data(), sizeof(int) * b->resident_ids.size(),
-                            cudaMemcpyHostToDevice)) != cudaSuccess)
-            return fail(bfail(e, "cudaMemcpy(ids)"));
-        if ((e = cudaFuncSetAttribute(lbmk::pp_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smax)) != cudaSuccess)
-            return fail(bfail(e, "cudaFuncSetAttribute(resident smem)"));
-    }
+    if ((e = cudaStreamCreateWithFlags(&b->s_tile, cudaStreamNonBlocking)) != cudaSuccess)
+        return fail(bfail(e, "cudaStreamCreate"));
+    if ((rc = build_groups(b))) return fail(rc);
     if ((e = cudaFuncSetAttribute(lbmk::pp_batch_pair<kBPWarps, kBPStages>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BPSmem))) != cudaSuccess)
         return fail(bfail(e, "cudaFuncSetAttribute(batch strip smem)"));
@@ -793,9 +908,10 @@ extern "C" int lbm_batch_run(lbm_batch* b) {
         if (rc) return rc;
     }
     b->ran = true;
-    // resident lattices: one persistent launch, concurrent with the tiled replays
-    int rc = launch_resident(b, -1, b->s_res);
-    if (rc) return rc;
+    // resident lattices: one persistent launch per group, concurrent with the tiled replays
+    int rc = LBM_OK;
+    for (const ResidentGroup& g : b->groups)
+        if ((rc = launch_resident(b, g, -1))) return rc;
     // tiled lattices: replays of a captured chunk of single-step launches and a clock step; strips
     // while the unfinished lattices hold enough cells for them, then tiles
     for (int s = 0; s < b->max_tiled_steps; s += kChunk) {
@@ -806,8 +922,10 @@ extern "C" int lbm_batch_run(lbm_batch* b) {
         if (!g && (rc = capture_chunk(b, cells >= kStripCells, &g))) return rc;
         BCK(cudaGraphLaunch(g, b->s_tile));
     }
-    BCK(cudaEventRecord(b->ev_join, b->s_res));
-    BCK(cudaStreamWaitEvent(b->s_tile, b->ev_join, 0));
+    for (const ResidentGroup& g : b->groups) {
+        BCK(cudaEventRecord(g.done, g.stream));
+        BCK(cudaStreamWaitEvent(b->s_tile, g.done, 0));
+    }
     return LBM_OK;
 }
 
@@ -840,8 +958,7 @@ extern "C" int lbm_batch_observables(lbm_batch* b, lbm_obs* out) {
 extern "C" int lbm_batch_populations(lbm_batch* b, int i, double* f) {
     if (!b || !f || i < 0 || i >= b->n) return LBM_ERR_ARG;
     if (!b->ran) return LBM_ERR_STATE;
-    BCK(cudaStreamSynchronize(b->s_tile));
-    BCK(cudaStreamSynchronize(b->s_res));
+    BCK(cudaStreamSynchronize(b->s_tile));  // (the resident groups have been joined to it)
     const BatchLattice& L = b->lat[i];
     const int nx = L.P.nx, ny = L.P.ny;
     const size_t n = (size_t)nx * ny;
@@ -866,9 +983,14 @@ extern "C" int lbm_batch_populations(lbm_batch* b, int i, double* f) {
 extern "C" int lbm_batch_info(const lbm_batch* b, int* n_resident, int* n_items, int* resident_threads,
                               int* strip_rows) {
     if (!b) return LBM_ERR_ARG;
-    if (n_resident) *n_resident = (int)b->resident_ids.size();
+    int resident = 0, threads = 0;
+    for (const ResidentGroup& g : b->groups) {
+        resident += (int)g.ids.size();
+        threads = g.threads;  // (of the largest lattices)
+    }
+    if (n_resident) *n_resident = resident;
     if (n_items) *n_items = (int)b->items.size();
-    if (resident_threads) *resident_threads = b->resident_threads;
+    if (resident_threads) *resident_threads = threads;
     if (strip_rows) *strip_rows = b->strip_rows;
     return LBM_OK;
 }

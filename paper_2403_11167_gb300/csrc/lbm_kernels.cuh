@@ -529,14 +529,6 @@ __device__ __forceinline__ void rest_update_v(F& hi, F& qf, F d, const StepParam
 __device__ __forceinline__ float rest_q_float(int q) { return (float)q; }
 __device__ __forceinline__ int rest_q_int(float qf) { return max(-32767, min(32767, __float2int_rn(qf))); }
 
-// Single cell: hi and its int16 q updated by the rest increment d.
-__device__ __forceinline__ void rest_update(float& hi, int& q, float d, const StepParams<float>& P) {
-    F1 h(hi), qf(rest_q_float(q));
-    rest_update_v(h, qf, F1(d), P);
-    hi = h.v;
-    q = rest_q_int(qf.v);
-}
-
 // Two cells of a lane (packed FP32): w holds both int16 extensions (first cell low half).
 __device__ __forceinline__ unsigned rest_update_pair(F2& hi, unsigned w, F2 d, const StepParams<float>& P) {
     F2 qf(rest_q_float((int)(short)(w & 0xffffu)), rest_q_float((int)w >> 16));
@@ -569,21 +561,6 @@ __device__ __forceinline__ float sum9_rest(const float v[9], int q, const StepPa
 __device__ __forceinline__ float pseudo_psi(float rho, const StepParams<float>& P) {
     return pseudo_psi_v(F1(rho), P).v;
 }
-// The collision with a compensated rest population (v[0] and q updated together).
-__device__ __forceinline__ void pp_collide_comp(float v[9], int& q, float rho, float pc, const float pn[9],
-                                                const StepParams<float>& P) {
-    F1 vv[9], n[9], d0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        vv[i] = F1(v[i]);
-        n[i] = F1(pn[i]);
-    }
-    pp_collide_v<F1, true>(vv, F1(rho), F1(pc), n, P, &d0);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) v[i] = vv[i].v;
-    rest_update(v[0], q, d0.v, P);
-}
-
 __device__ __forceinline__ float fe_mu(float rc, const float rn[9], const StepParams<float>& P) {
     // rn[0] is not used and callers need not set it
     F1 r[9];
@@ -602,23 +579,6 @@ __device__ __forceinline__ long long shifted_cell(int x, int y, int cx, int cy, 
     xs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
     ys = ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys);
     return (long long)ys * nx + xs;
-}
-
-// Pulled populations of cell (x, y) from populations in shared memory (plain loads; the
-// read-only global path of pull9 must not be given a shared-memory address).
-template <typename real>
-__device__ __forceinline__ void pull_cell_shared(const real* S, int N, int x, int y, int nx, int ny, real v[9]) {
-    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    const int om = (y == 0 ? ny - 1 : y - 1) * nx, o0 = y * nx, op = (y == ny - 1 ? 0 : y + 1) * nx;
-    v[0] = S[0 * N + o0 + x];
-    v[1] = S[1 * N + o0 + xm];
-    v[2] = S[2 * N + om + x];
-    v[3] = S[3 * N + o0 + xp];
-    v[4] = S[4 * N + op + x];
-    v[5] = S[5 * N + om + xm];
-    v[6] = S[6 * N + om + xp];
-    v[7] = S[7 * N + op + xp];
-    v[8] = S[8 * N + op + xm];
 }
 
 // Pulled populations of cell (x, y) from global memory: v_i = S_i(x - c_i) = f_i(x).

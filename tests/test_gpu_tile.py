@@ -148,3 +148,32 @@ def test_batch_strips_and_tiles_match_single_lattices():
             assert np.array_equal(b.populations(i), ctx.populations()), (i, sizes[i])
             ctx.close()
     b.close()
+
+
+@pytest.mark.parametrize("sizes", [
+    [(1, 1), (1, 6), (5, 1), (3, 3), (31, 33), (101, 1)],                # odd widths, odd cell counts, one cell
+    [(2, 1), (2, 3), (64, 4), (256, 4), (32, 32), (8, 141)],             # up to one pair per thread of 512
+    [(43, 45), (1, 2047), (47, 49)], [(512, 4), (2, 1025), (40, 52)],    # the middle class, odd and even
+    [(63, 65), (1, 4452), (61, 72)], [(64, 64), (4, 1113), (4452, 1)]])  # the largest, odd and even
+def test_resident_lattices_match_single_lattices(sizes):
+    """Resident lattices of every size class and parity of width, uneven step counts (0 and 1 among them):
+    the same bits as single-lattice runs."""
+    from paper_2403_11167_gb300 import lbm
+
+    specs, rhos = [], []
+    for k, (nx, ny) in enumerate(sizes):
+        p = lbm.lbm_params_default(PP, precision=F32, a=0.25, Tr=0.8 + 0.01 * k, tau_nu=0.8, kappa_P=0.7, kappa_Li=-0.1,
+                                   body_fx=1e-5)
+        _, th = lbm.lbm_resolve_params(p)
+        specs.append(dict(nx=nx, ny=ny, geometry=0, nsteps=(40, 0, 1, 33)[k % 4], params=p))
+        rhos.append(inputs.spinodal_noise(nx, ny, 0.5 * (th.rho_l + th.rho_v), 0.01, seed=k))
+    b = lbm.Batch(specs, rhos)
+    assert b.info()["n_resident"] == len(sizes)
+    b.run()
+    for i, (s, r) in enumerate(zip(specs, rhos)):
+        ctx = lbm.Context(s["params"], s["nx"], s["ny"])
+        ctx.set_density(r)
+        ctx.step(s["nsteps"])
+        assert np.array_equal(b.populations(i), ctx.populations()), sizes[i]
+        ctx.close()
+    b.close()
