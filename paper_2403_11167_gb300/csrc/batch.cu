@@ -69,7 +69,8 @@ constexpr size_t kResidentSmemMax = 200 * 1024;
 struct BatchLattice {
     lbmk::StepParams<float> P;  // physics and geometry (nx, ny, rows, pitch)
     float* buf[2];              // ping-pong stored populations
-    float* scratch;             // 2 N floats: rho and psi for observables / density staging
+    float* scratch;             // 2 N floats: rho and psi for observables
+    double* rho0;               // N initial densities
     double RT, a, b4;           // FP64 EOS constants for the observables (pressure jump)
     int nsteps;
     int geometry;
@@ -340,26 +341,52 @@ __global__ void batch_clock_kernel(int* state, int by, const int2* __restrict__ 
     }
 }
 
-// Observables of every lattice (one CTA per lattice): rho and psi of the final state into
-// the lattice scratch, then u (Eq. 6b with the Shan-Chen force), mass, u_max, probes,
-// tangent width, pressure jump and equimolar radius -- the definitions of lbm_observables.
-__global__ void batch_obs_kernel(const BatchLattice* __restrict__ lats, double* __restrict__ out) {
-    const BatchLattice& L = lats[blockIdx.x];
+// Cells of every lattice in runs of kRunCells, one CTA each (lat, first cell): the kernels off the step
+// path work on these, so that a 512 x 512 lattice does not wait for one CTA (observables of the 96-lattice
+// sweep: 1.25 ms with a CTA per lattice, 0.33 with these).
+constexpr int kRunCells = 2048;
+
+// f = f^eq(rho0, u = 0) of every lattice from its initial densities on the device.
+__global__ void __launch_bounds__(256)
+    batch_init_kernel(const BatchLattice* __restrict__ lats, const int2* __restrict__ runs) {
+    const int2 run = runs[blockIdx.x];
+    const BatchLattice& L = lats[run.x];
+    const int nx = L.P.nx, ny = L.P.ny, end = min(run.y + kRunCells, nx * ny);
+    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x)
+        init_cell(L.rho0, L.buf[0], LBM_PSEUDOPOTENTIAL, nx, ny, L.P.pitch, L.P.rest_inv, c);
+}
+
+// Observables, the definitions of lbm_observables, in three launches: rho and psi of the final state into
+// the lattice scratch; per run the sums and maxima of u (Eq. 6b with the Shan-Chen force), mass and probes;
+// per lattice their total in run order, tangent width, pressure jump and equimolar radius.
+__global__ void __launch_bounds__(256)
+    batch_fields_kernel(const BatchLattice* __restrict__ lats, const int2* __restrict__ runs) {
+    const int2 run = runs[blockIdx.x];
+    const BatchLattice& L = lats[run.x];
     const StepParams<float> P = L.P;
-    const int nx = P.nx, ny = P.ny, N = nx * ny;
+    const int nx = P.nx, ny = P.ny, N = nx * ny, end = min(run.y + kRunCells, N);
     const float* f = L.buf[L.nsteps & 1];
-    float* rho = L.scratch;
-    float* ps = L.scratch + N;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
+    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x) {
         float v[9];
         pull_cell(f, P.pitch, c % nx, c / nx, nx, ny, v);
         const float r = sum9_rest(v, rest_lo_plane(f, P.pitch)[c], P);
-        rho[c] = r;
-        ps[c] = pseudo_psi(r, P);
+        L.scratch[c] = r;
+        L.scratch[N + c] = pseudo_psi(r, P);
     }
-    __syncthreads();
+}
+
+constexpr int kRunSums = 6;  // mass, liquid and vapour probes, bad cells; max u^2, max slope
+__global__ void __launch_bounds__(256)
+    batch_sums_kernel(const BatchLattice* __restrict__ lats, const int2* __restrict__ runs, double* __restrict__ sums) {
+    const int2 run = runs[blockIdx.x];
+    const BatchLattice& L = lats[run.x];
+    const StepParams<float> P = L.P;
+    const int nx = P.nx, ny = P.ny, N = nx * ny, end = min(run.y + kRunCells, N);
+    const float* f = L.buf[L.nsteps & 1];
+    const float* rho = L.scratch;
+    const float* ps = L.scratch + N;
     double m = 0.0, u2 = 0.0, bad = 0.0, liq = 0.0, vap = 0.0, dmax = 0.0;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
+    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x) {
         const int x = c % nx, y = c / nx;
         float v[9], an[9];
         pull_cell(f, P.pitch, x, y, nx, ny, v);
@@ -390,7 +417,7 @@ __global__ void batch_obs_kernel(const BatchLattice* __restrict__ lats, double* 
             dmax = fmax(dmax, fabs(a - b) * 0.5);
         }
     }
-    __shared__ double red[6][32];
+    __shared__ double red[kRunSums][8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
         m += __shfl_down_sync(0xffffffffu, m, o);
@@ -409,14 +436,32 @@ __global__ void batch_obs_kernel(const BatchLattice* __restrict__ lats, double* 
         red[5][wid] = dmax;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        double s[6] = {0, 0, 0, 0, 0, 0};
-        for (int w = 0; w < nw; ++w) {
-            for (int j = 0; j < 4; ++j) s[j] += red[j][w];
-            s[4] = fmax(s[4], red[4][w]);
-            s[5] = fmax(s[5], red[5][w]);
+    if (threadIdx.x < kRunSums) {
+        double t = red[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w)
+            t = threadIdx.x < 4 ? t + red[threadIdx.x][w] : fmax(t, red[threadIdx.x][w]);
+        sums[kRunSums * (size_t)blockIdx.x + threadIdx.x] = t;
+    }
+}
+
+// first[i], first[i + 1]: the runs of lattice i (one warp per lattice).
+__global__ void __launch_bounds__(32)
+    batch_obs_kernel(const BatchLattice* __restrict__ lats, const int* __restrict__ first,
+                     const double* __restrict__ sums, double* __restrict__ out) {
+    const BatchLattice& L = lats[blockIdx.x];
+    const int nx = L.P.nx, ny = L.P.ny, N = nx * ny, lane = threadIdx.x;
+    double s[kRunSums] = {0, 0, 0, 0, 0, 0};
+    for (int r = first[blockIdx.x] + lane; r < first[blockIdx.x + 1]; r += 32)
+        for (int j = 0; j < kRunSums; ++j) {
+            const double t = sums[kRunSums * (size_t)r + j];
+            s[j] = j < 4 ? s[j] + t : fmax(s[j], t);
         }
+    for (int o = 16; o > 0; o >>= 1)
+        for (int j = 0; j < kRunSums; ++j) {
+            const double t = __shfl_xor_sync(0xffffffffu, s[j], o);
+            s[j] = j < 4 ? s[j] + t : fmax(s[j], t);
+        }
+    if (lane == 0) {
         const double nl = L.geometry == 0 ? 2.0 * ny : 16.0, nv = L.geometry == 0 ? 2.0 * ny : 64.0;
         const double rl = s[1] / nl, rv = s[2] / nv;
         auto pcs = [&](double r) {
@@ -475,7 +520,11 @@ struct lbm_batch {
     cudaStream_t s_tile;
     cudaGraphExec_t chunk[2];            // kChunk steps with strips, with tiles
     bool ran;
-    std::vector<std::vector<double>> rho0;  // kept for re-initialisation after autotuning trials
+    std::vector<int2> runs;                 // cells in runs of kRunCells: lattice, first cell
+    int2* d_runs;
+    int* d_first;                           // each lattice's first run (n + 1)
+    double* d_sums;                         // kRunSums per run
+    cudaEvent_t ready;                      // the initial state is there (for the resident groups)
 };
 
 namespace {
@@ -489,22 +538,33 @@ struct TuneKey {
 std::map<TuneKey, int> g_tune_cache;
 std::mutex g_tune_mu;
 
+// f^eq(rho0) for every lattice and the clock at 0, enqueued behind whatever ran before.
 int batch_init_state(lbm_batch* b) {
-    for (const ResidentGroup& g : b->groups) BCK(cudaStreamSynchronize(g.stream));
-    BCK(cudaStreamSynchronize(b->s_tile));
-    for (int i = 0; i < b->n; ++i) {
-        const BatchLattice& L = b->lat[i];
-        const size_t n = (size_t)L.P.nx * L.P.ny;
-        BCK(cudaMemcpyAsync(L.scratch, b->rho0[i].data(), n * sizeof(double), cudaMemcpyHostToDevice, b->s_tile));
-        lbmk::init_kernel<float, double><<<std::min<long long>(304, (n + 255) / 256), 256, 0, b->s_tile>>>(
-            reinterpret_cast<const double*>(L.scratch), L.buf[0], LBM_PSEUDOPOTENTIAL, L.P.nx, L.P.ny, L.P.pitch,
-            L.P.rest_inv);
-    }
-    BCK(cudaGetLastError());
-    if (b->d_order) lbmk::batch_clock_kernel<<<1, 32, 0, b->s_tile>>>(b->d_step, -1, b->d_order, (int)b->order.size());
-    BCK(cudaGetLastError());
     BCK(cudaMemsetAsync(b->d_err, 0, sizeof(int) * 16, b->s_tile));
-    BCK(cudaStreamSynchronize(b->s_tile));
+    if (b->d_order) lbmk::batch_clock_kernel<<<1, 32, 0, b->s_tile>>>(b->d_step, -1, b->d_order, (int)b->order.size());
+    lbmk::batch_init_kernel<<<(unsigned)b->runs.size(), 256, 0, b->s_tile>>>(b->d_lat, b->d_runs);
+    BCK(cudaGetLastError());
+    BCK(cudaEventRecord(b->ready, b->s_tile));
+    for (const ResidentGroup& g : b->groups) BCK(cudaStreamWaitEvent(g.stream, b->ready, 0));
+    return LBM_OK;
+}
+
+// The runs of all lattices and their initial densities, to the device.
+int upload_state(lbm_batch* b, const double* const* rho0) {
+    std::vector<int> first;
+    for (int i = 0; i < b->n; ++i) {
+        const int cells = b->lat[i].P.nx * b->lat[i].P.ny;
+        first.push_back((int)b->runs.size());
+        for (int c = 0; c < cells; c += lbmk::kRunCells) b->runs.push_back(make_int2(i, c));
+        BCK(cudaMemcpyAsync(b->lat[i].rho0, rho0[i], sizeof(double) * (size_t)cells, cudaMemcpyHostToDevice, b->s_tile));
+    }
+    first.push_back((int)b->runs.size());
+    BCK(cudaMalloc(&b->d_runs, sizeof(int2) * b->runs.size()));
+    BCK(cudaMalloc(&b->d_first, sizeof(int) * first.size()));
+    BCK(cudaMalloc(&b->d_sums, sizeof(double) * lbmk::kRunSums * b->runs.size()));
+    BCK(cudaMemcpyAsync(b->d_runs, b->runs.data(), sizeof(int2) * b->runs.size(), cudaMemcpyHostToDevice, b->s_tile));
+    BCK(cudaMemcpyAsync(b->d_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice, b->s_tile));
+    BCK(cudaStreamSynchronize(b->s_tile));  // the caller's arrays have been read
     return LBM_OK;
 }
 
@@ -553,7 +613,7 @@ int build_groups(lbm_batch* b) {
         BCK(cudaStreamCreateWithFlags(&o.stream, cudaStreamNonBlocking));
         BCK(cudaEventCreateWithFlags(&o.done, cudaEventDisableTiming));
         BCK(cudaMalloc(&o.d_ids, sizeof(int) * o.ids.size()));
-        BCK(cudaMemcpy(o.d_ids, o.ids.data(), sizeof(int) * o.ids.size(), cudaMemcpyHostToDevice));
+        BCK(cudaMemcpyAsync(o.d_ids, o.ids.data(), sizeof(int) * o.ids.size(), cudaMemcpyHostToDevice, b->s_tile));
     }
     return LBM_OK;
 }
@@ -591,9 +651,9 @@ int build_tiles(lbm_batch* b) {
     }
     const size_t tb = sizeof(BatchItem) * b->tiles.size(), ob = sizeof(int2) * b->order.size();
     BCK(cudaMalloc(&b->d_tiles, tb));
-    BCK(cudaMemcpy(b->d_tiles, b->tiles.data(), tb, cudaMemcpyHostToDevice));
+    BCK(cudaMemcpyAsync(b->d_tiles, b->tiles.data(), tb, cudaMemcpyHostToDevice, b->s_tile));
     BCK(cudaMalloc(&b->d_order, ob));
-    BCK(cudaMemcpy(b->d_order, b->order.data(), ob, cudaMemcpyHostToDevice));
+    BCK(cudaMemcpyAsync(b->d_order, b->order.data(), ob, cudaMemcpyHostToDevice, b->s_tile));
     return LBM_OK;
 }
 
@@ -620,10 +680,11 @@ void build_items(lbm_batch* b, int rows) {
 int upload_tables(lbm_batch* b) {
     if (b->d_items) cudaFree(b->d_items);
     b->d_items = nullptr;
-    BCK(cudaMemcpy(b->d_lat, b->lat.data(), sizeof(BatchLattice) * b->n, cudaMemcpyHostToDevice));
+    BCK(cudaMemcpyAsync(b->d_lat, b->lat.data(), sizeof(BatchLattice) * b->n, cudaMemcpyHostToDevice, b->s_tile));
     if (!b->items.empty()) {
         BCK(cudaMalloc(&b->d_items, sizeof(BatchItem) * b->items.size()));
-        BCK(cudaMemcpy(b->d_items, b->items.data(), sizeof(BatchItem) * b->items.size(), cudaMemcpyHostToDevice));
+        BCK(cudaMemcpyAsync(b->d_items, b->items.data(), sizeof(BatchItem) * b->items.size(), cudaMemcpyHostToDevice,
+                            b->s_tile));
     }
     return LBM_OK;
 }
@@ -770,6 +831,10 @@ extern "C" void lbm_batch_destroy(lbm_batch* b) {
         if (g) cudaGraphExecDestroy(g);
     if (b->d_items) cudaFree(b->d_items);
     if (b->d_tiles) cudaFree(b->d_tiles);
+    if (b->d_runs) cudaFree(b->d_runs);
+    if (b->d_first) cudaFree(b->d_first);
+    if (b->d_sums) cudaFree(b->d_sums);
+    if (b->ready) cudaEventDestroy(b->ready);
     if (b->d_order) cudaFree(b->d_order);
     if (b->pool) cudaFree(b->pool);
     if (b->s_tile) cudaStreamDestroy(b->s_tile);
@@ -785,7 +850,6 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     b->n = n;
     b->spec.assign(specs, specs + n);
     b->lat.resize(n);
-    b->rho0.resize(n);
     // resolve parameters and validate on the host first
     size_t pool_bytes = 0;
     std::vector<size_t> offs(n);
@@ -819,7 +883,6 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
                 delete b;
                 return LBM_ERR_ARG;
             }
-        b->rho0[i].assign(rho0[i], rho0[i] + N);
         BatchLattice& L = b->lat[i];
         std::memset(&L, 0, sizeof(L));
         lbmk::StepParams<float>& P = L.P;
@@ -875,6 +938,7 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         L.buf[0] = reinterpret_cast<float*>(b->pool + offs[i]);
         L.buf[1] = reinterpret_cast<float*>(b->pool + offs[i] + fb);
         L.scratch = reinterpret_cast<float*>(b->pool + offs[i] + 2 * fb);
+        L.rho0 = reinterpret_cast<double*>(L.scratch + 2 * (size_t)L.P.nx * L.P.ny);
     }
     b->d_lat = reinterpret_cast<BatchLattice*>(b->pool + tail);
     b->d_step = reinterpret_cast<int*>(b->pool + tail + a256(sizeof(BatchLattice) * n));
@@ -886,8 +950,9 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         lbm_batch_destroy(b);
         return code;
     };
-    if ((e = cudaStreamCreateWithFlags(&b->s_tile, cudaStreamNonBlocking)) != cudaSuccess)
-        return fail(bfail(e, "cudaStreamCreate"));
+    if ((e = cudaStreamCreateWithFlags(&b->s_tile, cudaStreamNonBlocking)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&b->ready, cudaEventDisableTiming)) != cudaSuccess)
+        return fail(bfail(e, "stream/event create"));
     if ((rc = build_groups(b))) return fail(rc);
     if ((e = cudaFuncSetAttribute(lbmk::pp_batch_pair<kBPWarps, kBPStages>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BPSmem))) != cudaSuccess)
@@ -895,6 +960,7 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     if ((rc = build_tiles(b))) return fail(rc);
     build_items(b, 32);
     if ((rc = upload_tables(b))) return fail(rc);
+    if ((rc = upload_state(b, rho0))) return fail(rc);
     if ((rc = batch_init_state(b))) return fail(rc);
     if ((rc = autotune(b))) return fail(rc);
     *out = b;
@@ -932,7 +998,10 @@ extern "C" int lbm_batch_run(lbm_batch* b) {
 extern "C" int lbm_batch_observables(lbm_batch* b, lbm_obs* out) {
     if (!b || !out) return LBM_ERR_ARG;
     if (!b->ran) return LBM_ERR_STATE;
-    lbmk::batch_obs_kernel<<<b->n, 1024, 0, b->s_tile>>>(b->d_lat, b->d_obs);
+    const unsigned runs = (unsigned)b->runs.size();
+    lbmk::batch_fields_kernel<<<runs, 256, 0, b->s_tile>>>(b->d_lat, b->d_runs);
+    lbmk::batch_sums_kernel<<<runs, 256, 0, b->s_tile>>>(b->d_lat, b->d_runs, b->d_sums);
+    lbmk::batch_obs_kernel<<<b->n, 32, 0, b->s_tile>>>(b->d_lat, b->d_first, b->d_sums, b->d_obs);
     BCK(cudaGetLastError());
     BCK(cudaMemcpyAsync(b->h_obs.data(), b->d_obs, sizeof(double) * 8 * b->n, cudaMemcpyDeviceToHost, b->s_tile));
     int herr = 0;

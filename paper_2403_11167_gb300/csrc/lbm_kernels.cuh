@@ -592,31 +592,35 @@ __device__ __forceinline__ void pull_cell(const real* __restrict__ S, long long 
 }
 
 // f = f^eq(rho0, u = 0): Eq. (4) (weights w_i rho) or Eq. (20) (f_0 = rho, others 0),
-// stored as S_i(y) = f^eq_i(rho0(y + c_i)).
+// stored as S_i(y) = f^eq_i(rho0(y + c_i)).  One cell c.
+template <typename real, typename src_t>
+__device__ __forceinline__ void init_cell(const src_t* __restrict__ rho0, real* __restrict__ S, int model, int nx, int ny,
+                                          long long pitch, float rest_inv, long long c) {
+    const int cxs[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+    const int cys[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    const int x = (int)(c % nx), y = (int)(c / nx);
+    if (model == 0) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const real w = i == 0 ? real(4.0 / 9.0) : (i < 5 ? real(1.0 / 9.0) : real(1.0 / 36.0));
+            S[i * pitch + c] = w * (real)rho0[shifted_cell(x, y, cxs[i], cys[i], nx, ny)];
+        }
+        if constexpr (std::is_same<real, float>::value)  // the rest population to ~40 bits
+            rest_lo_plane(S, pitch)[c] = rest_encode(4.0 / 9.0 * (double)rho0[c], S[c], rest_inv);
+    } else {
+        S[c] = (real)rho0[c];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) S[i * pitch + c] = real(0);
+        if constexpr (std::is_same<real, float>::value)
+            rest_lo_plane(S, pitch)[c] = rest_encode((double)rho0[c], S[c], rest_inv);
+    }
+}
 template <typename real, typename src_t>
 __global__ void init_kernel(const src_t* __restrict__ rho0, real* __restrict__ S, int model, int nx, int ny,
                             long long pitch, float rest_inv) {
-    const int cxs[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
-    const int cys[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     const long long n = (long long)nx * ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % nx), y = (int)(c / nx);
-        if (model == 0) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const real w = i == 0 ? real(4.0 / 9.0) : (i < 5 ? real(1.0 / 9.0) : real(1.0 / 36.0));
-                S[i * pitch + c] = w * (real)rho0[shifted_cell(x, y, cxs[i], cys[i], nx, ny)];
-            }
-            if constexpr (std::is_same<real, float>::value)  // the rest population to ~40 bits
-                rest_lo_plane(S, pitch)[c] = rest_encode(4.0 / 9.0 * (double)rho0[c], S[c], rest_inv);
-        } else {
-            S[c] = (real)rho0[c];
-#pragma unroll
-            for (int i = 1; i < 9; ++i) S[i * pitch + c] = real(0);
-            if constexpr (std::is_same<real, float>::value)
-                rest_lo_plane(S, pitch)[c] = rest_encode((double)rho0[c], S[c], rest_inv);
-        }
-    }
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
+        init_cell(rho0, S, model, nx, ny, pitch, rest_inv, c);
 }
 
 // ---------------------------------------------------------------------------------
