@@ -417,7 +417,7 @@ static int choose_tile_rows(int prec, int model, int nx, int ny) {
     static const int ops[3][4] = {{28, 0, 0, 125}, {8, 45, 0, 120}, {8, 45, 40, 140}};
     int best = 1;
     long long least = -1;
-    for (int r = 1; r <= lbmk::kTileRows; ++r) {
+    for (int r = 1; r <= lbmk::Tile<double, 0>::kRows; ++r) {
         long long t = 0;
         for (int p = 0; p < 4; ++p) {  // phase p works on the rows of the tile and of the halo it needs
             const int halo = p == 3 ? 0 : model + 1 - p;

@@ -2,7 +2,7 @@
 // lattices whose width is not a multiple of 4 or that are too small for strips, no-slip walls, the
 // droplet-collision drive and the full free-energy model.
 //
-// A CTA updates a tile of at most kTileRows rows and one warp's columns.  Each warp holds one row
+// A CTA updates a tile of a few rows and one warp's columns.  Each warp holds one row
 // of the tile or of its halo; a lane holds two adjacent cells in FP32 (packed, F2) or one in FP64.
 // A warp pulls its row's populations once and keeps them in registers; the neighbour fields (psi;
 // rho and mu; rho, mu and u) go through shared memory between rows and through shuffles within a
@@ -32,11 +32,11 @@
 
 namespace lbmk {
 
-constexpr int kTileRows = 8;  // most rows of a tile
-
 // Lane layout of a tile row: V the cells of a lane, kPer of them; HC halo columns on each side of
-// the (at most) kCols columns a warp updates.  MODEL: 0 pseudopotential, 1 free energy, 2 full
-// free energy; LV is its number of halo rows.
+// the (at most) kCols columns a warp updates; kRows the most rows of a tile.  MODEL: 0 pseudopotential, 1
+// free energy, 2 full free energy; LV is its number of halo rows.  kCtas: CTAs per SM that the registers
+// have to allow (56 and 64 registers in FP32; with one CTA less a 2048^2 step, which streams from HBM,
+// took 73.6 us instead of 66.6 and 99.0 instead of 85.4).
 template <typename real, int MODEL>
 struct Tile {
     using V = typename std::conditional<std::is_same<real, float>::value, F2, double>::type;
@@ -44,7 +44,9 @@ struct Tile {
     static constexpr int LV = MODEL + 1;
     static constexpr int HC = kPer == 1 ? LV : (MODEL == 2 ? 4 : 2);
     static constexpr int kCols = 32 * kPer - 2 * HC;
-    static constexpr int kThreads = 32 * (kTileRows + 2 * LV);
+    static constexpr int kRows = kPer == 2 && MODEL < 2 ? 4 : 8;
+    static constexpr int kThreads = 32 * (kRows + 2 * LV);
+    static constexpr int kCtas = kPer == 1 ? 1 : MODEL == 0 ? 6 : MODEL == 1 ? 4 : 2;
 };
 
 // The stored mass of driven steps.  FP64: one slot per tile row, summed by every CTA of the next
@@ -163,6 +165,27 @@ __device__ __forceinline__ void pull_tile(const double* __restrict__ f, long lon
     pull9(f, pitch, xa, xl, xr, om, o0, op, v);
 }
 
+// The same for a buffer of less than 4 GB and even nx, by 32-bit byte offsets from its start: o0, om, op of
+// column xa in rows y, y-1, y+1, l and r of the neighbours left and right of the pair (-4 and 8 away from the
+// edges), pb the plane pitch.  One integer addition per plane instead of 64-bit address arithmetic per load.
+__device__ __forceinline__ void pull_tile32(const float* __restrict__ f, unsigned pb, unsigned o0, unsigned om,
+                                            unsigned op, int l, int r, F2 v[9]) {
+    const char* b = reinterpret_cast<const char*>(f);
+    auto one = [&](unsigned o) { return __ldg(reinterpret_cast<const float*>(b + o)); };
+    auto pair = [&](unsigned o) { return F2(__ldg(reinterpret_cast<const float2*>(b + o))); };
+    const unsigned a1 = o0 + pb, a3 = o0 + 3 * pb, a5 = om + 5 * pb, a6 = om + 6 * pb, a7 = op + 7 * pb,
+                   a8 = op + 8 * pb;
+    v[0] = pair(o0);
+    v[2] = pair(om + 2 * pb);
+    v[4] = pair(op + 4 * pb);
+    v[1] = F2(one(a1 + l), one(a1));
+    v[5] = F2(one(a5 + l), one(a5));
+    v[8] = F2(one(a8 + l), one(a8));
+    v[3] = F2(one(a3 + 4), one(a3 + r));
+    v[6] = F2(one(a6 + 4), one(a6 + r));
+    v[7] = F2(one(a7 + 4), one(a7 + r));
+}
+
 // Zou-He completion of a wall row's cells (wall_fill of step_ext.cuh).
 template <class V>
 __device__ __forceinline__ void tile_wall_fill(V v[9], bool top, V Jx, V Jy) {
@@ -191,13 +214,14 @@ __device__ __forceinline__ V tile_grad_y_onesided(const V n[9], bool top) {
     return -fmav(a, n[4] - n[0], d * ((n[8] - n[1]) + (n[7] - n[3])));
 }
 
-template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN>
-__global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
+// EVEN: FP32 with even nx (cells of a lane 8-byte aligned); NEAR: and a buffer of less than 4 GB.
+template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN, bool NEAR>
+__global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>::kCtas)
     tile_step(const real* __restrict__ fin, real* __restrict__ fout, const StepParams<real> P,
               const TileArgs<real> T) {
     using L = Tile<real, MODEL>;
     using V = typename L::V;
-    constexpr int LV = L::LV, HC = L::HC, KP = L::kPer, RMAX = kTileRows + 2 * LV;
+    constexpr int LV = L::LV, HC = L::HC, KP = L::kPer, RMAX = L::kRows + 2 * LV;
     __shared__ V s_a[RMAX][32];                        // psi or rho
     __shared__ V s_mu[MODEL > 0 ? RMAX : 1][32];       // mu
     __shared__ V s_u[MODEL > 1 ? 2 * RMAX : 1][32];    // u_x, then u_y
@@ -213,7 +237,7 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
     const int x0 = blockIdx.x * T.wb;
     const int w = min(T.wb, nx - x0);  // > 0 (the host's grid)
     const int y = y0 - LV + warp;      // this warp's row (rows beyond the lattice mirrored or wrapped)
-    const int yr = WALLS ? mirror_row(y, ny) : wrap_idx(y, ny);
+    const int yr = WALLS ? mirror_row(y, ny) : ny >= 16 ? wrap_once(y, ny) : wrap_idx(y, ny);
     const bool wall = WALLS && (y == 0 || y == ny - 1);      // a wall row of the lattice or its image
     const bool wall_img = WALLS && (yr == 0 || yr == ny - 1);
     const bool top = WALLS && yr != 0;
@@ -221,7 +245,9 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
     const bool out_row = warp >= LV && y < y1;
     const bool out_a = out_row && c >= 0 && c < w;
     const bool out_b = KP == 2 && out_row && c >= 0 && c + 1 < w;
-    const long long oc = (long long)y * nx + x0 + c;  // (out rows and lanes only)
+    // the lane's place in a plane (out rows and lanes only), and with NEAR in bytes in the rest plane
+    const long long oc = NEAR ? 0 : (long long)y * nx + x0 + c;
+    const unsigned oc32 = NEAR ? (unsigned)(y * nx + x0 + c) * 4u : 0u, qo = (unsigned)P.pitch * 36u + oc32 / 2;
 
     // the state's mean density: every CTA sums in the same order
     if constexpr (DRIVE) {
@@ -248,21 +274,36 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
     [[maybe_unused]] unsigned qw = 0;              // FP32: the cells' int16 rest extensions
     if (y < y1 + LV && c < w + HC) {
         int xl = x0 + c - 1, xa = x0 + c, xb = x0 + c + 1, xr = x0 + c + KP;
-        auto wrap = [nx](int x) {
-            while (x < 0) x += nx;
-            while (x >= nx) x -= nx;
-            return x;
-        };
-        xl = wrap(xl);
-        xa = wrap(xa);
-        xb = wrap(xb);
-        xr = wrap(xr);
-        const long long o0 = (long long)yr * nx, om = yr == 0 ? (long long)(ny - 1) * nx : o0 - nx,
-                        op = yr == ny - 1 ? 0 : o0 + nx;
-        pull_tile<EVEN>(fin, P.pitch, xl, xa, xb, xr, om, o0, op, v);
+        const bool edge = x0 < HC + 1 || x0 + w + HC >= nx;  // (of the tile) some column wraps
+        if (edge) {
+            auto wrap = [nx](int x) {
+                while (x < 0) x += nx;
+                while (x >= nx) x -= nx;
+                return x;
+            };
+            xl = wrap(xl);
+            xa = wrap(xa);
+            xb = wrap(xb);
+            xr = wrap(xr);
+        }
+        if constexpr (NEAR) {
+            const unsigned row = 4u * nx, o0 = yr * row + 4u * xa;
+            const unsigned om = yr == 0 ? o0 + (ny - 1) * row : o0 - row, op = yr == ny - 1 ? o0 - yr * row : o0 + row;
+            const unsigned pb = (unsigned)P.pitch * 4u;
+            if (edge)
+                pull_tile32(fin, pb, o0, om, op, 4 * (xl - xa), 4 * (xr - xa), v);
+            else
+                pull_tile32(fin, pb, o0, om, op, -4, 8, v);
+        } else {
+            const long long o0 = (long long)yr * nx, om = yr == 0 ? (long long)(ny - 1) * nx : o0 - nx,
+                            op = yr == ny - 1 ? 0 : o0 + nx;
+            pull_tile<EVEN>(fin, P.pitch, xl, xa, xb, xr, om, o0, op, v);
+        }
         if constexpr (std::is_same<real, float>::value) {
             const short* q = rest_lo_plane(fin, P.pitch);
-            if constexpr (EVEN) {
+            if constexpr (NEAR) {
+                if (out_a) qw = __ldg(reinterpret_cast<const unsigned*>(reinterpret_cast<const char*>(fin) + qo));
+            } else if constexpr (EVEN) {
                 if (out_a) qw = __ldg(reinterpret_cast<const unsigned*>(q + oc));
             } else {
                 if (out_a) qw = (unsigned)(unsigned short)__ldg(q + oc);
@@ -407,6 +448,14 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads)
         if (out_a)
 #pragma unroll
             for (int i = 0; i < 9; ++i) fout[i * P.pitch + oc] = v[i];
+    } else if constexpr (NEAR) {
+        if (out_a) {
+            char* b = reinterpret_cast<char*>(fout);
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                *reinterpret_cast<float2*>(b + (oc32 + (unsigned)P.pitch * 4u * i)) = v[i].v;
+            *reinterpret_cast<unsigned*>(b + qo) = qw;
+        }
     } else if constexpr (EVEN) {
         if (out_a) {
 #pragma unroll

@@ -10,11 +10,13 @@ cudaError_t launch(const real* fin, real* fout, const StepParams<real>& P, const
     const int gy = WALLS && T.band > 0 ? 2 : (P.ny + rows - 1) / rows, gz = (gy + 65534) / 65535;
     const dim3 grid((P.nx + T.wb - 1) / T.wb, (gy + gz - 1) / gz, gz);
     const int threads = 32 * (rows + 2 * Tile<real, MODEL>::LV);
-    if (std::is_same<real, double>::value || P.nx % 2 == 0)
-        tile_step<real, MODEL, WALLS, DRIVE, true><<<grid, threads, 0, s>>>(fin, fout, P, T);
+    constexpr bool f32 = std::is_same<real, float>::value;
+    if (!f32 || P.nx % 2 != 0)
+        tile_step<real, MODEL, WALLS, DRIVE, false, false><<<grid, threads, 0, s>>>(fin, fout, P, T);
+    else if (P.pitch * 40 >= (1LL << 32))
+        tile_step<real, MODEL, WALLS, DRIVE, f32, false><<<grid, threads, 0, s>>>(fin, fout, P, T);
     else
-        tile_step<real, MODEL, WALLS, DRIVE, std::is_same<real, double>::value>
-            <<<grid, threads, 0, s>>>(fin, fout, P, T);
+        tile_step<real, MODEL, WALLS, DRIVE, f32, f32><<<grid, threads, 0, s>>>(fin, fout, P, T);
     return cudaGetLastError();
 }
 
