@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     extern __shared__ __align__(16) float rsm[];
     __shared__ StepParams<float> P;  // (read where they are used: registers are short)
     const BatchLattice& L = lats[ids[blockIdx.x]];
-    if (threadIdx.x < sizeof(P) / 4)
-        reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
+    for (int i = threadIdx.x; i < (int)sizeof(P) / 4; i += blockDim.x)  // (a CTA may be one warp)
+        reinterpret_cast<int*>(&P)[i] = reinterpret_cast<const int*>(&L.P)[i];
     const int nx = L.P.nx, ny = L.P.ny, N = nx * ny, H = (N + 1) / 2;
     const int Ns = (N + 3) & ~3;  // plane stride
     const long long pitch = L.P.pitch;
@@ -255,6 +255,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 4)
     // in shared memory, not in registers: 94 of them allow four CTAs per SM, 110 three (a sweep of 3.9
     // million cells: 25.6 ms against 29.1)
     __shared__ StepParams<float> P;
+    static_assert(sizeof(P) / 4 <= (NW + 1) * 32, "one word per thread");
     if (threadIdx.x < sizeof(P) / 4)
         reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
     __syncthreads();
@@ -290,6 +291,7 @@ __global__ void __launch_bounds__(32 * (kBatchTileRows + 2))
             fin = L.buf[step & 1];
             fout = L.buf[(step + 1) & 1];
             __syncthreads();  // every warp is done with the previous lattice's constants
+            static_assert(sizeof(P) / 4 <= 32 * (R + 2), "one word per thread");
             if (threadIdx.x < sizeof(P) / 4)
                 reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
             __syncthreads();
