@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 // Tiled lattices, two cells per lane: one strip of one lattice per CTA, one step per launch.
-template <int NW, int S>
+template <int NW, int S, bool NEAR>
 __global__ void __launch_bounds__((NW + 1) * 32, 4)
     pp_batch_pair(const BatchLattice* __restrict__ lats, const BatchItem* __restrict__ items,
                   const int* __restrict__ state, int k, int* __restrict__ err) {
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 4)
     if (threadIdx.x < sizeof(P) / 4)
         reinterpret_cast<int*>(&P)[threadIdx.x] = reinterpret_cast<const int*>(&L.P)[threadIdx.x];
     __syncthreads();
-    pp_pair_strip<NW, S>(L.buf[step & 1], L.buf[(step + 1) & 1], P, it.x0, it.w, it.y0, it.y1, sm, err);
+    pp_pair_strip<NW, S, false, NEAR>(L.buf[step & 1], L.buf[(step + 1) & 1], P, it.x0, it.w, it.y0, it.y1, sm, err);
 }
 
 // The same lattices in tiles of kBatchTileRows rows, one row per warp (step_tile.cuh): CTA b takes its
@@ -627,10 +627,18 @@ int launch_tile_step(lbm_batch* b, int k, cudaStream_t s) {
     return LBM_OK;
 }
 
+// The strip kernel that addresses every lattice of the batch.
+decltype(&lbmk::pp_batch_pair<kBPWarps, kBPStages, true>) strip_kernel(const lbm_batch* b) {
+    for (const auto& l : b->lat)
+        if (!lbmk::near_buffer(l.P.pitch)) return lbmk::pp_batch_pair<kBPWarps, kBPStages, false>;
+    return lbmk::pp_batch_pair<kBPWarps, kBPStages, true>;
+}
+
 int launch_tiled_step(lbm_batch* b, int k, cudaStream_t s) {
     if (b->items.empty()) return LBM_OK;
-    lbmk::pp_batch_pair<kBPWarps, kBPStages><<<(unsigned)b->items.size(), (kBPWarps + 1) * 32, sizeof(BPSmem), s>>>(
-        b->d_lat, b->d_items, b->d_step, k, b->d_err);
+    const auto kernel = strip_kernel(b);
+    kernel<<<(unsigned)b->items.size(), (kBPWarps + 1) * 32, sizeof(BPSmem), s>>>(b->d_lat, b->d_items, b->d_step, k,
+                                                                                  b->d_err);
     BCK(cudaGetLastError());
     return LBM_OK;
 }
@@ -956,8 +964,8 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         (e = cudaEventCreateWithFlags(&b->ready, cudaEventDisableTiming)) != cudaSuccess)
         return fail(bfail(e, "stream/event create"));
     if ((rc = build_groups(b))) return fail(rc);
-    if ((e = cudaFuncSetAttribute(lbmk::pp_batch_pair<kBPWarps, kBPStages>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BPSmem))) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(strip_kernel(b), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(BPSmem))) != cudaSuccess)
         return fail(bfail(e, "cudaFuncSetAttribute(batch strip smem)"));
     if ((rc = build_tiles(b))) return fail(rc);
     build_items(b, 32);

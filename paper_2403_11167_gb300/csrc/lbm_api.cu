@@ -72,6 +72,20 @@ constexpr int kIWBStages = 8;
 using IWBSmem = lbmk::IwbStripSmem<kIWBWarps, kIWBStages>;
 constexpr int kFEPTX = FEPSmem::TX;            // widest strip (240 columns)
 
+// Dynamic shared memory of every strip kernel.
+template <bool NEAR>
+cudaError_t strip_attributes() {
+    const auto max_smem = [](auto* kernel, size_t bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    cudaError_t e = max_smem(lbmk::pp_step_pair<kPPPWarps, kPPPStages, false, NEAR>, sizeof(PPPSmem));
+    if (e == cudaSuccess) e = max_smem(lbmk::pp_step_pair<kPPPWarps, kPPPStages, true, NEAR>, sizeof(PPPSmem));
+    if (e == cudaSuccess) e = max_smem(lbmk::fe_step_pair<kFEPWarps, kFEPStages, false, NEAR>, sizeof(FEPSmem));
+    if (e == cudaSuccess) e = max_smem(lbmk::fe_step_pair<kFEPWarps, kFEPStages, true, NEAR>, sizeof(FEPSmem));
+    if (e == cudaSuccess) e = max_smem(lbmk::fe_iwb_pair<kIWBWarps, kIWBStages, NEAR>, sizeof(IWBSmem));
+    return e;
+}
+
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
 }  // namespace
@@ -404,7 +418,7 @@ static void fill_step_params(lbmk::StepParams<real>& s, const lbm_ctx* c) {
 // the populations or psi, mu, u, collision).  It picks the fastest of the measured heights 1..8 on
 // 256 x 4 (6.2 us with 1), 101 x 50 (8.6 us with 2), 200 x 100 (12.8 us with 6), 256 x 128 (12.7
 // and 20.9 us with 8 and 3) and 400 x 300 (41 and 56 us with 4 and 8).
-// FP32: 4 rows (1022 x 770: 13.7 us against 15.8 with 2 and 14.2 with 8), the full model with its
+// FP32: 4 rows (1022 x 770: 12.2 us, where 13.7 compared with 15.8 with 2 rows and 14.2 with 8), the full model with its
 // three halo rows 8 (1024^2: 29 us against 40 with 4), fewer while that leaves SMs without a tile.
 static int choose_tile_rows(int prec, int model, int nx, int ny) {
     const int wb = prec == LBM_F64 ? lbmk::tile_columns<double>(model, nx) : lbmk::tile_columns<float>(model, nx);
@@ -540,22 +554,10 @@ extern "C" int lbm_create(const lbm_params* p, int nx, int ny, int bc_x, int bc_
     fill_step_params(c->spd, c);
     if (c->use_tma) {
         // the stage rings exceed the default 48 KB of dynamic shared memory
-        cudaError_t e1 = cudaFuncSetAttribute(lbmk::fe_step_pair<kFEPWarps, kFEPStages>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FEPSmem));
-        cudaError_t e2 = cudaFuncSetAttribute(lbmk::pp_step_pair<kPPPWarps, kPPPStages>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PPPSmem));
-        if (e1 == cudaSuccess)  // the driven instantiations (Sec. 5.4 drive)
-            e1 = cudaFuncSetAttribute(lbmk::fe_step_pair<kFEPWarps, kFEPStages, true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FEPSmem));
-        if (e2 == cudaSuccess)
-            e2 = cudaFuncSetAttribute(lbmk::pp_step_pair<kPPPWarps, kPPPStages, true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PPPSmem));
-        if (e1 == cudaSuccess)  // the full free-energy model's strip kernel
-            e1 = cudaFuncSetAttribute(lbmk::fe_iwb_pair<kIWBWarps, kIWBStages>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(IWBSmem));
-        if (e1 != cudaSuccess || e2 != cudaSuccess) {
+        const cudaError_t e = lbmk::near_buffer(c->spf.pitch) ? strip_attributes<true>() : strip_attributes<false>();
+        if (e != cudaSuccess) {
             lbm_destroy(c);
-            return cuda_fail(e1 != cudaSuccess ? e1 : e2, "cudaFuncSetAttribute(max dynamic smem)");
+            return cuda_fail(e, "cudaFuncSetAttribute(max dynamic smem)");
         }
     }
     *out = c;
@@ -711,20 +713,54 @@ static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int ban
 // Whether a step runs the strip kernels: FP32 lattices of TMA-copyable rows, and for the full
 // free-energy model neither walls nor the drive nor a reference density; above the size where the
 // strips' streaming beats the tiles' short chains (us per step, tile and strip):
-//   pseudopotential        1792^2  51.9, 59.0   2048^2  67.9, 69.9   2560^2 102.9, 98.5
-//   free energy            1536^2  50.8, 52.8   1792^2  67.2, 63.0   2048^2  87.9, 81.8
-//   full free energy       1536^2  66.4, 67.0   1792^2  87.7, 80.1
-//   walls (P; FE)          1536^2  44.0, 51.1; 57.2, 56.0   2048^2  76.0, 72.8; 99.2, 85.0
-//   drive (P; FE)          1024^2  20.9, 30.9; 29.9, 35.1   1536^2  47.6, 52.1; 66.5, 56.9
-//                          2048^2  82.4, 74.5; 115.5, 86.0
+//   pseudopotential        2048^2  66.8, 66.6   2176^2  75.0, 77.3   2560^2 100.9, 95.0
+//   free energy            1600^2  53.4, 56.2   1664^2  57.7, 56.9   1792^2  65.5, 60.9
+//   full free energy       1600^2  69.3, 74.4   1792^2  84.0, 78.4
+//   walls (P)              2176^2  75.8, 80.5   2304^2  84.4, 83.0
+//   walls (FE)             1664^2  57.8, 59.9   1792^2  66.0, 64.0
+//   drive (P)              1536^2  49.9, 50.8   1600^2  53.9, 51.6
+//   drive (FE)             1664^2  59.1, 61.3   1792^2  67.3, 65.2
 static bool strip_step(const lbm_ctx* c, bool driven) {
     if (!c->use_tma) return false;
     const long long cells = (long long)c->nx * c->ny;
     if (uses_iwb(c)) return cells >= 2800000 && !c->walls && !driven && (!c->grav || c->rho_g == 0.0);
     const bool pp = c->prm.model == LBM_PSEUDOPOTENTIAL;
-    if (driven) return cells >= (pp ? 3000000 : 1500000);
-    if (c->walls) return cells >= (pp ? 3400000 : 2100000);
-    return cells >= (pp ? 4500000 : 2800000);
+    if (driven) return cells >= (pp ? 2500000 : 3100000);
+    if (c->walls) return cells >= (pp ? 5200000 : 3100000);
+    return cells >= (pp ? 4800000 : 2800000);
+}
+
+// The strip kernels of one step (the walls' rows excepted).
+template <bool NEAR>
+static int launch_strips(lbm_ctx* c, int src, bool driven, int chain) {
+    const float* fin = static_cast<const float*>(c->f[src]);
+    float* fout = static_cast<float*>(c->f[src ^ 1]);
+    const int m = model_index(c);
+    const int tx = m == 0 ? kPPPTX : m == 1 ? kFEPTX : IWBSmem::TX;
+    const dim3 grid((c->nx + tx - 1) / tx, (c->ny + c->rows - 1) / c->rows);
+    if (m == 2) {
+        lbmk::fe_iwb_pair<kIWBWarps, kIWBStages, NEAR>
+            <<<grid, (kIWBWarps + 1) * 32, sizeof(IWBSmem), c->stream>>>(fin, fout, c->spf, ext_terms<float>(c), c->d_err);
+    } else if (driven) {
+        // the state's mass: what the previous driven strip step stored, by warp, or a reduction
+        const lbmk::Drive<float> d =
+            chain > 0 ? sum_drive<float>(c, c->dmass, (int)(grid.x * grid.y) * (m == 0 ? kPPPWarps : kFEPWarps))
+                    : launch_drive<float>(c, src);
+        if (m == 0)
+            lbmk::pp_step_pair<kPPPWarps, kPPPStages, true, NEAR>
+                <<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(fin, fout, c->spf, c->d_err, d, c->dmass);
+        else
+            lbmk::fe_step_pair<kFEPWarps, kFEPStages, true, NEAR>
+                <<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(fin, fout, c->spf, c->d_err, d, c->dmass);
+    } else if (m == 0) {
+        lbmk::pp_step_pair<kPPPWarps, kPPPStages, false, NEAR>
+            <<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
+    } else {
+        lbmk::fe_step_pair<kFEPWarps, kFEPStages, false, NEAR>
+            <<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
+    }
+    CK(cudaGetLastError());
+    return LBM_OK;
 }
 
 // chain: how many driven steps of the same sequence precede this one on the stream (a graph replays
@@ -733,36 +769,12 @@ static int launch_step(lbm_ctx* c, int src, bool driven = false, int chain = 0) 
     if (!strip_step(c, driven))
         return c->prec == LBM_F32 ? launch_tile_step<float>(c, src, driven, chain, 0, c->spf)
                                   : launch_tile_step<double>(c, src, driven, chain, 0, c->spd);
-    const float* fin = static_cast<const float*>(c->f[src]);
-    float* fout = static_cast<float*>(c->f[src ^ 1]);
-    const int m = model_index(c);
-    const int tx = m == 0 ? kPPPTX : m == 1 ? kFEPTX : IWBSmem::TX;
-    const dim3 grid((c->nx + tx - 1) / tx, (c->ny + c->rows - 1) / c->rows);
-    if (m == 2) {
-        lbmk::fe_iwb_pair<kIWBWarps, kIWBStages>
-            <<<grid, (kIWBWarps + 1) * 32, sizeof(IWBSmem), c->stream>>>(fin, fout, c->spf, ext_terms<float>(c), c->d_err);
-    } else if (driven) {
-        // the state's mass: what the previous driven strip step stored, by warp, or a reduction
-        const lbmk::Drive<float> d =
-            chain > 0 ? sum_drive<float>(c, c->dmass, (int)(grid.x * grid.y) * (m == 0 ? kPPPWarps : kFEPWarps))
-                    : launch_drive<float>(c, src);
-        if (m == 0)
-            lbmk::pp_step_pair<kPPPWarps, kPPPStages, true><<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(
-                fin, fout, c->spf, c->d_err, d, c->dmass);
-        else
-            lbmk::fe_step_pair<kFEPWarps, kFEPStages, true><<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(
-                fin, fout, c->spf, c->d_err, d, c->dmass);
-    } else if (m == 0) {
-        lbmk::pp_step_pair<kPPPWarps, kPPPStages>
-            <<<grid, (kPPPWarps + 1) * 32, sizeof(PPPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
-    } else {
-        lbmk::fe_step_pair<kFEPWarps, kFEPStages>
-            <<<grid, (kFEPWarps + 1) * 32, sizeof(FEPSmem), c->stream>>>(fin, fout, c->spf, c->d_err);
-    }
-    CK(cudaGetLastError());
+    const bool near = lbmk::near_buffer(c->spf.pitch);
+    int rc = near ? launch_strips<true>(c, src, driven, chain) : launch_strips<false>(c, src, driven, chain);
     // walls: the periodic step is right except on the rows next to them
-    if (c->walls) return launch_tile_step<float>(c, src, false, 0, m == 0 ? kWallBandPP : kWallBandFE, c->spf);
-    return LBM_OK;
+    if (rc == LBM_OK && c->walls)
+        rc = launch_tile_step<float>(c, src, false, 0, model_index(c) == 0 ? kWallBandPP : kWallBandFE, c->spf);
+    return rc;
 }
 
 static int build_graph(lbm_ctx* c, int parity, int driven) {

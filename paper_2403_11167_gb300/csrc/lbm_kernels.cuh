@@ -536,6 +536,10 @@ __device__ __forceinline__ unsigned rest_update_pair(F2& hi, unsigned w, F2 d, c
     return ((unsigned)rest_q_int(qf.v.x) & 0xffffu) | ((unsigned)rest_q_int(qf.v.y) << 16);
 }
 
+// Whether an FP32 buffer (nine planes and the int16 one, 38 bytes per cell) is addressed by 32-bit byte
+// offsets.
+__host__ __device__ inline bool near_buffer(long long pitch) { return pitch * 40 < (1LL << 32); }
+
 // The rest-population plane of an FP32 buffer (plane 9, int16).
 __device__ __forceinline__ short* rest_lo_plane(float* f, long long pitch) {
     return reinterpret_cast<short*>(f + 9 * pitch);

@@ -175,11 +175,11 @@ struct WarpStripSmem {
     float stage[S][9 * W8];
     uint64_t full[S];
     uint64_t empty[S];
-    // rest-population extensions (two int16 per lane) of the last three pulled rows, each lane
+    // rest-population extensions (two int16 per lane) of the last four pulled rows, each lane
     // its own word: copied asynchronously when a row is pulled and read by the same lane when
     // that row is collided one (pseudopotential) or two (free energy) rows later, so that no
     // register waits on the global load in between
-    uint32_t qext[3][NW][32];
+    uint32_t qext[4][NW][32];
 };
 
 // Strip geometry shared by the host and the kernels: nx is split into gx strips of equal
@@ -188,6 +188,49 @@ struct WarpStripSmem {
 __host__ __device__ __forceinline__ int warp_strip_width(int nx, int gx) {
     return ((nx + gx - 1) / gx + 3) & ~3;
 }
+
+// A consumer's place in the ring: the stage of the newest row and the parity of its phase, advanced row
+// by row (an index modulo S costs five instructions, and a row needs ten of them).
+template <int S>
+struct RingPos {
+    int s;
+    uint32_t parity;
+    __device__ __forceinline__ void next() {
+        s = s == S - 1 ? 0 : s + 1;
+        parity ^= s == 0 ? 1u : 0u;
+    }
+};
+
+// The cells of a strip kernel's output row.  NEAR: buffers of less than 4 GB, by 32-bit byte offsets (one
+// addition per plane); otherwise by pointers.
+template <bool NEAR>
+struct StripOut {
+    float* f;
+    unsigned* q;        // the rest plane
+    long long pitch, c; // the pair's first cell
+    unsigned pb, o;     // NEAR: plane pitch and o = 4 c in bytes
+    __device__ __forceinline__ StripOut(float* fout, long long pitch_, long long cell)
+        : f(fout), q(reinterpret_cast<unsigned*>(rest_lo_plane(fout, pitch_))), pitch(pitch_), c(cell),
+          pb((unsigned)pitch_ * 4u), o((unsigned)cell * 4u) {}
+    __device__ __forceinline__ void next_row(int nx) {
+        if constexpr (NEAR)
+            o += 4u * nx;
+        else
+            c += nx;
+    }
+    __device__ __forceinline__ void store(const F2 v[9], unsigned qw) const {
+        if constexpr (NEAR) {
+            char* b = reinterpret_cast<char*>(f);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(b + (o + i * pb)) = v[i].v;
+            *reinterpret_cast<unsigned*>(b + (9 * pb + o / 2)) = qw;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(f + c + i * pitch) = v[i].v;
+            q[c >> 1] = qw;
+        }
+    }
+};
 
 // Producer side of the ring, run by one thread: issue the first S rows, then refill each
 // stage once all NW consumer warps have released it.  Returns false on timeout.

@@ -15,6 +15,9 @@
 // The tile kernel (step_tile.cuh) serves smaller lattices, FP64, walls, the drive and gravity with a
 // non-zero reference density, in FP32 with this arithmetic and to the same bits.
 //
+// Bounded by instruction issue at 128 registers (334 us per step at 4096^2; 344 before the stores went by
+// 32-bit offsets).  With eight stages the ring indexes are masks; held as pointers they spill (585 us).
+//
 // Requirements (checked on the host): nx % 4 == 0, nx >= 8, ny >= 4; every wait bounded.
 #pragma once
 #include <cuda_runtime.h>
@@ -176,7 +179,7 @@ __device__ __forceinline__ bool iwb_ring_produce(const float* __restrict__ fin, 
 }
 
 // E.rho_g must be 0 (checked on the host): the buoyancy is -rho g and p_g vanishes.
-template <int NW, int S>
+template <int NW, int S, bool NEAR = true>
 __global__ void __launch_bounds__((NW + 1) * 32, 3) fe_iwb_pair(const float* __restrict__ fin,
                                                                 float* __restrict__ fout, const StepParams<float> P,
                                                                 const Ext<float> E, int* __restrict__ err) {
@@ -232,8 +235,10 @@ __global__ void __launch_bounds__((NW + 1) * 32, 3) fe_iwb_pair(const float* __r
     m2.c = m3.c = m4.c = m2.xm = m3.xm = m4.xm = m2.xp = m3.xp = m4.xp = F2::c(0.0f);
     ux3.c = ux4.c = uy3.c = uy4.c = ux3.xm = ux4.xm = uy3.xm = uy4.xm = F2::c(0.0f);
     ux3.xp = ux4.xp = uy3.xp = uy4.xp = F2::c(0.0f);
-    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch));
-    unsigned* qout = reinterpret_cast<unsigned*>(rest_lo_plane(fout, P.pitch));
+    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch)) +
+                          (((long long)y0 * nx + x0 + col) >> 1);
+    uint32_t* const qslot = &sm.qext[0][warp][lane];
+    StripOut<NEAR> O(fout, P.pitch, (long long)y0 * nx + x0 + col);
     const F2 fx = F2::c(P.fx);
     // y force: body force plus the buoyancy -rho g (reference density 0)
     auto fy_of = [&](F2 rho) { return fmav(F2::c(-E.g), rho, F2::c(P.fy)); };
@@ -243,8 +248,10 @@ __global__ void __launch_bounds__((NW + 1) * 32, 3) fe_iwb_pair(const float* __r
         const int k = q + 1 - rbase;  // ring index of row q+1
         ok = mbar_wait_bounded(&sm.full[k % S], (uint32_t)((k / S) & 1));
         if (!ok) break;
-        if (out && q >= y0 && q < y1)
-            cp_async4(&sm.qext[(q - y0 + 4) & 3][warp][lane], qin + (((long long)q * nx + x0 + col) >> 1));
+        if (out && q >= y0 && q < y1) {
+            cp_async4(qslot + ((q - y0) & 3) * (NW * 32), qin);
+            qin += nx >> 1;
+        }
         cp_async_commit();
         // pull row q, rho(q)
         F2 rho0 = F2::c(1.0f);
@@ -293,13 +300,10 @@ __global__ void __launch_bounds__((NW + 1) * 32, 3) fe_iwb_pair(const float* __r
             F2 d0;
             fe_collide_iwb_v<F2, true>(v, r3.c, mn, rn, st, fx, fy_of(r3.c), F2::c(0.0f), 0.0f, E.A, P, &d0);
             cp_async_wait<3>();  // the copy of row q-3's extensions (three groups ago) has landed
-            const unsigned ql3 = sm.qext[(q - 3 - y0 + 4) & 3][warp][lane];
+            const unsigned ql3 = qslot[((q - 3 - y0) & 3) * (NW * 32)];
             const unsigned qw = rest_update_pair(v[0], ql3, d0, P);  // compensated rest population
-            const long long oc = (long long)(q - 3) * nx + x0 + col;
-            float* o = fout + oc;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(o + i * P.pitch) = v[i].v;
-            qout[oc >> 1] = qw;
+            O.store(v, qw);
+            O.next_row(nx);
         }
         // row q-4 (ring index k-5) is no longer read by this warp
         __syncwarp();

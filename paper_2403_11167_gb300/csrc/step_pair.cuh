@@ -19,6 +19,12 @@
 // loaded when the row is pulled and used when that row is collided (two iterations later for
 // the free-energy kernel, one for the pseudopotential kernel).
 //
+// What bounds them: instruction issue (0.6 per cycle and sub-partition) close to memory; 4096^2 takes
+// 219 us (pseudopotential) and 242 us (free energy) per step where a copy of the same bytes takes 191.
+// The ring position and the output offsets move from row to row by additions, and a buffer below 4 GB is
+// stored to by 32-bit offsets: indexes modulo the stages and 64-bit plane addresses were a tenth of the
+// instructions (226 and 246 us).
+//
 // Requirements (checked on the host): nx % 4 == 0, nx >= 8, ny >= 4; every wait bounded.
 #pragma once
 #include <cuda_runtime.h>
@@ -96,7 +102,7 @@ __device__ __forceinline__ void store_warp_mass(F2 macc, double* slot) {
     if ((threadIdx.x & 31) == 0) *slot = s;
 }
 
-template <int NW, int S, bool DRIVE = false>
+template <int NW, int S, bool DRIVE = false, bool NEAR = true>
 __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __restrict__ fin,
                                                                  float* __restrict__ fout, const StepParams<float> P,
                                                                  int* __restrict__ err, const Drive<float> D = {},
@@ -155,10 +161,12 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
     const int sc = col + 4;
     Row2 r1, r2, r3;  // rho of rows q-1, q-2, q-3
     Row2 m2, m3;      // mu of rows q-2, q-3
-    // rest-population extensions q (two int16 per lane): copied into slot (row mod 3) of the
+    // rest-population extensions q (two int16 per lane): copied into slot (row mod 4) of the
     // lane's qext ring when the row is pulled, read two iterations later by its collision
-    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch));
-    unsigned* qout = reinterpret_cast<unsigned*>(rest_lo_plane(fout, P.pitch));
+    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch)) +
+                          (((long long)y0 * nx + x0 + col) >> 1);
+    uint32_t* const qslot = &sm.qext[0][warp][lane];
+    StripOut<NEAR> O(fout, P.pitch, (long long)y0 * nx + x0 + col);
     r1.c = r2.c = r3.c = m2.c = m3.c = F2::c(1.0f);
     r1.xm = r1.xp = r2.xm = r2.xp = r3.xm = r3.xp = F2::c(1.0f);
     m2.xm = m2.xp = m3.xm = m3.xp = F2::c(1.0f);
@@ -166,19 +174,23 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
     const F2 ax = DRIVE ? drive_ax(D, x0 + col) : F2::c(0.0f);
     F2 macc = F2::c(0.0f);
     bool ok = mbar_wait_bounded(&sm.full[0], 0) && mbar_wait_bounded(&sm.full[1], 0);
+    RingPos<S> pos{2, 0};  // row q+1 (ring index 2 at first), and the stages of the rows up to it
+    const float *a0 = sm.stage[0], *a1 = sm.stage[0], *a2 = sm.stage[0], *a3 = sm.stage[1], *a4 = sm.stage[2];
+    int release = 0;  // stage of row q-3, from the iteration that has read all of it
 #pragma unroll 1
     for (int q = y0 - 2; q <= y1 + 1 && ok; ++q) {
-        const int k = q + 1 - rbase;  // ring index of row q+1
-        ok = mbar_wait_bounded(&sm.full[k % S], (uint32_t)((k / S) & 1));
+        ok = mbar_wait_bounded(&sm.full[pos.s], pos.parity);
         if (!ok) break;
-        if (out && q >= y0 && q < y1)
-            cp_async4(&sm.qext[(q - y0 + 3) % 3][warp][lane], qin + (((long long)q * nx + x0 + col) >> 1));
+        if (out && q >= y0 && q < y1) {
+            cp_async4(qslot + ((q - y0) & 3) * (NW * 32), qin);
+            qin += nx >> 1;
+        }
         cp_async_commit();
         // pull row q, rho(q)
         F2 rho0 = F2::c(1.0f);
         if (act) {
             F2 v[9];
-            pull_pair<W8>(sm.stage[(k - 2) % S], sm.stage[(k - 1) % S], sm.stage[k % S], sc, v);
+            pull_pair<W8>(a2, a3, a4, sc, v);
             rho0 = sum9_v(v);
         }
         const Row2 r0 = with_shifted(rho0);
@@ -190,10 +202,10 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
             const F2 mu = (act && q >= y0) ? fe_mu_v(r1.c, rn, P) : F2::c(0.0f);
             m1 = with_shifted(mu);
         }
-        // collide row q-2 (ring indices k-4 .. k-2 hold source rows q-3 .. q-1)
+        // collide row q-2 (a0 .. a2 hold source rows q-3 .. q-1)
         if (out && q >= y0 + 2) {
             F2 v[9], mn[9], rn[9];
-            pull_pair<W8>(sm.stage[(k - 4) % S], sm.stage[(k - 3) % S], sm.stage[(k - 2) % S], sc, v);
+            pull_pair<W8>(a0, a1, a2, sc, v);
             neighbours_pair(m3, m2, m1, mn);
             neighbours_pair(r3, r2, r1, rn);
             F2 d0;
@@ -202,18 +214,24 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
             else
                 fe_collide_v<F2, true>(v, r2.c, mn, rn, P, &d0);
             cp_async_wait<2>();  // the copy of row q-2's extensions (two groups ago) has landed
-            const unsigned ql2 = sm.qext[(q - 2 - y0 + 3) % 3][warp][lane];
+            const unsigned ql2 = qslot[((q - 2 - y0) & 3) * (NW * 32)];
             const unsigned qw = rest_update_pair(v[0], ql2, d0, P);  // compensated rest population
             if constexpr (DRIVE) macc = macc + sum9_v(v);
-            const long long oc = (long long)(q - 2) * nx + x0 + col;
-            float* o = fout + oc;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(o + i * P.pitch) = v[i].v;
-            qout[oc >> 1] = qw;
+            O.store(v, qw);
+            O.next_row(nx);
         }
-        // row q-3 (ring index k-4) is no longer read by this warp
+        // row q-3 is no longer read by this warp (the first, y0-3, from q = y0)
         __syncwarp();
-        if (lane == 0 && k >= 4) mbar_arrive(&sm.empty[(k - 4) % S]);
+        if (q >= y0) {
+            if (lane == 0) mbar_arrive(&sm.empty[release]);
+            release = release == S - 1 ? 0 : release + 1;
+        }
+        a0 = a1;
+        a1 = a2;
+        a2 = a3;
+        a3 = a4;
+        pos.next();
+        a4 = sm.stage[pos.s];
         r3 = r2;
         r2 = r1;
         r1 = r0;
@@ -232,7 +250,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) fe_step_pair(const float* __
 // One CTA's strip of the pseudopotential step: columns [x0, x0 + w) (w <= 60 NW, x0 and w
 // multiples of 4), rows [y0, y1).  Called by every thread of the CTA.
 // DRIVE: as for fe_step_pair; mass points to this CTA's NW slots.
-template <int NW, int S, bool DRIVE = false>
+template <int NW, int S, bool DRIVE = false, bool NEAR = true>
 __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, float* __restrict__ fout,
                                               const StepParams<float>& P, int x0, int w, int y0, int y1,
                                               WarpStripSmem<NW, S, 60>& sm, int* __restrict__ err,
@@ -274,10 +292,12 @@ __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, flo
     const bool out = act && lane >= 1 && 2 * lane <= nw;
     const int sc = col + 4;
     Row2 p1, p2;  // psi of rows q-1, q-2
-    // rest-population extensions q (two int16 per lane): copied into slot (row mod 3) of the
+    // rest-population extensions q (two int16 per lane): copied into slot (row mod 4) of the
     // lane's qext ring when the row is pulled, read by its collision in the next iteration
-    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch));
-    unsigned* qout = reinterpret_cast<unsigned*>(rest_lo_plane(fout, P.pitch));
+    const unsigned* qin = reinterpret_cast<const unsigned*>(rest_lo_plane(fin, P.pitch)) +
+                          (((long long)y0 * nx + x0 + col) >> 1);
+    uint32_t* const qslot = &sm.qext[0][warp][lane];
+    StripOut<NEAR> O(fout, P.pitch, (long long)y0 * nx + x0 + col);
     p1.c = p2.c = F2::c(0.0f);
     p1.xm = p1.xp = p2.xm = p2.xp = F2::c(0.0f);
     F2 rho1 = F2::c(1.0f);  // rho of row q-1
@@ -285,26 +305,30 @@ __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, flo
     const F2 ax = DRIVE ? drive_ax(*D, x0 + col) : F2::c(0.0f);
     F2 macc = F2::c(0.0f);
     bool ok = mbar_wait_bounded(&sm.full[0], 0) && mbar_wait_bounded(&sm.full[1], 0);
+    RingPos<S> pos{2, 0};  // row q+1 (ring index 2 at first), and the stages of the rows up to it
+    const float *a0 = sm.stage[0], *a1 = sm.stage[0], *a2 = sm.stage[1], *a3 = sm.stage[2];
+    int release = 0;  // stage of row q-2, from the iteration that has read all of it
 #pragma unroll 1
     for (int q = y0 - 1; q <= y1 && ok; ++q) {
-        const int k = q + 1 - rbase;  // ring index of row q+1
-        ok = mbar_wait_bounded(&sm.full[k % S], (uint32_t)((k / S) & 1));
+        ok = mbar_wait_bounded(&sm.full[pos.s], pos.parity);
         if (!ok) break;
-        if (out && q >= y0 && q < y1)
-            cp_async4(&sm.qext[(q - y0 + 3) % 3][warp][lane], qin + (((long long)q * nx + x0 + col) >> 1));
+        if (out && q >= y0 && q < y1) {
+            cp_async4(qslot + ((q - y0) & 3) * (NW * 32), qin);
+            qin += nx >> 1;
+        }
         cp_async_commit();
         F2 rho0 = F2::c(1.0f), psi = F2::c(0.0f);
         if (act) {
             F2 v[9];
-            pull_pair<W8>(sm.stage[(k - 2) % S], sm.stage[(k - 1) % S], sm.stage[k % S], sc, v);
+            pull_pair<W8>(a1, a2, a3, sc, v);
             rho0 = sum9_v(v);
             psi = pseudo_psi_v(rho0, P);
         }
         const Row2 p0 = with_shifted(psi);
-        // collide row q-1 (ring indices k-3 .. k-1 hold source rows q-2 .. q)
+        // collide row q-1 (a0 .. a2 hold source rows q-2 .. q)
         if (out && q > y0) {
             F2 v[9], pn[9];
-            pull_pair<W8>(sm.stage[(k - 3) % S], sm.stage[(k - 2) % S], sm.stage[(k - 1) % S], sc, v);
+            pull_pair<W8>(a0, a1, a2, sc, v);
             neighbours_pair(p2, p1, p0, pn);
             F2 d0;
             if constexpr (DRIVE)
@@ -312,18 +336,23 @@ __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, flo
             else
                 pp_collide_v<F2, true>(v, rho1, pn[0], pn, P, &d0);
             cp_async_wait<1>();  // the copy of row q-1's extensions (one group ago) has landed
-            const unsigned ql1 = sm.qext[(q - 1 - y0 + 3) % 3][warp][lane];
+            const unsigned ql1 = qslot[((q - 1 - y0) & 3) * (NW * 32)];
             const unsigned qw = rest_update_pair(v[0], ql1, d0, P);  // compensated rest population
             if constexpr (DRIVE) macc = macc + sum9_v(v);
-            const long long oc = (long long)(q - 1) * nx + x0 + col;
-            float* o = fout + oc;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(o + i * P.pitch) = v[i].v;
-            qout[oc >> 1] = qw;
+            O.store(v, qw);
+            O.next_row(nx);
         }
-        // row q-2 (ring index k-3) is no longer read by this warp
+        // row q-2 is no longer read by this warp (the first, y0-2, from q = y0)
         __syncwarp();
-        if (lane == 0 && k >= 3) mbar_arrive(&sm.empty[(k - 3) % S]);
+        if (q >= y0) {
+            if (lane == 0) mbar_arrive(&sm.empty[release]);
+            release = release == S - 1 ? 0 : release + 1;
+        }
+        a0 = a1;
+        a1 = a2;
+        a2 = a3;
+        pos.next();
+        a3 = sm.stage[pos.s];
         p2 = p1;
         p1 = p0;
         rho1 = rho0;
@@ -333,7 +362,7 @@ __device__ __forceinline__ void pp_pair_strip(const float* __restrict__ fin, flo
     if (!ok) atomicExch(err, 1);
 }
 
-template <int NW, int S, bool DRIVE = false>
+template <int NW, int S, bool DRIVE = false, bool NEAR = true>
 __global__ void __launch_bounds__((NW + 1) * 32, 1) pp_step_pair(const float* __restrict__ fin,
                                                                  float* __restrict__ fout, const StepParams<float> P,
                                                                  int* __restrict__ err, const Drive<float> D = {},
@@ -349,7 +378,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, 1) pp_step_pair(const float* __
         return;
     }
     const int y0 = blockIdx.y * P.rows;
-    pp_pair_strip<NW, S, DRIVE>(fin, fout, P, x0, w, y0, min(y0 + P.rows, P.ny), sm, err, &D,
+    pp_pair_strip<NW, S, DRIVE, NEAR>(fin, fout, P, x0, w, y0, min(y0 + P.rows, P.ny), sm, err, &D,
                                 DRIVE ? mass + (blockIdx.y * gridDim.x + blockIdx.x) * NW : nullptr);
 }
 

@@ -13,7 +13,7 @@ cudaError_t launch(const real* fin, real* fout, const StepParams<real>& P, const
     constexpr bool f32 = std::is_same<real, float>::value;
     if (!f32 || P.nx % 2 != 0)
         tile_step<real, MODEL, WALLS, DRIVE, false, false><<<grid, threads, 0, s>>>(fin, fout, P, T);
-    else if (P.pitch * 40 >= (1LL << 32))
+    else if (!near_buffer(P.pitch))
         tile_step<real, MODEL, WALLS, DRIVE, f32, false><<<grid, threads, 0, s>>>(fin, fout, P, T);
     else
         tile_step<real, MODEL, WALLS, DRIVE, f32, f32><<<grid, threads, 0, s>>>(fin, fout, P, T);

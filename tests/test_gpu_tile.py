@@ -81,11 +81,11 @@ def _device_populations(ctx):
 
 
 @pytest.mark.parametrize("case", [
-    (PP, 2052, 2196, {}), (PP, 8, 563000, {}), (PP, 600004, 8, {}), (PP, 4100, 1101, {}),
+    (PP, 2196, 2192, {}), (PP, 8, 600400, {}), (PP, 600004, 8, {}), (PP, 4100, 1173, {}),
     (FE, 1684, 1680, {}), (FE, 8, 350400, {}), (FE, 300004, 10, {}), (FE, 484, 5801, {}),
     (FE, 1684, 1680, dict(A=0.15)), (FE, 300004, 10, dict(A=0.1)),
-    (PP, 1848, 1844, dict(walls=1)), (FE, 1452, 1450, dict(walls=1)), (FE, 1452, 1450, dict(walls=2)),
-    (PP, 1740, 1732, dict(drive=5e-4)), (FE, 1228, 1226, dict(drive=5e-4))])
+    (PP, 2284, 2280, dict(walls=1)), (FE, 1764, 1762, dict(walls=1)), (FE, 1764, 1762, dict(walls=2)),
+    (PP, 1588, 1580, dict(drive=5e-4)), (FE, 1764, 1760, dict(drive=5e-4))])
 def test_strips_match_tiles(case, monkeypatch):
     """Just above the size rule a lattice runs the strip kernels, with LBM_NO_TMA the tile kernel: the
     same bits, rest extensions included, after one graph of steps and some single ones (square, one
@@ -119,6 +119,56 @@ def test_strips_match_tiles(case, monkeypatch):
         assert float((a - b).abs().max()) <= 1e-6 * float(b.abs().max())
     else:
         assert torch.equal(fa, fb) and torch.equal(qa, qb)
+
+
+@pytest.mark.parametrize("model,A", [(PP, 0.0), (FE, 0.0), (FE, 0.1)])
+def test_buffers_of_4_gb(model, A, monkeypatch):
+    """From 4 GB a buffer's cells are not reached by 32-bit byte offsets: strips and tiles, the same bits
+    after three steps (cells of a row above 2^31 bytes of a plane's offset included)."""
+    import torch
+
+    n = 10364
+    assert n * n * 40 >= 2**32
+    rng = torch.Generator(device="cuda").manual_seed(1)
+    rho, want = None, None
+    for tiles in (False, True):
+        if tiles:
+            monkeypatch.setenv("LBM_NO_TMA", "1")
+        ctx, rp, th = gpu_context(model, F32, n, n, a=0.25, Tr=0.85, tau_nu=0.8, **(dict(A=A) if A else {}))
+        if rho is None:
+            rho = 0.5 * (th.rho_l + th.rho_v) * (0.98 + 0.04 * torch.rand((n, n), device="cuda", generator=rng))
+            torch.cuda.synchronize()
+        ctx.set_density_device(rho)
+        ctx.step(3)
+        got = _device_populations(ctx)
+        ctx.close()
+        if want is None:
+            want = got
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def test_batch_lattice_of_4_gb():
+    """A batch that holds a lattice of 4 GB takes the strip kernel with 64-bit addresses: the observables
+    of single-lattice runs to FP64 rounding of their sums."""
+    from paper_2403_11167_gb300 import lbm
+
+    p = lbm.lbm_params_default(PP, precision=F32, a=0.25, Tr=0.85, tau_nu=0.8)
+    _, th = lbm.lbm_resolve_params(p)
+    specs, rhos = [], []
+    for nx, ny in ((10364, 10364), (512, 64)):
+        specs.append(dict(nx=nx, ny=ny, geometry=0, nsteps=3, params=p))
+        rhos.append(inputs.random_field(nx, ny, 0.45 * (th.rho_l + th.rho_v), 0.55 * (th.rho_l + th.rho_v), seed=ny))
+    b = lbm.Batch(specs, rhos)
+    b.run()
+    for got, s, r in zip(b.observables(), specs, rhos):
+        ctx = lbm.Context(p, s["nx"], s["ny"])
+        ctx.set_density(r)
+        ctx.step(3)
+        want = ctx.observables(0)
+        ctx.close()
+        for key in set(got) & set(want):
+            assert got[key] == pytest.approx(want[key], rel=1e-9, abs=1e-12, nan_ok=True), key
+    b.close()
 
 
 def test_batch_strips_and_tiles_match_single_lattices():
