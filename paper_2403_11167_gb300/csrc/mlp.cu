@@ -315,20 +315,35 @@ extern "C" int lbm_surrogate_predict_fp32(lbm_surrogate* m, const float* X, int 
     return LBM_OK;
 }
 
+// Up to kSmallQueries, three rounds of 32 queries on every SM, the layers are split over a CTA's warps, one
+// tile of 16 queries per CTA while there are SMs for that, else two; above it a warp takes its tiles through
+// the network alone (split mode, us per call, split over warps and not: 1 query 8.1, 14.6; 4864 10.5, 14.7;
+// 9728 14.5, 15.3; 14592 17.6, 18.8; 19456 20.8, 19.6; 65536 56, 46).
+constexpr int kSmallQueries = 3 * kSMs * 2 * kInferRows;
+template <bool kSplit>
+static cudaError_t infer(const lbm_surrogate* m, const float* X, int n, float* Y, cudaStream_t s) {
+    const int tiles = n / kInferRows + (n % kInferRows != 0);
+    if (n <= kSmallQueries) {
+        if (tiles <= kSMs)
+            mlp_infer_small_kernel<kSplit, 1><<<tiles, kSmallThreads, 0, s>>>(X, n, m->d_params, m->d_stats, Y);
+        else
+            mlp_infer_small_kernel<kSplit, 2>
+                <<<std::min(kSMs, (tiles + 1) / 2), kSmallThreads, 0, s>>>(X, n, m->d_params, m->d_stats, Y);
+        return cudaGetLastError();
+    }
+    const int smem = (int)sizeof(InferSmem);
+    const cudaError_t e =
+        cudaFuncSetAttribute(mlp_infer_kernel<kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    mlp_infer_kernel<kSplit><<<std::min(kSMs, tiles), kInferThreads, smem, s>>>(X, n, m->d_params, m->d_stats, Y);
+    return cudaGetLastError();
+}
+
 extern "C" int lbm_surrogate_predict_device(lbm_surrogate* m, const float* X_dev, int n, float* Y_dev, int mode,
                                             void* stream) {
     if (!m || !X_dev || !Y_dev || n < 1 || (mode != LBM_INFER_SPLIT_BF16 && mode != LBM_INFER_BF16)) return LBM_ERR_ARG;
     cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : m->stream;
-    const int smem = (int)sizeof(InferSmem);
-    const int grid = std::min(kSMs, (n + kInferRows - 1) / kInferRows);
-    if (mode == LBM_INFER_SPLIT_BF16) {
-        MCK(cudaFuncSetAttribute(mlp_infer_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        mlp_infer_kernel<true><<<grid, kInferThreads, smem, s>>>(X_dev, n, m->d_params, m->d_stats, Y_dev);
-    } else {
-        MCK(cudaFuncSetAttribute(mlp_infer_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        mlp_infer_kernel<false><<<grid, kInferThreads, smem, s>>>(X_dev, n, m->d_params, m->d_stats, Y_dev);
-    }
-    MCK(cudaGetLastError());
+    MCK(mode == LBM_INFER_SPLIT_BF16 ? infer<true>(m, X_dev, n, Y_dev, s) : infer<false>(m, X_dev, n, Y_dev, s));
     return LBM_OK;
 }
 

@@ -70,3 +70,28 @@ def test_queries_at_tile_edges(lbm, n, mode):
     bound = M.bf16_error_bound(th.astype(np.float64), X.astype(np.float64), st64, u=2.0 ** -14 if mode == "split" else 2.0 ** -8)
     assert np.all(np.abs(yn - ref) <= bound + 1e-5)
     m.close()
+
+
+@pytest.mark.parametrize("mode", ["split", "single"])
+def test_predictions_do_not_depend_on_their_number(lbm, mode):
+    """The kernel for few queries (one tile of 16 per CTA to 2432, two above, several rounds to 14592) and
+    the one for many: the same bits for the same query."""
+    import torch
+
+    sizes = [1, 16, 17, 33, 152 * 16, 152 * 16 + 1, 152 * 32, 152 * 32 + 1, 152 * 64 + 17, 152 * 96, 152 * 96 + 1]
+    X, _ = _data(sizes[-1], seed=7)
+    m = lbm.Surrogate(lbm.Surrogate.standardisation(X, _data(sizes[-1], seed=7)[1]), seed=1)
+    m.set_params(_theta(6))
+    x = torch.from_numpy(np.ascontiguousarray(X, dtype=np.float32)).cuda()
+    torch.cuda.synchronize()
+    got = []
+    for n in sizes:
+        y = torch.full((n + 1, 4), -7.0, device="cuda")
+        torch.cuda.synchronize()
+        m.predict_device(x[-n:], y[:n], mode=lbm.LBM_INFER_SPLIT_BF16 if mode == "split" else lbm.LBM_INFER_BF16)
+        torch.cuda.synchronize()
+        assert bool((y[n:] == -7.0).all())
+        got.append(y[:n])
+    for y in got[:-1]:
+        assert torch.equal(y, got[-1][-len(y):])
+    m.close()
