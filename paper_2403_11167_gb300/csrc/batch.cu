@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(32 * (kBatchTileRows + 2))
         if (!out_row) continue;
         F2 pn[9];
         neighbours(shifted(s[warp - 1][lane]), shifted(psi), shifted(s[warp + 1][lane]), pn);
-        tile_collide_pp(v, rho, pn, F2::c(P.fx), F2::c(P.fy), qw, P);
+        tile_collide_pp<-1>(v, rho, pn, F2::c(P.fx), F2::c(P.fy), qw, P, Exchange{});
         if (out) {
 #pragma unroll
             for (int j = 0; j < 9; ++j) *reinterpret_cast<float2*>(fout + j * P.pitch + oc) = v[j].v;

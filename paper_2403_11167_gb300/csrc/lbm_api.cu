@@ -331,17 +331,12 @@ static size_t buffer_bytes(int precision, int nx, int ny) {
     return align256((precision == LBM_F64 ? 9 : 10) * (size_t)plane_pitch(nx, ny) * esz);
 }
 
-// Narrowest tile of the tile kernel (full model, FP64): the most tiles across a lattice.
-constexpr int kTileMinCols = lbmk::Tile<double, 2>::kCols;
-
 // Slots of the driven steps' stored mass: strip kernels, one per consumer warp of every strip CTA
-// (strips of at least one row); FP64 tile kernel, one per tile row, for the state that is read and
-// for the one that is written; FP32 tile kernel, three sets of accumulators.
+// (strips of at least one row); tile kernel, three sets of accumulators.
 static size_t drive_mass_slots(int nx, int ny) {
     const size_t pp = (size_t)((nx + kPPPTX - 1) / kPPPTX) * kPPPWarps;
     const size_t fe = (size_t)((nx + kFEPTX - 1) / kFEPTX) * kFEPWarps;
-    const size_t tile = 2 * (size_t)((nx + kTileMinCols - 1) / kTileMinCols);
-    return std::max(std::max(std::max(pp, fe), tile) * (size_t)ny, (size_t)3 * lbmk::kDriveParts);
+    return std::max(std::max(pp, fe) * (size_t)ny, (size_t)3 * lbmk::kDriveParts);
 }
 
 extern "C" size_t lbm_workspace_bytes(int precision, int nx, int ny) {
@@ -416,11 +411,14 @@ static void fill_step_params(lbmk::StepParams<real>& s, const lbm_ctx* c) {
 // FP64: the height that minimises tiles per SM x the FP64 operations of one tile in sequence, each
 // phase's warps spread over the SM's four sub-partitions (operations per cell of step64.cuh: sum of
 // the populations or psi, mu, u, collision).  It picks the fastest of the measured heights 1..8 on
-// 256 x 4 (6.2 us with 1), 101 x 50 (8.6 us with 2), 200 x 100 (12.8 us with 6), 256 x 128 (12.7
-// and 20.9 us with 8 and 3) and 400 x 300 (41 and 56 us with 4 and 8).
+// 256 x 4 (5.2 us with 1), 101 x 50 (7.9 us with 2), 200 x 100 (9.1 us with 5), 256 x 128 (12.4
+// and 20.5 us with 8 and 3) and 400 x 300 (40 and 56 us with 4 and 8).  A tile of one or two rows leaves
+// sub-partitions idle in the collision: two warps share a row (*share) while no SM has a second tile to
+// fill them (100 x 100, two tiles of two rows per SM: 11.9 us shared, 10.4 not; five rows of 200 x 100
+// with the fifth shared: 12.3, not: 12.2).
 // FP32: 4 rows (1022 x 770: 12.2 us, where 13.7 compared with 15.8 with 2 rows and 14.2 with 8), the full model with its
 // three halo rows 8 (1024^2: 29 us against 40 with 4), fewer while that leaves SMs without a tile.
-static int choose_tile_rows(int prec, int model, int nx, int ny) {
+static int choose_tile_rows(int prec, int model, int nx, int ny, int* share) {
     const int wb = prec == LBM_F64 ? lbmk::tile_columns<double>(model, nx) : lbmk::tile_columns<float>(model, nx);
     const long long gx = (nx + wb - 1) / wb;
     if (prec == LBM_F32) {
@@ -429,18 +427,20 @@ static int choose_tile_rows(int prec, int model, int nx, int ny) {
         return r;
     }
     static const int ops[3][4] = {{28, 0, 0, 125}, {8, 45, 0, 120}, {8, 45, 40, 140}};
+    static const int shared[2][2] = {{80, 95}, {88, 104}};  // one row; two (76 cycles an operation, not 64)
     int best = 1;
     long long least = -1;
     for (int r = 1; r <= lbmk::Tile<double, 0>::kRows; ++r) {
-        long long t = 0;
-        for (int p = 0; p < 4; ++p) {  // phase p works on the rows of the tile and of the halo it needs
-            const int halo = p == 3 ? 0 : model + 1 - p;
-            t += (long long)((r + 2 * halo + 3) / 4) * ops[model][p];
-        }
-        t *= (gx * ((ny + r - 1) / r) + 151) / 152;
+        const long long waves = (gx * ((ny + r - 1) / r) + 151) / 152;
+        const bool two = model < 2 && r <= lbmk::Tile<double, 0>::kShared && waves == 1;
+        long long t = two ? shared[model][r - 1] : (r + 3) / 4 * ops[model][3];
+        for (int p = 0; p < 3; ++p)  // phase p works on the rows of the tile and of the halo it needs
+            t += (long long)((r + 2 * (model + 1 - p) + 3) / 4) * ops[model][p];
+        t *= waves;
         if (least < 0 || t < least) {
             least = t;
             best = r;
+            *share = two;
         }
     }
     return best;
@@ -590,8 +590,6 @@ extern "C" int lbm_derived(const lbm_ctx* c, lbm_params* resolved, lbm_thermo* t
 
 constexpr int kMassBlocks = 608;  // block sums of the drive's domain mean (4 x 152 SMs)
 static_assert(kMassBlocks + lbmk::kDriveParts <= 3 * kRedBlocks, "the drive's sums share the reduction partials");
-// Most slots that every CTA of a driven FP64 tile step sums itself; above, a reduction launch precedes it.
-constexpr size_t kTileSlots = 1024;
 
 template <typename real>
 static lbmk::Drive<real> no_drive() {
@@ -680,33 +678,27 @@ static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int ban
     T.wjy = c->walls ? launch_wall_solve<real>(c, src, sp) : nullptr;
     if (driven) {
         T.driven = true;
-        if (c->prec == LBM_F32) {
-            unsigned long long* acc = reinterpret_cast<unsigned long long*>(c->dmass);
-            auto set = [&](int k) { return acc + (k % 3) * lbmk::kDriveParts; };
-            if (chain > 0) {
-                T.D = drive_terms<real>(c);
-                T.acc_in = set(chain - 1);
-            } else {
-                T.D = launch_drive<real>(c, src);
-                CK(cudaMemsetAsync(acc, 0, 3 * lbmk::kDriveParts * sizeof(*acc), c->stream));
-            }
-            T.acc_out = set(chain);
-            T.acc_zero = set(chain + 1);
+        unsigned long long* acc = reinterpret_cast<unsigned long long*>(c->dmass);
+        auto set = [&](int k) { return acc + (k % 3) * lbmk::kDriveParts; };
+        if (chain > 0) {
+            T.D = drive_terms<real>(c);
+            T.acc_in = set(chain - 1);
         } else {
-            const size_t half = (size_t)((c->nx + T.wb - 1) / T.wb) * c->ny;
-            const double* slots = c->dmass + src * half;
-            if (chain > 0 && half <= kTileSlots) {
-                T.D = drive_terms<real>(c);
-                T.slots = slots;
-                T.nslots = (int)half;
-            } else {
-                T.D = chain > 0 ? sum_drive<real>(c, slots, (int)half) : launch_drive<real>(c, src);
-            }
-            T.mass = c->dmass + (src ^ 1) * half;
+            T.D = launch_drive<real>(c, src);
+            CK(cudaMemsetAsync(acc, 0, 3 * lbmk::kDriveParts * sizeof(*acc), c->stream));
         }
+        T.acc_out = set(chain);
+        T.acc_zero = set(chain + 1);
+        // below the packing limit 4 / b = 2^e x, x in [0.5, 1), a density takes at most 49 bits and N of them 61
+        int e = 0;
+        std::frexp(4.0 / c->prm.b, &e);
+        const int bits = std::min(49, 61 - (int)std::ceil(std::log2((double)c->nx * c->ny)));
+        T.mass_scale = std::ldexp(1.0, bits - e);
+        T.mass_unit = T.D.inv_cells * (c->prec == LBM_F64 ? 1.0 / T.mass_scale : lbmk::kTileMassUnit * sp.rest_unit);
     }
+    T.rows = band > 0 ? band : choose_tile_rows(c->prec, m, c->nx, c->ny, &T.share);
     CK(lbmk::launch_tile<real>(m, c->walls, static_cast<const real*>(c->f[src]), static_cast<real*>(c->f[src ^ 1]), sp,
-                               T, band > 0 ? band : choose_tile_rows(c->prec, m, c->nx, c->ny), c->stream));
+                               T, c->stream));
     return LBM_OK;
 }
 

@@ -88,27 +88,76 @@ __device__ __forceinline__ void grad12(const double n[9], double& gx, double& gy
     gy = fma(4.0, n[2] - n[4], d57 - d86);
 }
 
+// A cell's collision by two warps (where a tile has fewer rows than the SM sub-partitions): role 0 takes the
+// energy moments and updates f_0 .. f_4, role 1 the fluxes and stresses and f_5 .. f_8; both form the force
+// and the velocity.  x: the pair's exchange in shared memory, 32 per value and the lane's own; bar: its
+// barrier.  The operations on each number are those of one warp alone (role -1), so the bits are too.
+struct Exchange {
+    int bar;
+    double* x;
+    __device__ __forceinline__ void meet() const { asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory"); }
+};
+
 // Populations from the moment increments; P4 = d pxx / 4, Z = d pxy / 4 (M^-1 of Eq. S49).
 __device__ __forceinline__ void apply_pairs(double v[9], double de, double dz, double Fx, double dqx, double Fy,
                                             double dqy, double P4, double Z) {
     const double A = fma(de, -1.0 / 36.0, dz * (-1.0 / 18.0)), B = fma(de, 1.0 / 18.0, dz * (1.0 / 36.0));
-    const double X1 = (Fx - dqx) * (1.0 / 6.0), Y1 = (Fy - dqy) * (1.0 / 6.0);
+    const double X1 = Fx - dqx, Y1 = Fy - dqy;  // times 6
     const double X2 = fma(dqx, 1.0 / 12.0, Fx * (1.0 / 6.0)), Y2 = fma(dqy, 1.0 / 12.0, Fy * (1.0 / 6.0));
     const double Ap = A + P4, Am = A - P4, Bp = B + Z, Bm = B - Z, Sp = X2 + Y2, Sm = X2 - Y2;
     v[0] = fma(dz - de, 1.0 / 9.0, v[0]);
-    v[1] += Ap + X1;
-    v[3] += Ap - X1;
-    v[2] += Am + Y1;
-    v[4] += Am - Y1;
+    v[1] += fma(X1, 1.0 / 6.0, Ap);
+    v[3] += fma(X1, -1.0 / 6.0, Ap);
+    v[2] += fma(Y1, 1.0 / 6.0, Am);
+    v[4] += fma(Y1, -1.0 / 6.0, Am);
     v[5] += Bp + Sp;
     v[7] += Bp - Sp;
     v[6] += Bm - Sm;
     v[8] += Bm + Sm;
 }
 
+__device__ __forceinline__ void apply_energy(double v[9], double de, double dz, const Exchange& E) {
+    const double A = fma(de, -1.0 / 36.0, dz * (-1.0 / 18.0)), B = fma(de, 1.0 / 18.0, dz * (1.0 / 36.0));
+    E.x[0] = B;
+    v[0] = fma(dz - de, 1.0 / 9.0, v[0]);
+    E.meet();
+    const double P4 = E.x[32], X1 = E.x[64], Y1 = E.x[96];
+    const double Ap = A + P4, Am = A - P4;
+    v[1] += fma(X1, 1.0 / 6.0, Ap);
+    v[3] += fma(X1, -1.0 / 6.0, Ap);
+    v[2] += fma(Y1, 1.0 / 6.0, Am);
+    v[4] += fma(Y1, -1.0 / 6.0, Am);
+}
+__device__ __forceinline__ void apply_flux(double v[9], double Fx, double dqx, double Fy, double dqy, double P4,
+                                           double Z, const Exchange& E) {
+    E.x[32] = P4;
+    E.x[64] = Fx - dqx;
+    E.x[96] = Fy - dqy;
+    const double X2 = fma(dqx, 1.0 / 12.0, Fx * (1.0 / 6.0)), Y2 = fma(dqy, 1.0 / 12.0, Fy * (1.0 / 6.0));
+    const double Sp = X2 + Y2, Sm = X2 - Y2;
+    E.meet();
+    const double B = E.x[0], Bp = B + Z, Bm = B - Z;
+    v[5] += Bp + Sp;
+    v[7] += Bp - Sp;
+    v[6] += Bm - Sm;
+    v[8] += Bm + Sm;
+}
+
+template <int ROLE>
+__device__ __forceinline__ void apply_role(double v[9], double de, double dz, double Fx, double dqx, double Fy,
+                                           double dqy, double P4, double Z, const Exchange& E) {
+    if (ROLE < 0)
+        apply_pairs(v, de, dz, Fx, dqx, Fy, dqy, P4, Z);
+    else if (ROLE == 0)
+        apply_energy(v, de, dz, E);
+    else
+        apply_flux(v, Fx, dqx, Fy, dqy, P4, Z, E);
+}
+
 // Pseudopotential collision (Eqs. 1, 4, 6, 10, 13, 30-32); pn: psi at the cell and at x + c_i.
+template <int ROLE>
 __device__ __forceinline__ void tile_collide_pp(double v[9], double rho, const double pn[9], double fx, double fy,
-                                                unsigned&, const StepParams<double>& P) {
+                                                unsigned&, const StepParams<double>& P, const Exchange& E) {
     const double pc = pn[0];
     const Pairs p = pairs_of(v);
     double Sx, Sy;
@@ -130,18 +179,19 @@ __device__ __forceinline__ void tile_collide_pp(double v[9], double rho, const d
     const double r = rcp_d(rho);
     const double hx = fma(0.5, Fx, p.jx), hy = fma(0.5, Fy, p.jy);  // rho u
     const double ux = hx * r, uy = hy * r;
-    const double X = hx * ux, Y = hy * uy, uFx = ux * Fx, uFy = uy * Fy;
-    const double ruu = X + Y, uF = uFx + uFy;
+    // (sums and differences of products as explicit fma, so that every role rounds them alike)
+    const double Y = hy * uy, uFy = uy * Fy, ruu = fma(hx, ux, Y), uF = fma(ux, Fx, uFy);
     // e - e_eq = -2 f0 + sax + 4 sdg - 3 rho uu, zeta - zeta_eq = 3 (f0 - sax + rho uu)
+    // (what a role has no use for is not computed)
     const double ene = fma(-3.0, ruu, fma(4.0, p.sdg, fma(-2.0, v[0], p.sax)));
     const double zne = fma(3.0, (v[0] - p.sax) + ruu, Ls);
     const double de = fma(P.h6_e, uF, P.s_e * (Ls - ene));
     const double dz = -fma(P.h6_z, uF, P.s_z * zne);
     const double dqx = -fma(P.h_q, Fx, P.s_q * (fma(-2.0, p.d13, p.t) + hx));
     const double dqy = -fma(P.h_q, Fy, P.s_q * (fma(-2.0, p.d24, p.s) + hy));
-    const double P4 = fma(P.hn2, uFx - uFy, P.sn4 * ((X - Y) - p.pxx - dQ));
+    const double P4 = fma(P.hn2, fma(ux, Fx, -uFy), P.sn4 * (fma(hx, ux, -Y) - p.pxx - dQ));
     const double Z = fma(P.hn4, fma(ux, Fy, uy * Fx), P.sn4 * (fma(hx, uy, -p.pxy) - Qxy));
-    apply_pairs(v, de, dz, Fx, dqx, Fy, dqy, P4, Z);
+    apply_role<ROLE>(v, de, dz, Fx, dqx, Fy, dqy, P4, Z, E);
 }
 
 // Free-energy collision (Eqs. 1, 6, 20, 21, 24) from the cell's force F, its velocity and the
@@ -150,20 +200,20 @@ struct Iwb64 {
     double dxux, dyux, dxuy, dyuy;  // 12 times the velocity derivatives
     double pg, dpg, A;
 };
-template <bool IWB>
+template <bool IWB, int ROLE>
 __device__ __forceinline__ void fe_collide_d(double v[9], double rho, const double rn[9], double hx, double hy,
                                              double ux, double uy, double Fx, double Fy, const Pairs& p,
-                                             const Iwb64& W, const StepParams<double>& P) {
+                                             const Iwb64& W, const StepParams<double>& P, const Exchange& E) {
     double gx, gy;
     grad12(rn, gx, gy);
-    const double X = hx * ux, Y = hy * uy, ruu = X + Y;
+    const double Y = hy * uy, ruu = fma(hx, ux, Y);
     const double Fg = IWB ? Fy - W.dpg : Fy;
     const double s = fma(ux, gx, uy * gy);                               // 12 u . grad rho
     const double Gx = fma(gx, 1.0 / 36.0, Fx), Gy = fma(gy, 1.0 / 36.0, Fg);  // F + c_s^2 grad rho
     const double fe = fma(6.0, fma(ux, Fx, uy * Fg), s * (1.0 / 3.0));   // 6 u.F + 4 u.grad rho
     // (e - e_eq) / 3 = sax + 2 sdg - rho uu, -(zeta - zeta_eq) / 3 = 2 sax + sdg - rho uu
     double ene = fma(2.0, p.sdg, p.sax) - ruu, zne = fma(2.0, p.sax, p.sdg) - ruu;
-    double Nx = (X - Y) - p.pxx, Nxy = fma(hx, uy, -p.pxy);
+    double Nx = fma(hx, ux, -Y) - p.pxx, Nxy = fma(hx, uy, -p.pxy);
     if (IWB) {
         // rho A tr S / 3, rho A (S_xx - S_yy) / 3, rho A S_xy / 3
         const double rA = rho * (W.A * (1.0 / 36.0)), rA2 = rA + rA;
@@ -173,23 +223,26 @@ __device__ __forceinline__ void fe_collide_d(double v[9], double rho, const doub
         Nx = fma(rA2, W.dxux - W.dyuy, Nx);
         Nxy = fma(rA, W.dxuy + W.dyux, Nxy);
     }
+    // (what a role has no use for is not computed)
     const double de = fma(P.h_e, fe, P.me3 * ene);
     const double dz = fma(-P.h_z, fe, P.sz3 * zne);
     const double dqx = -fma(P.h_q, Fx, P.s_q * (fma(-2.0, p.d13, p.t) + hx));
     const double dqy = -fma(P.h_q, Fy, P.s_q * (fma(-2.0, p.d24, p.s) + hy));
     const double P4 = fma(P.hn2, fma(ux, Gx, -(uy * Gy)), P.sn4 * Nx);
     const double Z = fma(P.hn4, fma(ux, Gy, uy * Gx), P.sn4 * Nxy);
-    apply_pairs(v, de, dz, Fx, dqx, Fy, dqy, P4, Z);
+    apply_role<ROLE>(v, de, dz, Fx, dqx, Fy, dqy, P4, Z, E);
 }
+template <int ROLE>
 __device__ __forceinline__ void tile_collide_fe(double v[9], double rho, const double mn[9], const double rn[9],
-                                                double fx, double fy, unsigned&, const StepParams<double>& P) {
+                                                double fx, double fy, unsigned&, const StepParams<double>& P,
+                                                const Exchange& E) {
     const Pairs p = pairs_of(v);
     double gx, gy;
     grad12(mn, gx, gy);
     const double m = rho * (-1.0 / 12.0);
     const double Fx = fma(m, gx, fx), Fy = fma(m, gy, fy);
     const double hx = fma(0.5, Fx, p.jx), hy = fma(0.5, Fy, p.jy), r = rcp_d(rho);
-    fe_collide_d<false>(v, rho, rn, hx, hy, hx * r, hy * r, Fx, Fy, p, Iwb64{}, P);
+    fe_collide_d<false, ROLE>(v, rho, rn, hx, hy, hx * r, hy * r, Fx, Fy, p, Iwb64{}, P, E);
 }
 __device__ __forceinline__ void tile_velocity(const double v[9], double rho, const double mn[9], double fx, double fy,
                                               double& ux, double& uy, double& Fx, double& Fy) {
@@ -214,7 +267,7 @@ __device__ __forceinline__ void tile_collide_iwb(double v[9], double rho, const 
     W.pg = pg;
     W.dpg = dpg;
     W.A = A;
-    fe_collide_d<true>(v, rho, rn, fma(0.5, Fx, p.jx), fma(0.5, Fy, p.jy), ux, uy, Fx, Fy, p, W, P);
+    fe_collide_d<true, -1>(v, rho, rn, fma(0.5, Fx, p.jx), fma(0.5, Fy, p.jy), ux, uy, Fx, Fy, p, W, P, Exchange{});
 }
 
 }  // namespace lbmk

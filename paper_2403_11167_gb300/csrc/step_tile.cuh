@@ -45,32 +45,36 @@ struct Tile {
     static constexpr int HC = kPer == 1 ? LV : (MODEL == 2 ? 4 : 2);
     static constexpr int kCols = 32 * kPer - 2 * HC;
     static constexpr int kRows = kPer == 2 && MODEL < 2 ? 4 : 8;
-    static constexpr int kThreads = 32 * (kRows + 2 * LV);
+    // FP64: a tile of at most kShared rows may have each row's collision done by two warps
+    static constexpr int kShared = kPer == 1 && MODEL < 2 ? 2 : 0;
+    static constexpr int kThreads = 32 * (kRows + 2 * LV + (kShared > LV ? kShared - LV : 0));
     static constexpr int kCtas = kPer == 1 ? 1 : MODEL == 0 ? 6 : MODEL == 1 ? 4 : 2;
 };
 
-// The stored mass of driven steps.  FP64: one slot per tile row, summed by every CTA of the next
-// step.  FP32: fixed-point numbers of unit 2^9 rest_unit (2^-29 of the EOS packing limit, at or below
-// the rounding of the densities they add up), added atomically to kDriveParts accumulators: integer
-// sums are exact in any order, and cost a driven FP32 step no FP64 instructions but the mean's (with
-// FP64 sums per row a 1024^2 step took 38 us, with these 21 us).  Three sets of accumulators take
-// turns: a step reads the set of the step before, adds to its own and zeroes the next one's.
+// The stored mass of driven steps: fixed-point numbers added atomically to kDriveParts accumulators.
+// Integer sums are exact in any order and cost no FP64 instructions but the mean's (FP32: with FP64 sums
+// per row a 1024^2 step took 38 us, with these 21 us; FP64: with sums per row that every CTA added up
+// 200 x 100 took 12.0 us, with these 10.1).  Three sets of accumulators take turns: a step reads the set of
+// the step before, adds to its own and zeroes the next one's.  The unit in FP32 is 2^9 rest_unit (2^-29 of
+// the EOS packing limit, at or below the rounding of the densities); in FP64 the power of two that leaves
+// the lattice's sum 61 bits and a cell's 49 (mass_scale units per density), so that the mean's rounding
+// stays below 2^-53.
 constexpr double kTileMassUnit = 512.0;  // in units of rest_unit
 
 // What a tile step takes besides StepParams: the full model's terms, the walls' solved J_y, and the
-// drive: the state's mass is the sum of D.parts, of nslots slots (FP64), or of the accumulators acc_in.
+// drive: the state's mass is the sum of D.parts or of the accumulators acc_in.
 template <typename real>
 struct TileArgs {
     int wb;    // columns per tile
+    int rows;  // rows per tile (band: of the band)
     int band;  // > 0: only the rows next to each wall
+    int share;  // two warps per row's collision (rows <= Tile::kShared)
     Ext<real> E;
     real fyg, dpg;  // fy + rho_g g (the force is fyg - rho g) and d_y p_g = rho_g g
     const real* wjy;
     bool driven;
     Drive<real> D;
-    const double* slots;
-    int nslots;
-    double* mass;  // the next state's slots (FP64)
+    double mass_unit, mass_scale;  // the accumulators' unit as a mean density; FP64: units per density
     const unsigned long long* acc_in;
     unsigned long long *acc_out, *acc_zero;
 };
@@ -87,14 +91,16 @@ __device__ __forceinline__ F2 abs_v(F2 a) { return F2(fabsf(a.v.x), fabsf(a.v.y)
 // FP32: the strip kernels' arithmetic (step64.cuh has the FP64 overloads)
 __device__ __forceinline__ F2 tile_psi(F2 rho, const StepParams<float>& P) { return pseudo_psi_v(rho, P); }
 __device__ __forceinline__ F2 tile_mu(F2 rho, const F2 n[9], const StepParams<float>& P) { return fe_mu_v(rho, n, P); }
+template <int>
 __device__ __forceinline__ void tile_collide_pp(F2 v[9], F2 rho, const F2 pn[9], F2 fx, F2, unsigned& qw,
-                                                const StepParams<float>& P) {
+                                                const StepParams<float>& P, const Exchange&) {
     F2 d0;
     pp_collide_fx_v<F2, true>(v, rho, pn[0], pn, fx, P, &d0);
     qw = rest_update_pair(v[0], qw, d0, P);
 }
+template <int>
 __device__ __forceinline__ void tile_collide_fe(F2 v[9], F2 rho, const F2 mn[9], const F2 rn[9], F2 fx, F2 fy,
-                                                unsigned& qw, const StepParams<float>& P) {
+                                                unsigned& qw, const StepParams<float>& P, const Exchange&) {
     F2 d0;
     fe_collide_f_v<F2, true>(v, rho, mn, rn, fx, fy, P, &d0);
     qw = rest_update_pair(v[0], qw, d0, P);
@@ -214,8 +220,9 @@ __device__ __forceinline__ V tile_grad_y_onesided(const V n[9], bool top) {
     return -fmav(a, n[4] - n[0], d * ((n[8] - n[1]) + (n[7] - n[3])));
 }
 
-// EVEN: FP32 with even nx (cells of a lane 8-byte aligned); NEAR: and a buffer of less than 4 GB.
-template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN, bool NEAR>
+// EVEN: FP32 with even nx (cells of a lane 8-byte aligned); NEAR: and a buffer of less than 4 GB.  SHARE: FP64,
+// a tile of at most kShared rows, two warps per row's collision.
+template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN, bool NEAR, bool SHARE>
 __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>::kCtas)
     tile_step(const real* __restrict__ fin, real* __restrict__ fout, const StepParams<real> P,
               const TileArgs<real> T) {
@@ -225,54 +232,49 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
     __shared__ V s_a[RMAX][32];                        // psi or rho
     __shared__ V s_mu[MODEL > 0 ? RMAX : 1][32];       // mu
     __shared__ V s_u[MODEL > 1 ? 2 * RMAX : 1][32];    // u_x, then u_y
-    __shared__ double s_mass[16];
     __shared__ real s_rave;
+    __shared__ double s_v[SHARE ? L::kShared : 1][10][32], s_x[SHARE ? L::kShared : 1][5][32];
     const int nx = P.nx, ny = P.ny;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nwarps = blockDim.x >> 5, rows = nwarps - 2 * LV;
+    const int rows = SHARE ? T.rows : (int)(blockDim.x >> 5) - 2 * LV, nwarps = rows + 2 * LV;  // warps with a row
     const int by = blockIdx.y + gridDim.y * blockIdx.z;  // more than 65535 tiles in y use z
     const int y0 = WALLS && T.band > 0 ? (by == 0 ? 0 : ny - T.band) : by * rows;
     if (y0 >= ny) return;
     const int y1 = WALLS && T.band > 0 ? y0 + T.band : min(y0 + rows, ny);
     const int x0 = blockIdx.x * T.wb;
     const int w = min(T.wb, nx - x0);  // > 0 (the host's grid)
-    const int y = y0 - LV + warp;      // this warp's row (rows beyond the lattice mirrored or wrapped)
+    int y = y0 - LV + warp;            // this warp's row (rows beyond the lattice mirrored or wrapped)
     const int yr = WALLS ? mirror_row(y, ny) : ny >= 16 ? wrap_once(y, ny) : wrap_idx(y, ny);
-    const bool wall = WALLS && (y == 0 || y == ny - 1);      // a wall row of the lattice or its image
+    bool wall = WALLS && (y == 0 || y == ny - 1);            // a wall row of the lattice or its image
     const bool wall_img = WALLS && (yr == 0 || yr == ny - 1);
-    const bool top = WALLS && yr != 0;
+    bool top = WALLS && yr != 0;
     const int c = KP * lane - HC;  // first column of the lane, from x0
-    const bool out_row = warp >= LV && y < y1;
-    const bool out_a = out_row && c >= 0 && c < w;
+    bool out_row = warp >= LV && y < y1;
+    bool out_a = out_row && c >= 0 && c < w;
     const bool out_b = KP == 2 && out_row && c >= 0 && c + 1 < w;
     // the lane's place in a plane (out rows and lanes only), and with NEAR in bytes in the rest plane
-    const long long oc = NEAR ? 0 : (long long)y * nx + x0 + c;
+    long long oc = NEAR ? 0 : (long long)y * nx + x0 + c;
     const unsigned oc32 = NEAR ? (unsigned)(y * nx + x0 + c) * 4u : 0u, qo = (unsigned)P.pitch * 36u + oc32 / 2;
 
     // the state's mean density: every CTA sums in the same order
     if constexpr (DRIVE) {
-        if (KP == 1 && T.nslots > 0) {
-            double s = 0.0;
-            for (int k = threadIdx.x; k < T.nslots; k += blockDim.x) s += __ldg(T.slots + k);
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) s_mass[warp] = s;
-        } else if (warp == 0) {
+        if (warp == 0) {
             double m;
-            if (KP == 2 && T.acc_in) {
+            if (T.acc_in) {
                 unsigned long long s = T.acc_in[lane];
                 for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                m = (double)(long long)s * (kTileMassUnit * (double)P.rest_unit * T.D.inv_cells);
+                m = (double)(long long)s * T.mass_unit;
             } else {
                 m = drive_mean(T.D);
             }
             if (lane == 0) s_rave = (real)m;
         }
-        if (KP == 2 && blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
+        if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
     }
 
     V v[9], rho = cst<V>(1.0), f0 = cst<V>(0.0);  // f0: psi (MODEL 0)
     [[maybe_unused]] unsigned qw = 0;              // FP32: the cells' int16 rest extensions
-    if (y < y1 + LV && c < w + HC) {
+    if ((!SHARE || warp < nwarps) && y < y1 + LV && c < w + HC) {
         int xl = x0 + c - 1, xa = x0 + c, xb = x0 + c + 1, xr = x0 + c + KP;
         const bool edge = x0 < HC + 1 || x0 + w + HC >= nx;  // (of the tile) some column wraps
         if (edge) {
@@ -330,39 +332,76 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
         rho = sum9_v(v);
         if (MODEL == 0) f0 = tile_psi(rho, P);
     }
-    s_a[warp][lane] = MODEL == 0 ? f0 : rho;
+    // SHARE, a tile of n rows: warp LV + i collides row i (role 0) together with warp
+    // LV + n + i (role 1), on another sub-partition.  The two take 80 and 88 operations in sequence
+    // (pseudopotential, free energy) where one takes 125 and 120, each 64 cycles, or 76 with all four
+    // sub-partitions busy (256 x 4: 6.1 us per step alone, 5.2 shared; 101 x 50 channel: 8.4, 7.9).
+    [[maybe_unused]] int rw = warp, role = -1, sh = 0;
+    if constexpr (SHARE) {
+        const int n = y1 - y0, i = warp - LV;
+        if (i >= 0 && i < 2 * n) {
+            role = i < n ? 0 : 1;
+            sh = i - role * n;
+            rw = LV + sh;
+        }
+        if (role == 0) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) s_v[sh][k][lane] = v[k];
+            s_v[sh][9][lane] = rho;
+        }
+    }
+    if (!SHARE || warp < nwarps) s_a[warp][lane] = MODEL == 0 ? f0 : rho;
     __syncthreads();
+    // the second warp of a row takes the row's place once the field of its own row is written
+    auto join = [&]() {
+        if constexpr (SHARE) {
+            if (role != 1) return;
+            y = y0 - LV + rw;
+            wall = WALLS && (y == 0 || y == ny - 1);
+            top = WALLS && y != 0;
+            out_row = true;
+            out_a = c >= 0 && c < w;
+            oc = (long long)y * nx + x0 + c;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = s_v[sh][i][lane];
+            rho = s_v[sh][9][lane];
+        }
+    };
+    if (MODEL == 0) join();
 
     // external force of the lane's cells (body force, drive, buoyancy)
     V fx = cst<V>(P.fx), fy = cst<V>(P.fy);
-    if constexpr (DRIVE) {
-        real rave;
-        if (KP == 1 && T.nslots > 0) {
-            double s = (lane & 15) < nwarps ? s_mass[lane & 15] : 0.0;
-            for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            rave = (real)(s * T.D.inv_cells);
-        } else {
-            rave = s_rave;
-        }
+    [[maybe_unused]] real rave = real(0);
+    [[maybe_unused]] auto drive = [&]() {
         const int gx = x0 + c;
         const real al = gx <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi, ah = gx + 1 <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi;
         if constexpr (KP == 1)
-            fx = fma(al, fabs(rho - rave), fx);
+            fx = fma(al, fabs(rho - rave), P.fx);
         else
-            fx = fmav(F2(al, ah), abs_v(rho - F2::c(rave)), fx);
+            fx = fmav(F2(al, ah), abs_v(rho - F2::c(rave)), F2::c(P.fx));
+    };
+    if constexpr (DRIVE) {
+        rave = s_rave;
+        drive();
     }
     if (MODEL == 2) fy = fmav(cst<V>(-T.E.g), rho, cst<V>(T.fyg));
 
     if constexpr (MODEL == 0) {
         if (!out_row) return;
         V pn[9];
-        neighbours(shifted(s_a[warp - 1][lane]), shifted(f0), shifted(s_a[warp + 1][lane]), pn);
+        neighbours(shifted(s_a[rw - 1][lane]), shifted(role == 1 ? s_a[rw][lane] : f0), shifted(s_a[rw + 1][lane]), pn);
         if (wall) {
             mirror_neighbours(pn, top);
             const V Fx = fmav(pn[0], tile_grad_x(pn), fx);  // Eq. (10) + external
             tile_wall_fill(v, top, cst<V>(-0.5) * Fx, cst<V>(-0.5) * fy);
         }
-        tile_collide_pp(v, rho, pn, fx, fy, qw, P);
+        const Exchange E{1 + sh, &s_x[sh][0][lane]};
+        if (SHARE && role == 0)
+            tile_collide_pp<0>(v, rho, pn, fx, fy, qw, P, E);
+        else if (SHARE && role == 1)
+            tile_collide_pp<1>(v, rho, pn, fx, fy, qw, P, E);
+        else
+            tile_collide_pp<-1>(v, rho, pn, fx, fy, qw, P, E);
     } else {
         Row<V> rm, r0 = shifted(rho), rp, m0;
         V mu = cst<V>(0.0);
@@ -373,12 +412,20 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
             neighbours(rm, r0, rp, n);
             mu = tile_mu(rho, n, P);
         }
-        s_mu[warp][lane] = mu;
+        if (!SHARE || warp < nwarps) s_mu[warp][lane] = mu;
         __syncthreads();
         if constexpr (MODEL == 1) {
+            join();
             if (!out_row) return;
             V mn[9], rn[9];
-            neighbours(shifted(s_mu[warp - 1][lane]), shifted(mu), shifted(s_mu[warp + 1][lane]), mn);
+            if (SHARE && role == 1) {
+                rm = shifted(s_a[rw - 1][lane]);
+                r0 = shifted(rho);
+                rp = shifted(s_a[rw + 1][lane]);
+                mu = s_mu[rw][lane];
+                if (DRIVE) drive();
+            }
+            neighbours(shifted(s_mu[rw - 1][lane]), shifted(mu), shifted(s_mu[rw + 1][lane]), mn);
             neighbours(rm, r0, rp, rn);
             if (wall) {
                 // the one-sided reading's normal force -rho d_y mu enters through fy
@@ -388,7 +435,13 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
                 const V Fx = fmav(-rho, tile_grad_x(mn), fx);
                 tile_wall_fill(v, top, cst<V>(-0.5) * Fx, cst<V>(-0.5) * fy);
             }
-            tile_collide_fe(v, rho, mn, rn, fx, fy, qw, P);
+            const Exchange E{1 + sh, &s_x[sh][0][lane]};
+            if (SHARE && role == 0)
+                tile_collide_fe<0>(v, rho, mn, rn, fx, fy, qw, P, E);
+            else if (SHARE && role == 1)
+                tile_collide_fe<1>(v, rho, mn, rn, fx, fy, qw, P, E);
+            else
+                tile_collide_fe<-1>(v, rho, mn, rn, fx, fy, qw, P, E);
         } else {
             V ux = cst<V>(0.0), uy = cst<V>(0.0), Fx = cst<V>(0.0), Fy = cst<V>(0.0);
             if (warp >= 2 && warp < nwarps - 2 && y < y1 + 1) {
@@ -430,9 +483,21 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
     if constexpr (DRIVE) {
         // the mass this warp stored
         if constexpr (KP == 1) {
-            double s = out_a ? sum9_v(v) : 0.0;
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) T.mass[(long long)y * gridDim.x + blockIdx.x] = s;
+            double s = (v[5] + v[7]) + (v[6] + v[8]);
+            if (SHARE && role >= 0) {
+                const Exchange E{1 + sh, &s_x[sh][0][lane]};
+                if (role == 1) E.x[128] = s;
+                E.meet();
+                s = E.x[128];
+            }
+            s = v[0] + (((v[1] + v[3]) + (v[2] + v[4])) + s);
+            // in the low bits of s scale + 1.5 2^52; summed over the warp in two halves
+            const long long k = __double_as_longlong(fma(s, T.mass_scale, 6755399441055744.0)) - 0x4338000000000000ll;
+            const int lo = __reduce_add_sync(0xffffffffu, out_a ? (int)(k & 0x3ffffff) : 0);
+            const int hi = __reduce_add_sync(0xffffffffu, out_a ? (int)(k >> 26) : 0);
+            if (lane == 0 && role != 1)
+                atomicAdd(T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts,
+                          (unsigned long long)(((long long)hi << 26) + lo));
         } else {
             const F2 m = sum9_v(v) * F2::c(P.rest_inv * (float)(1.0 / kTileMassUnit));
             const int k = out_a ? __float2int_rn(m.v.x) : 0, l = out_b ? __float2int_rn(m.v.y) : 0;
@@ -447,7 +512,8 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
     if constexpr (KP == 1) {
         if (out_a)
 #pragma unroll
-            for (int i = 0; i < 9; ++i) fout[i * P.pitch + oc] = v[i];
+            for (int i = 0; i < 9; ++i)
+                if (role < 0 || (i < 5) == (role == 0)) fout[i * P.pitch + oc] = v[i];
     } else if constexpr (NEAR) {
         if (out_a) {
             char* b = reinterpret_cast<char*>(fout);

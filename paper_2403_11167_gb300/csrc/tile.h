@@ -19,10 +19,9 @@ inline int tile_columns(int model, int nx) {
                         : tile_columns(nx, Tile<real, 2>::kCols, Tile<real, 2>::kPer);
 }
 
-// One step of the tile kernel.  model: 0 pseudopotential, 1 free energy, 2 full free energy; rows:
-// rows per tile (T.band > 0: the band).  walls and drive (T.driven) exclude each other.
+// One step of the tile kernel.  model: 0 pseudopotential, 1 free energy, 2 full free energy.  walls and drive (T.driven) exclude each other.
 template <typename real>
 cudaError_t launch_tile(int model, bool walls, const real* fin, real* fout, const StepParams<real>& P,
-                        const TileArgs<real>& T, int rows, cudaStream_t s);
+                        const TileArgs<real>& T, cudaStream_t s);
 
 }  // namespace lbmk

@@ -69,6 +69,38 @@ def test_tile_edges_against_oracle(model, precision, option):
         ctx.close()
 
 
+@pytest.mark.parametrize("model", [PP, FE])
+@pytest.mark.parametrize("option", ["plain", "drive", "walls", "onesided"])
+@pytest.mark.parametrize("nx,ny", [(31, 1), (29, 2), (50, 4), (101, 50), (28, 150), (200, 100), (256, 4), (57, 310)])
+def test_shared_rows_match_unshared(model, option, nx, ny):
+    """FP64 tiles with one or two rows left over by fours split them between two warps while there is one
+    tile per SM; copies of the lattice side by side have more tiles and do not.  The same bits in every
+    copy; with the drive the mean density is summed in another order, 1e-13 of the densities."""
+    if option in ("walls", "onesided") and (ny < 4 or (option == "onesided" and model == PP)):
+        pytest.skip("walls")
+    walls = {"walls": 1, "onesided": 2}.get(option, 0)
+    copies = -(-160 * 28 * 8 // (nx * ny)) + 1
+    kw = dict(a=0.25, Tr=0.85, tau_nu=0.9, body_fx=1e-5, body_fy=-2e-5 if walls == 2 else 0.0)
+    if model == PP:
+        kw.update(kappa_P=0.7, kappa_Li=-0.2)
+    got = []
+    for k in (1, copies):
+        ctx, rp, th = gpu_context(model, F64, nx * k, ny, walls=walls, **kw)
+        rho0 = inputs.random_field(nx, ny, th.rho_v * 1.5, th.rho_l * 0.8, seed=nx + ny)
+        ctx.set_density(np.tile(rho0, (1, k)))
+        if option == "drive":
+            ctx.set_drive(5e-4, 5e-4, nx * k, 2)
+        ctx.step(STEPS)
+        got.append(ctx.populations())
+        ctx.close()
+    small, big = got[0], got[1].reshape(9, ny, copies, nx)
+    for c in range(copies):
+        if option == "drive":
+            assert np.max(np.abs(big[:, :, c] - small)) <= 1e-13 * np.max(small)
+        else:
+            assert np.array_equal(big[:, :, c], small), c
+
+
 def _device_populations(ctx):
     import torch
 
