@@ -411,8 +411,8 @@ static void fill_step_params(lbmk::StepParams<real>& s, const lbm_ctx* c) {
 // FP64: the height that minimises tiles per SM x the FP64 operations of one tile in sequence, each
 // phase's warps spread over the SM's four sub-partitions (operations per cell of step64.cuh: sum of
 // the populations or psi, mu, u, collision).  It picks the fastest of the measured heights 1..8 on
-// 256 x 4 (5.2 us with 1), 101 x 50 (7.9 us with 2), 200 x 100 (9.1 us with 5), 256 x 128 (12.4
-// and 20.5 us with 8 and 3) and 400 x 300 (40 and 56 us with 4 and 8).  A tile of one or two rows leaves
+// 256 x 4 (5.2 us with 1), 101 x 50 (7.3 us with 2), 200 x 100 (9.1 us with 5), 256 x 128 (12.4
+// and 18.2 us with 8 and 3) and 400 x 300 (40 us with 4).  A tile of one or two rows leaves
 // sub-partitions idle in the collision: two warps share a row (*share) while no SM has a second tile to
 // fill them (100 x 100, two tiles of two rows per SM: 11.9 us shared, 10.4 not; five rows of 200 x 100
 // with the fifth shared: 12.3, not: 12.2).
@@ -426,7 +426,7 @@ static int choose_tile_rows(int prec, int model, int nx, int ny, int* share) {
         while (r > 2 && gx * ((ny + r - 1) / r) < 152) r /= 2;
         return r;
     }
-    static const int ops[3][4] = {{28, 0, 0, 125}, {8, 45, 0, 120}, {8, 45, 40, 140}};
+    static const int ops[3][4] = {{28, 0, 0, 125}, {8, 33, 0, 120}, {8, 33, 40, 140}};
     static const int shared[2][2] = {{80, 95}, {88, 104}};  // one row; two (76 cycles an operation, not 64)
     int best = 1;
     long long least = -1;

@@ -12,7 +12,7 @@
 // What bounds it (GB300).  FP64: the FP64 pipe, 64 cycles per warp instruction on each of the 608
 // sub-partitions whatever the number of active lanes, so the arithmetic below is written for few
 // operations (step64.cuh) and the tile height spreads the rows over the sub-partitions
-// (tile_rows_f64 in lbm_api.cu).  FP32 on small lattices: the latency of one row's chain plus a
+// (choose_tile_rows in lbm_api.cu).  FP32 on small lattices: the latency of one row's chain plus a
 // launch; on lattices that fill the GPU: instruction issue.
 //
 // Per-cell FP32 arithmetic is that of the strip kernels (lbm_kernels.cuh, step_iwb_pair.cuh) on
@@ -36,7 +36,8 @@ namespace lbmk {
 // the (at most) kCols columns a warp updates; kRows the most rows of a tile.  MODEL: 0 pseudopotential, 1
 // free energy, 2 full free energy; LV is its number of halo rows.  kCtas: CTAs per SM that the registers
 // have to allow (56 and 64 registers in FP32; with one CTA less a 2048^2 step, which streams from HBM,
-// took 73.6 us instead of 66.6 and 99.0 instead of 85.4).
+// took 73.6 us instead of 66.6 and 99.0 instead of 85.4; 72 in FP64 for the full model's periodic step,
+// 256 x 128 of which took 32 us with 76).
 template <typename real, int MODEL>
 struct Tile {
     using V = typename std::conditional<std::is_same<real, float>::value, F2, double>::type;
@@ -48,7 +49,7 @@ struct Tile {
     // FP64: a tile of at most kShared rows may have each row's collision done by two warps
     static constexpr int kShared = kPer == 1 && MODEL < 2 ? 2 : 0;
     static constexpr int kThreads = 32 * (kRows + 2 * LV + (kShared > LV ? kShared - LV : 0));
-    static constexpr int kCtas = kPer == 1 ? 1 : MODEL == 0 ? 6 : MODEL == 1 ? 4 : 2;
+    static constexpr int kCtas = kPer == 1 ? (MODEL == 2 ? 2 : 1) : MODEL == 0 ? 6 : MODEL == 1 ? 4 : 2;
 };
 
 // The stored mass of driven steps: fixed-point numbers added atomically to kDriveParts accumulators.
@@ -90,7 +91,9 @@ __device__ __forceinline__ F2 abs_v(F2 a) { return F2(fabsf(a.v.x), fabsf(a.v.y)
 
 // FP32: the strip kernels' arithmetic (step64.cuh has the FP64 overloads)
 __device__ __forceinline__ F2 tile_psi(F2 rho, const StepParams<float>& P) { return pseudo_psi_v(rho, P); }
-__device__ __forceinline__ F2 tile_mu(F2 rho, const F2 n[9], const StepParams<float>& P) { return fe_mu_v(rho, n, P); }
+__device__ __forceinline__ F2 tile_mu(F2 rho, const F2 n[9], const StepParams<float>& P, const LogTable&) {
+    return fe_mu_v(rho, n, P);
+}
 template <int>
 __device__ __forceinline__ void tile_collide_pp(F2 v[9], F2 rho, const F2 pn[9], F2 fx, F2, unsigned& qw,
                                                 const StepParams<float>& P, const Exchange&) {
@@ -223,7 +226,8 @@ __device__ __forceinline__ V tile_grad_y_onesided(const V n[9], bool top) {
 // EVEN: FP32 with even nx (cells of a lane 8-byte aligned); NEAR: and a buffer of less than 4 GB.  SHARE: FP64,
 // a tile of at most kShared rows, two warps per row's collision.
 template <typename real, int MODEL, bool WALLS, bool DRIVE, bool EVEN, bool NEAR, bool SHARE>
-__global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>::kCtas)
+__global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
+                                  std::is_same<real, double>::value && (WALLS || DRIVE) ? 1 : Tile<real, MODEL>::kCtas)
     tile_step(const real* __restrict__ fin, real* __restrict__ fout, const StepParams<real> P,
               const TileArgs<real> T) {
     using L = Tile<real, MODEL>;
@@ -272,6 +276,8 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
         if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
     }
 
+    [[maybe_unused]] LogTable logs;
+    if constexpr (KP == 1 && MODEL > 0) logs.load();
     V v[9], rho = cst<V>(1.0), f0 = cst<V>(0.0);  // f0: psi (MODEL 0)
     [[maybe_unused]] unsigned qw = 0;              // FP32: the cells' int16 rest extensions
     if ((!SHARE || warp < nwarps) && y < y1 + LV && c < w + HC) {
@@ -410,7 +416,7 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads, Tile<real, MODEL>
             rp = shifted(s_a[warp + 1][lane]);
             V n[9];
             neighbours(rm, r0, rp, n);
-            mu = tile_mu(rho, n, P);
+            mu = tile_mu(rho, n, P, logs);
         }
         if (!SHARE || warp < nwarps) s_mu[warp][lane] = mu;
         __syncthreads();

@@ -101,6 +101,37 @@ def test_shared_rows_match_unshared(model, option, nx, ny):
             assert np.array_equal(big[:, :, c], small), c
 
 
+@pytest.mark.parametrize("Tr", [0.55, 0.7, 0.95])
+def test_logarithm_over_the_phase_diagram(Tr):
+    """FP64 free energy: ln rho from the vapour to the liquid density, every interval of the table and several
+    exponents, against the oracle after two steps; 1e-12 of the cell's density (its exponents and the force
+    stencil carry 1e-15)."""
+    ctx, rp, th = gpu_context(FE, F64, 64, 40, a=0.25, Tr=Tr, tau_nu=0.9)
+    x, y = np.meshgrid(np.arange(64), np.arange(40))
+    t = 0.5 - 0.25 * (np.cos(2 * np.pi * x / 64) + np.cos(2 * np.pi * y / 40))
+    rho0 = th.rho_v * (th.rho_l / th.rho_v) ** t
+    f_ref = O.run(FE, oracle_params(rp, th), O.init(FE, rho0), 2)
+    ctx.set_density(rho0)
+    ctx.step(2)
+    assert pop_err(ctx.populations(), f_ref) < 1e-12
+    ctx.close()
+
+
+@pytest.mark.parametrize("value", [-0.1, 0.0, np.nan, np.inf])
+def test_no_logarithm_is_divergence(value):
+    """A cell whose density has no logarithm ends in the divergence status, as with log()."""
+    from paper_2403_11167_gb300 import lbm
+
+    ctx, rp, th = gpu_context(FE, F64, 40, 20, a=0.25, Tr=0.85, tau_nu=0.9)
+    ctx.set_density(np.full((20, 40), th.rho_l))
+    f = ctx.populations()
+    f[:, 7, 9] = value
+    ctx.set_populations(f)
+    ctx.step(3)
+    assert ctx.observables(0)["status"] == lbm.LBM_ERR_DIVERGED
+    ctx.close()
+
+
 def _device_populations(ctx):
     import torch
 
