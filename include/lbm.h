@@ -292,11 +292,10 @@ typedef struct {
 typedef struct lbm_batch lbm_batch;
 
 /* Create a batch of n lattices.  rho0[i]: host array of nx*ny densities of lattice i
- * (copied; f starts at f^eq(rho0, u = 0)).  Lattices whose populations, psi and rho fit in
- * one CTA's shared memory (11 nx ny floats and nx ny int16 <= 200 KB, up to 4452 cells) run resident: one CTA
- * each, all steps in shared memory, in one persistent launch.  The others run as strips
- * of a work table, one launch per step for all of them, replayed as 64-step CUDA graphs on
- * a second stream concurrently.  An autotuner picks the resident block size and the strip
+ * (copied; f starts at f^eq(rho0, u = 0)).  Lattices of up to 4452 cells (11 nx ny floats and nx ny
+ * int16 <= 200 KB) run resident: one CTA each, all steps in shared memory and registers, in one
+ * persistent launch per size class.  The others run as strips or tiles of a work table, one launch per
+ * step for all of them, replayed as 64-step CUDA graphs on a further stream concurrently.  An autotuner picks the resident block size and the strip
  * height by timing short trials (cached per shape class); the state is re-initialised
  * afterwards.  The library allocates the device memory (one pooled cudaMalloc).
  * Errors: LBM_ERR_ARG (sizes, densities), LBM_ERR_UNSUPPORTED (other model or precision,
@@ -339,7 +338,7 @@ const char* lbm_batch_last_error(void);
 /* Parameters: 34,180 FP32 values, per layer l = 0..3 the weights W_l [out][in]          */
 /* (row-major) followed by the bias b_l.  Training: full-batch MSE in the standardised  */
 /* space, Adam with bias correction, cosine learning-rate decay, FP32 kernels.          */
-/* Inference: one fused kernel, BF16 inputs and weights, FP32 accumulation and          */
+/* Inference: fused kernels, BF16 inputs and weights, FP32 accumulation and             */
 /* epilogue (see the inference modes).  Host arrays are row-major n x 4 floats.  One    */
 /* surrogate owns a stream and                                                          */
 /* device buffers; calls on the same surrogate must not overlap.                       */

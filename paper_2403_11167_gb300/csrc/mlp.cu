@@ -6,7 +6,7 @@
 // calibration observables (rho_l, rho_v, W, sigma) of such runs: an MLP 4 -> 128 -> 128 ->
 // 128 -> 4 with GELU, 34,180 weights, trained in FP32 on the GPU by the kernels below
 // (one fused forward/backward kernel and one gradient-sum/Adam kernel, mlp_train.cuh), and
-// evaluated by one fused kernel with BF16 inputs and weights and FP32 accumulation on the
+// evaluated by fused kernels with BF16 inputs and weights and FP32 accumulation on the
 // tensor cores (mlp_infer.cuh).  Inputs and outputs are standardised with the training
 // set's statistics; rho_v is learned as ln(rho_v).
 #include <cuda_bf16.h>

@@ -2,7 +2,7 @@
 //
 // GB300 issues an FP64 warp instruction once per 64 cycles and sub-partition (measured, one warp or
 // four), so an FP64 step costs its number of FP64 operations and little else.  The algebra is that
-// of pp_collide / fe_collide / fe_mu (lbm_kernels.cuh) and fe_collide_iwb (step_ext.cuh) with the
+// of pp_collide_v / fe_collide_v / fe_mu (lbm_kernels.cuh) and fe_collide_iwb_v (step_iwb_pair.cuh) with the
 // population and stencil sums formed once as pair sums and differences, rho u taken as j + F/2, the
 // rest population eliminated from the non-equilibrium parts (rho = f_0 + sum of the others), and
 // every constant factor folded on the host (StepParams::d): per cell 141 operations for the
