@@ -58,8 +58,9 @@ struct Tile {
 // 200 x 100 took 12.0 us, with these 10.1).  Three sets of accumulators take turns: a step reads the set of
 // the step before, adds to its own and zeroes the next one's.  The unit in FP32 is 2^9 rest_unit (2^-29 of
 // the EOS packing limit, at or below the rounding of the densities); in FP64 the power of two that leaves
-// the lattice's sum 61 bits and a cell's 49 (mass_scale units per density), so that the mean's rounding
-// stays below 2^-53.
+// the lattice's sum 61 bits and a cell's 49 at the packing limit, with a factor of 4 above it (mass_scale
+// units per density): the mean's rounding stays below 2^-53 of the limit from about a hundred cells on, and
+// below 2^-50 on a single one.
 constexpr double kTileMassUnit = 512.0;  // in units of rest_unit
 
 // What a tile step takes besides StepParams: the full model's terms, the walls' solved J_y, and the
