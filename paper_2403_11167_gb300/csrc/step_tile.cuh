@@ -277,6 +277,11 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
         if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
     }
 
+    [[maybe_unused]] auto wrap_column = [nx](int x) {
+        while (x < 0) x += nx;
+        while (x >= nx) x -= nx;
+        return x;
+    };
     [[maybe_unused]] LogTable logs;
     if constexpr (KP == 1 && MODEL > 0) logs.load();
     V v[9], rho = cst<V>(1.0), f0 = cst<V>(0.0);  // f0: psi (MODEL 0)
@@ -285,15 +290,10 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
         int xl = x0 + c - 1, xa = x0 + c, xb = x0 + c + 1, xr = x0 + c + KP;
         const bool edge = x0 < HC + 1 || x0 + w + HC >= nx;  // (of the tile) some column wraps
         if (edge) {
-            auto wrap = [nx](int x) {
-                while (x < 0) x += nx;
-                while (x >= nx) x -= nx;
-                return x;
-            };
-            xl = wrap(xl);
-            xa = wrap(xa);
-            xb = wrap(xb);
-            xr = wrap(xr);
+            xl = wrap_column(xl);
+            xa = wrap_column(xa);
+            xb = wrap_column(xb);
+            xr = wrap_column(xr);
         }
         if constexpr (NEAR) {
             const unsigned row = 4u * nx, o0 = yr * row + 4u * xa;
@@ -380,8 +380,13 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
     V fx = cst<V>(P.fx), fy = cst<V>(P.fy);
     [[maybe_unused]] real rave = real(0);
     [[maybe_unused]] auto drive = [&]() {
-        const int gx = x0 + c;
-        const real al = gx <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi, ah = gx + 1 <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi;
+        // the side is that of the lattice column: in the full model the halo lanes' velocities take the force too
+        int ga = x0 + c, gb = ga + 1;
+        if constexpr (MODEL == 2) {
+            ga = wrap_column(ga);
+            gb = wrap_column(gb);
+        }
+        const real al = ga <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi, ah = gb <= T.D.x_split ? T.D.ax_lo : T.D.ax_hi;
         if constexpr (KP == 1)
             fx = fma(al, fabs(rho - rave), P.fx);
         else
