@@ -332,11 +332,11 @@ static size_t buffer_bytes(int precision, int nx, int ny) {
 }
 
 // Slots of the driven steps' stored mass: strip kernels, one per consumer warp of every strip CTA
-// (strips of at least one row); tile kernel, three sets of accumulators.
+// (strips of at least one row); tile kernel, three sets of accumulators (kDriveSet).
 static size_t drive_mass_slots(int nx, int ny) {
     const size_t pp = (size_t)((nx + kPPPTX - 1) / kPPPTX) * kPPPWarps;
     const size_t fe = (size_t)((nx + kFEPTX - 1) / kFEPTX) * kFEPWarps;
-    return std::max(std::max(pp, fe) * (size_t)ny, (size_t)3 * lbmk::kDriveParts);
+    return std::max(std::max(pp, fe) * (size_t)ny, (size_t)3 * lbmk::kDriveSet);
 }
 
 extern "C" size_t lbm_workspace_bytes(int precision, int nx, int ny) {
@@ -679,22 +679,25 @@ static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int ban
     if (driven) {
         T.driven = true;
         unsigned long long* acc = reinterpret_cast<unsigned long long*>(c->dmass);
-        auto set = [&](int k) { return acc + (k % 3) * lbmk::kDriveParts; };
+        auto set = [&](int k) { return acc + (k % 3) * lbmk::kDriveSet; };
         if (chain > 0) {
             T.D = drive_terms<real>(c);
             T.acc_in = set(chain - 1);
         } else {
             T.D = launch_drive<real>(c, src);
-            CK(cudaMemsetAsync(acc, 0, 3 * lbmk::kDriveParts * sizeof(*acc), c->stream));
+            CK(cudaMemsetAsync(acc, 0, 3 * lbmk::kDriveSet * sizeof(*acc), c->stream));
         }
         T.acc_out = set(chain);
         T.acc_zero = set(chain + 1);
-        // below the packing limit 4 / b = 2^e x, x in [0.5, 1), a density takes at most 49 bits and N of them 61
         int e = 0;
-        std::frexp(4.0 / c->prm.b, &e);
-        const int bits = std::min(49, 61 - (int)std::ceil(std::log2((double)c->nx * c->ny)));
-        T.mass_scale = std::ldexp(1.0, bits - e);
-        T.mass_unit = T.D.inv_cells * (c->prec == LBM_F64 ? 1.0 / T.mass_scale : lbmk::kTileMassUnit * sp.rest_unit);
+        std::frexp(4.0 / c->prm.b, &e);  // the packing limit is below 2^e
+        const int log2_cells = (int)std::ceil(std::log2((double)c->nx * c->ny));
+        const double unit = c->prec == LBM_F64
+                                ? std::ldexp(1.0, e - lbmk::kMassBits)
+                                : std::ldexp(lbm_host::rest_unit(c->prm.b), std::max(0, log2_cells - 21));
+        T.mass_unit = T.D.inv_cells * unit;
+        T.mass_scale = (float)(1.0 / unit);
+        T.mass_base = 1075 + e - lbmk::kMassBits;
     }
     T.rows = band > 0 ? band : choose_tile_rows(c->prec, m, c->nx, c->ny, &T.share);
     CK(lbmk::launch_tile<real>(m, c->walls, static_cast<const real*>(c->f[src]), static_cast<real*>(c->f[src ^ 1]), sp,

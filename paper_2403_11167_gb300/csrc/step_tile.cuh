@@ -52,16 +52,39 @@ struct Tile {
     static constexpr int kCtas = kPer == 1 ? (MODEL == 2 ? 2 : 1) : MODEL == 0 ? 6 : MODEL == 1 ? 4 : 2;
 };
 
-// The stored mass of driven steps: fixed-point numbers added atomically to kDriveParts accumulators.
-// Integer sums are exact in any order and cost no FP64 instructions but the mean's (FP32: with FP64 sums
-// per row a 1024^2 step took 38 us, with these 21 us; FP64: with sums per row that every CTA added up
-// 200 x 100 took 12.0 us, with these 10.1).  Three sets of accumulators take turns: a step reads the set of
-// the step before, adds to its own and zeroes the next one's.  The unit in FP32 is 2^9 rest_unit (2^-29 of
-// the EOS packing limit, at or below the rounding of the densities); in FP64 the power of two that leaves
-// the lattice's sum 61 bits and a cell's 49 at the packing limit, with a factor of 4 above it (mass_scale
-// units per density): the mean's rounding stays below 2^-53 of the limit from about a hundred cells on, and
-// below 2^-50 on a single one.
-constexpr double kTileMassUnit = 512.0;  // in units of rest_unit
+// The stored mass of driven steps: fixed-point numbers added atomically to kDriveParts 64-bit accumulators
+// (FP64: pairs of them, the low 26 bits of every number to one and the rest to the other, so that a cell keeps
+// its bits however many cells there are).  Integer sums are exact in any order and cost no FP64 instructions
+// but the mean's (FP32: with FP64 sums per row a 1024^2 step took 38 us, with these 20 us; FP64: with sums per
+// row that every CTA added up 200 x 100 took 12.0 us, with these 10.1).  Three sets of accumulators take turns:
+// a step reads the set of the step before, adds to its own and zeroes the next one's.  With 2^e the power of
+// two above the EOS packing limit, the range is 2^(e + 3) and the unit 2^(e - 55) in FP64, 2^(e - 39)
+// (rest_unit) in FP32 up to 2^21 cells and 2^21 / N of the cells' precision beyond, where the total needs the
+// bits.  So the mean is within half a unit and the roundings of its scaling of the mean of the densities as
+// the step sums them, in flat phases too, whose cells all round alike; in FP32 up to 2^21 cells a density
+// above 2^(e - 15) is exact.
+constexpr int kMassLow = 26;      // bits of the low accumulators' numbers
+constexpr int kMassBits = 55;     // FP64: the unit is 2^(e - kMassBits)
+constexpr int kMassHeadroom = 3;  // the range is 2^(e + kMassHeadroom): 2^31 cells' total >> kMassLow has 63 bits
+constexpr int kDriveSet = 2 * kDriveParts;  // low (FP32: all), high
+// s in units of 2^(base - 1075), rounded to nearest: the bits of s shifted as an integer
+__device__ __forceinline__ long long mass_fixed(double s, int base) {
+    const long long b = __double_as_longlong(s);
+    const int r = 10 + base - ((__double2hiint(s) >> 20) & 0x7ff);
+    const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const long long k = r > 63 ? 0ll : (long long)(((m << 10) + (1ull << max(r - 1, 0))) >> max(r, 0));
+    return b < 0 ? -k : k;
+}
+
+// (hi 2^kMassLow + lo) unit: the total's leading 63 bits, one conversion and one product (each a rounding)
+__device__ __forceinline__ double mass_mean(long long hi, unsigned long long lo, double unit) {
+    hi += (long long)(lo >> kMassLow);
+    const unsigned low = (unsigned)lo & ((1 << kMassLow) - 1);
+    const int drop = max(0, kMassLow + 1 - __clzll(hi));  // bits beyond the 63
+    const long long t = (long long)((unsigned long long)hi << (kMassLow - drop)) + (low >> drop);
+    const double m = (double)t * unit;
+    return t == 0 ? 0.0 : __hiloint2double(__double2hiint(m) + (drop << 20), __double2loint(m));
+}
 
 // What a tile step takes besides StepParams: the full model's terms, the walls' solved J_y, and the
 // drive: the state's mass is the sum of D.parts or of the accumulators acc_in.
@@ -76,7 +99,9 @@ struct TileArgs {
     const real* wjy;
     bool driven;
     Drive<real> D;
-    double mass_unit, mass_scale;  // the accumulators' unit as a mean density; FP64: units per density
+    double mass_unit;  // the accumulators' unit as a mean density
+    float mass_scale;  // FP32: 1 / unit
+    int mass_base;     // FP64: mass_fixed's
     const unsigned long long* acc_in;
     unsigned long long *acc_out, *acc_zero;
 };
@@ -266,15 +291,18 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
         if (warp == 0) {
             double m;
             if (T.acc_in) {
-                unsigned long long s = T.acc_in[lane];
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                m = (double)(long long)s * T.mass_unit;
+                unsigned long long lo = T.acc_in[lane], hi = KP == 1 ? T.acc_in[kDriveParts + lane] : 0ull;
+                for (int o = 16; o > 0; o >>= 1) {
+                    lo += __shfl_xor_sync(0xffffffffu, lo, o);
+                    if (KP == 1) hi += __shfl_xor_sync(0xffffffffu, hi, o);
+                }
+                m = KP == 1 ? mass_mean((long long)hi, lo, T.mass_unit) : (double)(long long)lo * T.mass_unit;
             } else {
                 m = drive_mean(T.D);
             }
             if (lane == 0) s_rave = (real)m;
         }
-        if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = 0ull;
+        if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = T.acc_zero[kDriveParts + lane] = 0ull;
     }
 
     [[maybe_unused]] auto wrap_column = [nx](int x) {
@@ -493,7 +521,9 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
     }
 
     if constexpr (DRIVE) {
-        // the mass this warp stored
+        // the mass this warp stored, summed in pieces of 26 bits
+        constexpr unsigned kMask = (1u << kMassLow) - 1;
+        unsigned long long* acc = T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts;
         if constexpr (KP == 1) {
             double s = (v[5] + v[7]) + (v[6] + v[8]);
             if (SHARE && role >= 0) {
@@ -503,22 +533,20 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
                 s = E.x[128];
             }
             s = v[0] + (((v[1] + v[3]) + (v[2] + v[4])) + s);
-            // in the low bits of s scale + 1.5 2^52; summed over the warp in two halves
-            const long long k = __double_as_longlong(fma(s, T.mass_scale, 6755399441055744.0)) - 0x4338000000000000ll;
-            const int lo = __reduce_add_sync(0xffffffffu, out_a ? (int)(k & 0x3ffffff) : 0);
-            const int hi = __reduce_add_sync(0xffffffffu, out_a ? (int)(k >> 26) : 0);
-            if (lane == 0 && role != 1)
-                atomicAdd(T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts,
-                          (unsigned long long)(((long long)hi << 26) + lo));
+            const long long k = out_a ? mass_fixed(s, T.mass_base) : 0ll;
+            const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)k & kMask);
+            const long long hi = (long long)__reduce_add_sync(0xffffffffu, (int)(k >> 2 * kMassLow)) * (1ll << kMassLow) +
+                                 __reduce_add_sync(0xffffffffu, (unsigned)(k >> kMassLow) & kMask);
+            if (lane == 0 && role != 1) {
+                atomicAdd(acc, (unsigned long long)lo);
+                atomicAdd(acc + kDriveParts, (unsigned long long)hi);
+            }
         } else {
-            const F2 m = sum9_v(v) * F2::c(P.rest_inv * (float)(1.0 / kTileMassUnit));
-            const int k = out_a ? __float2int_rn(m.v.x) : 0, l = out_b ? __float2int_rn(m.v.y) : 0;
-            // each below 2^30: summed over the warp in two 16-bit halves
-            const int lo = __reduce_add_sync(0xffffffffu, (k & 0xffff) + (l & 0xffff));
-            const int hi = __reduce_add_sync(0xffffffffu, (k >> 16) + (l >> 16));
-            if (lane == 0)
-                atomicAdd(T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts,
-                          (unsigned long long)(((long long)hi << 16) + lo));
+            const F2 m = sum9_v(v) * F2::c(T.mass_scale);
+            const long long k = (out_a ? __float2ll_rn(m.v.x) : 0ll) + (out_b ? __float2ll_rn(m.v.y) : 0ll);
+            const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)k & kMask);
+            const int hi = __reduce_add_sync(0xffffffffu, (int)(k >> kMassLow));
+            if (lane == 0) atomicAdd(acc, (unsigned long long)((long long)hi * (1ll << kMassLow) + lo));
         }
     }
     if constexpr (KP == 1) {
