@@ -697,6 +697,7 @@ static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int ban
                                 : std::ldexp(lbm_host::rest_unit(c->prm.b), std::max(0, log2_cells - 21));
         T.mass_unit = T.D.inv_cells * unit;
         T.mass_scale = (float)(1.0 / unit);
+        T.mass_range = (float)(std::ldexp(1.0, e + lbmk::kMassHeadroom) / unit);
         T.mass_base = 1075 + e - lbmk::kMassBits;
     }
     T.rows = band > 0 ? band : choose_tile_rows(c->prec, m, c->nx, c->ny, &T.share);

@@ -62,18 +62,20 @@ struct Tile {
 // (rest_unit) in FP32 up to 2^21 cells and 2^21 / N of the cells' precision beyond, where the total needs the
 // bits.  So the mean is within half a unit and the roundings of its scaling of the mean of the densities as
 // the step sums them, in flat phases too, whose cells all round alike; in FP32 up to 2^21 cells a density
-// above 2^(e - 15) is exact.
+// above 2^(e - 15) is exact.  A cell whose mass is not a number of that range (a diverged lattice) is counted
+// in a third word and makes the mean NaN, as a sum in floating point would.
 constexpr int kMassLow = 26;      // bits of the low accumulators' numbers
 constexpr int kMassBits = 55;     // FP64: the unit is 2^(e - kMassBits)
 constexpr int kMassHeadroom = 3;  // the range is 2^(e + kMassHeadroom): 2^31 cells' total >> kMassLow has 63 bits
-constexpr int kDriveSet = 2 * kDriveParts;  // low (FP32: all), high
-// s in units of 2^(base - 1075), rounded to nearest: the bits of s shifted as an integer
-__device__ __forceinline__ long long mass_fixed(double s, int base) {
+constexpr int kDriveSet = 3 * kDriveParts;  // low (FP32: all), high, warps with a cell out of range
+// s in units of 2^(base - 1075), rounded to nearest: the bits of s shifted as an integer; false out of range
+__device__ __forceinline__ bool mass_fixed(double s, int base, long long& out) {
     const long long b = __double_as_longlong(s);
     const int r = 10 + base - ((__double2hiint(s) >> 20) & 0x7ff);
     const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
     const long long k = r > 63 ? 0ll : (long long)(((m << 10) + (1ull << max(r - 1, 0))) >> max(r, 0));
-    return b < 0 ? -k : k;
+    out = b < 0 ? -k : k;
+    return r >= 10 - (kMassBits + kMassHeadroom - 53);
 }
 
 // (hi 2^kMassLow + lo) unit: the total's leading 63 bits, one conversion and one product (each a rounding)
@@ -100,7 +102,7 @@ struct TileArgs {
     bool driven;
     Drive<real> D;
     double mass_unit;  // the accumulators' unit as a mean density
-    float mass_scale;  // FP32: 1 / unit
+    float mass_scale, mass_range;  // FP32: 1 / unit, and the range in units
     int mass_base;     // FP64: mass_fixed's
     const unsigned long long* acc_in;
     unsigned long long *acc_out, *acc_zero;
@@ -292,17 +294,20 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
             double m;
             if (T.acc_in) {
                 unsigned long long lo = T.acc_in[lane], hi = KP == 1 ? T.acc_in[kDriveParts + lane] : 0ull;
+                const bool bad = __any_sync(0xffffffffu, T.acc_in[2 * kDriveParts + lane] != 0);
                 for (int o = 16; o > 0; o >>= 1) {
                     lo += __shfl_xor_sync(0xffffffffu, lo, o);
                     if (KP == 1) hi += __shfl_xor_sync(0xffffffffu, hi, o);
                 }
                 m = KP == 1 ? mass_mean((long long)hi, lo, T.mass_unit) : (double)(long long)lo * T.mass_unit;
+                if (bad) m = __longlong_as_double(-1ll);  // NaN
             } else {
                 m = drive_mean(T.D);
             }
             if (lane == 0) s_rave = (real)m;
         }
-        if (blockIdx.x == 0 && by == 0 && warp == 1) T.acc_zero[lane] = T.acc_zero[kDriveParts + lane] = 0ull;
+        if (blockIdx.x == 0 && by == 0 && warp == 1)
+            T.acc_zero[lane] = T.acc_zero[kDriveParts + lane] = T.acc_zero[2 * kDriveParts + lane] = 0ull;
     }
 
     [[maybe_unused]] auto wrap_column = [nx](int x) {
@@ -523,6 +528,7 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
     if constexpr (DRIVE) {
         // the mass this warp stored, summed in pieces of 26 bits
         constexpr unsigned kMask = (1u << kMassLow) - 1;
+        bool bad;
         unsigned long long* acc = T.acc_out + (unsigned)(by * 8 + blockIdx.x * 3 + warp) % kDriveParts;
         if constexpr (KP == 1) {
             double s = (v[5] + v[7]) + (v[6] + v[8]);
@@ -533,7 +539,9 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
                 s = E.x[128];
             }
             s = v[0] + (((v[1] + v[3]) + (v[2] + v[4])) + s);
-            const long long k = out_a ? mass_fixed(s, T.mass_base) : 0ll;
+            long long k;
+            bad = !mass_fixed(s, T.mass_base, k) && out_a;
+            if (!out_a) k = 0;
             const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)k & kMask);
             const long long hi = (long long)__reduce_add_sync(0xffffffffu, (int)(k >> 2 * kMassLow)) * (1ll << kMassLow) +
                                  __reduce_add_sync(0xffffffffu, (unsigned)(k >> kMassLow) & kMask);
@@ -543,11 +551,13 @@ __global__ void __launch_bounds__(Tile<real, MODEL>::kThreads,
             }
         } else {
             const F2 m = sum9_v(v) * F2::c(T.mass_scale);
+            bad = (out_a && !(fabsf(m.v.x) < T.mass_range)) || (out_b && !(fabsf(m.v.y) < T.mass_range));
             const long long k = (out_a ? __float2ll_rn(m.v.x) : 0ll) + (out_b ? __float2ll_rn(m.v.y) : 0ll);
             const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)k & kMask);
             const int hi = __reduce_add_sync(0xffffffffu, (int)(k >> kMassLow));
             if (lane == 0) atomicAdd(acc, (unsigned long long)((long long)hi * (1ll << kMassLow) + lo));
         }
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicAdd(acc + 2 * kDriveParts, 1ull);
     }
     if constexpr (KP == 1) {
         if (out_a)

@@ -94,3 +94,26 @@ def test_graph_of_driven_steps(model, precision, A):
             err = pop_err(f, ctx.populations())
             ctx.close()
             assert err < 5e-6, (nx, ny, err)
+
+
+@pytest.mark.parametrize("precision", [F64, F32])
+@pytest.mark.parametrize("model,A", [(PP, 0.0), (FE, 0.0), (FE, 0.1)])
+def test_divergence_reaches_the_mean(model, A, precision):
+    """One cell of negative density (neither psi nor the logarithm exists) turns into NaN at the first step
+    of a graph, two or three columns a step wider at each further one.  Its mean is NaN from the second step
+    on and every force with it, in a graph as in single steps: no cell stays finite."""
+    from paper_2403_11167_gb300 import lbm
+
+    nx, ny = 500, 20
+    for steps in ([64], [1] * 64):
+        ctx, rp, th = gpu_context(model, precision, nx, ny, a=0.25, Tr=0.85, tau_nu=0.9, **({"A": A} if A else {}))
+        ctx.set_density(inputs.random_field(nx, ny, th.rho_v * 1.5, th.rho_l * 0.8, seed=5))
+        f = ctx.populations()
+        f[:, 7, 9] *= -0.5
+        ctx.set_populations(f)
+        ctx.set_drive(5e-4, -3e-4, nx // 2, -1)
+        for n in steps:
+            ctx.step(n)
+        assert np.all(np.isnan(ctx.populations().sum(0)))
+        assert ctx.observables(0)["status"] == lbm.LBM_ERR_DIVERGED
+        ctx.close()
