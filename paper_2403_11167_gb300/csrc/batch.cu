@@ -84,9 +84,13 @@ struct BatchItem {
 
 size_t a256(size_t n) { return (n + 255) & ~size_t(255); }
 
-// The size rule of resident lattices: 11 floats and an int16 per cell within kResidentSmemMax (the kernel
-// keeps 9 floats per cell in shared memory).
-size_t resident_bytes(size_t N) { return 11 * N * sizeof(float) + ((2 * N + 15) & ~size_t(15)); }
+// The size rule of resident lattices: 11 floats and an int16 per cell within kResidentSmemMax, that is up to
+// kResidentCells (the kernel keeps 9 floats per cell in shared memory).
+constexpr size_t resident_bytes(size_t N) { return 11 * N * sizeof(float) + ((2 * N + 15) & ~size_t(15)); }
+constexpr int kResidentCells = 4452;
+static_assert(resident_bytes(kResidentCells) <= kResidentSmemMax && resident_bytes(kResidentCells + 1) > kResidentSmemMax,
+              "the largest resident lattice");
+constexpr size_t resident_smem(int cells) { return 9 * sizeof(float) * (size_t)((cells + 3) & ~3); }
 
 // One population buffer of a lattice: 9 FP32 planes plus the int16 rest plane (plane 9).
 size_t buffer_bytes(long long pitch) { return a256(10 * (size_t)pitch * 4); }
@@ -583,10 +587,11 @@ ResidentKernel resident_kernel(int pairs, bool even, int threads) {
 int resident_threads(int cells, int pairs) { return ((cells + 1) / 2 + 32 * pairs - 1) / (32 * pairs) * 32; }
 
 int launch_resident(const lbm_batch* b, const ResidentGroup& g, int step_limit) {
-    const size_t smem = 9 * sizeof(float) * (size_t)((g.max_cells + 3) & ~3);
     const ResidentKernel k = resident_kernel(g.pairs, g.even, g.threads);
-    BCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<(unsigned)g.ids.size(), g.threads, smem, g.stream>>>(b->d_lat, g.d_ids, step_limit);
+    // the limit belongs to the kernel, not to this launch: the same for every batch, since a smaller batch on
+    // another thread would lower it under this launch
+    BCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resident_smem(kResidentCells)));
+    k<<<(unsigned)g.ids.size(), g.threads, resident_smem(g.max_cells), g.stream>>>(b->d_lat, g.d_ids, step_limit);
     BCK(cudaGetLastError());
     return LBM_OK;
 }

@@ -1,0 +1,54 @@
+"""Batches at the edges of what a process and a device hold: several host threads, device memory."""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_2403_11167_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_2403_11167_gb300 import lbm as L
+
+    return L
+
+
+def _spec(lbm, nx, ny, nsteps, seed):
+    p = lbm.lbm_params_default(lbm.LBM_PSEUDOPOTENTIAL, precision=lbm.LBM_F32, a=0.25, Tr=0.85, tau_nu=0.8)
+    _, th = lbm.lbm_resolve_params(p)
+    return (dict(nx=nx, ny=ny, geometry=0, nsteps=nsteps, params=p),
+            inputs.spinodal_noise(nx, ny, 0.5 * (th.rho_l + th.rho_v), 0.01, seed=seed))
+
+
+def test_threads_with_resident_batches_of_different_sizes(lbm):
+    """Two host threads run batches whose resident lattices need the same kernel with different amounts of
+    shared memory, 3000 times each: no launch of either is refused, and the states are those of one thread."""
+    sizes = [(64, 64), (48, 50)]
+    batches = [lbm.Batch(*zip(_spec(lbm, nx, ny, 2, seed=nx))) for nx, ny in sizes]
+    for b in batches:
+        b.run()
+    want = [b.populations(0) for b in batches]
+    errors = []
+
+    def work(b):
+        try:
+            for _ in range(3000):
+                b.run()
+        except Exception as e:  # noqa: BLE001 (reported below)
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(b,)) for b in batches]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for b, w in zip(batches, want):
+        assert np.array_equal(b.populations(0), w)
+        b.close()
