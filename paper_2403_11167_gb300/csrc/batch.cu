@@ -70,7 +70,7 @@ struct BatchLattice {
     lbmk::StepParams<float> P;  // physics and geometry (nx, ny, rows, pitch)
     float* buf[2];              // ping-pong stored populations
     float* scratch;             // 2 N floats: rho and psi for observables
-    double* rho0;               // N initial densities
+    double* rho0;               // N initial densities (of their own, or in scratch: lbm_batch::rho0)
     double RT, a, b4;           // FP64 EOS constants for the observables (pressure jump)
     int nsteps;
     int geometry;
@@ -530,6 +530,7 @@ struct lbm_batch {
     int2* d_runs;
     int* d_first;                           // each lattice's first run (n + 1)
     double* d_sums;                         // kRunSums per run
+    std::vector<std::vector<double>> rho0;  // initial densities, where the device cannot hold them between runs
     cudaEvent_t ready;                      // the initial state is there (for the resident groups)
 };
 
@@ -547,6 +548,9 @@ std::mutex g_tune_mu;
 // f^eq(rho0) for every lattice and the clock at 0, enqueued behind whatever ran before.
 int batch_init_state(lbm_batch* b) {
     BCK(cudaMemsetAsync(b->d_err, 0, sizeof(int) * 16, b->s_tile));
+    for (size_t i = 0; i < b->rho0.size(); ++i)
+        BCK(cudaMemcpyAsync(b->lat[i].rho0, b->rho0[i].data(), sizeof(double) * b->rho0[i].size(),
+                            cudaMemcpyHostToDevice, b->s_tile));
     if (b->d_order) lbmk::batch_clock_kernel<<<1, 32, 0, b->s_tile>>>(b->d_step, -1, b->d_order, (int)b->order.size());
     lbmk::batch_init_kernel<<<(unsigned)b->runs.size(), 256, 0, b->s_tile>>>(b->d_lat, b->d_runs);
     BCK(cudaGetLastError());
@@ -562,7 +566,8 @@ int upload_state(lbm_batch* b, const double* const* rho0) {
         const int cells = b->lat[i].P.nx * b->lat[i].P.ny;
         first.push_back((int)b->runs.size());
         for (int c = 0; c < cells; c += lbmk::kRunCells) b->runs.push_back(make_int2(i, c));
-        BCK(cudaMemcpyAsync(b->lat[i].rho0, rho0[i], sizeof(double) * (size_t)cells, cudaMemcpyHostToDevice, b->s_tile));
+        if (b->rho0.empty())
+            BCK(cudaMemcpyAsync(b->lat[i].rho0, rho0[i], sizeof(double) * (size_t)cells, cudaMemcpyHostToDevice, b->s_tile));
     }
     first.push_back((int)b->runs.size());
     BCK(cudaMalloc(&b->d_runs, sizeof(int2) * b->runs.size()));
@@ -866,7 +871,6 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     b->spec.assign(specs, specs + n);
     b->lat.resize(n);
     // resolve parameters and validate on the host first
-    size_t pool_bytes = 0;
     std::vector<size_t> offs(n);
     b->max_tiled_steps = 0;
     std::vector<lbm_params> in_p(n), res_p(n);
@@ -937,12 +941,27 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
             return LBM_ERR_UNSUPPORTED;  // tiled lattices use the TMA strip kernels
         }
         if (!L.resident) b->max_tiled_steps = std::max(b->max_tiled_steps, L.nsteps);
-        offs[i] = pool_bytes;
-        pool_bytes += 2 * buffer_bytes(P.pitch) + a256(2 * N * 4 + 8 * N);
     }
-    const size_t tail = pool_bytes;
-    pool_bytes += a256(sizeof(BatchLattice) * n) + 256 + 256 + a256(8 * sizeof(double) * n);
-    cudaError_t e = cudaMalloc(&b->pool, pool_bytes);
+    // Two buffers, the scratch and the initial densities of every lattice; where the device has no room for
+    // the last (8 of 96 bytes per cell), they stay on the host and go to the scratch before each run.
+    size_t tail = 0;
+    auto allocate = [&](bool keep_rho0) {
+        size_t bytes = 0;
+        for (int i = 0; i < n; ++i) {
+            const size_t N = (size_t)specs[i].nx * specs[i].ny;
+            offs[i] = bytes;
+            bytes += 2 * buffer_bytes(b->lat[i].P.pitch) + a256(2 * N * 4 + (keep_rho0 ? 8 * N : 0));
+        }
+        tail = bytes;
+        bytes += a256(sizeof(BatchLattice) * n) + 256 + 256 + a256(8 * sizeof(double) * n);
+        return cudaMalloc(&b->pool, bytes);
+    };
+    cudaError_t e = allocate(true);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();  // (not an error of the calls below)
+        for (int i = 0; i < n; ++i) b->rho0.emplace_back(rho0[i], rho0[i] + (size_t)specs[i].nx * specs[i].ny);
+        e = allocate(false);
+    }
     if (e != cudaSuccess) {
         delete b;
         return bfail(e, "cudaMalloc(batch pool)");
@@ -953,7 +972,7 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
         L.buf[0] = reinterpret_cast<float*>(b->pool + offs[i]);
         L.buf[1] = reinterpret_cast<float*>(b->pool + offs[i] + fb);
         L.scratch = reinterpret_cast<float*>(b->pool + offs[i] + 2 * fb);
-        L.rho0 = reinterpret_cast<double*>(L.scratch + 2 * (size_t)L.P.nx * L.P.ny);
+        L.rho0 = reinterpret_cast<double*>(L.scratch + (b->rho0.empty() ? 2 * (size_t)L.P.nx * L.P.ny : 0));
     }
     b->d_lat = reinterpret_cast<BatchLattice*>(b->pool + tail);
     b->d_step = reinterpret_cast<int*>(b->pool + tail + a256(sizeof(BatchLattice) * n));

@@ -52,3 +52,32 @@ def test_threads_with_resident_batches_of_different_sizes(lbm):
     for b, w in zip(batches, want):
         assert np.array_equal(b.populations(0), w)
         b.close()
+
+
+def test_batch_that_fills_the_device(lbm):
+    """With room for the buffers and the scratch (88 bytes per cell) but not for the initial densities too
+    (96), a batch still runs, and runs again, to the bits of one with room."""
+    import torch
+
+    nx, ny = 8192, 4096
+    specs, rhos = zip(_spec(lbm, nx, ny, 3, seed=1), _spec(lbm, 40, 40, 3, seed=2))
+
+    def outputs():
+        b = lbm.Batch(specs, rhos)
+        out = []
+        for _ in range(2):
+            b.run()
+            out.append((b.observables(), b.populations(0), b.populations(1)))
+        b.close()
+        return out
+
+    want = outputs()
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - 92 * nx * ny, dtype=torch.uint8, device="cuda")
+    got = outputs()
+    del hold
+    torch.cuda.empty_cache()
+    for g, w in zip(got, want):
+        assert repr(g[0]) == repr(w[0])
+        assert np.array_equal(g[1], w[1]) and np.array_equal(g[2], w[2])
