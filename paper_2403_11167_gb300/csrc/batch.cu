@@ -347,18 +347,26 @@ __global__ void batch_clock_kernel(int* state, int by, const int2* __restrict__ 
     }
 }
 
-// Cells of every lattice in runs of kRunCells, one CTA each (lat, first cell): the kernels off the step
+// Cells of every lattice in runs of kRunCells, one CTA each (lattice, run of it): the kernels off the step
 // path work on these, so that a 512 x 512 lattice does not wait for one CTA (observables of the 96-lattice
 // sweep: 1.25 ms with a CTA per lattice, 0.33 with these).
-constexpr int kRunCells = 2048;
+constexpr unsigned kRunCells = 2048;
+// The cells of a run, [first, end) of N.  32-bit numbers without sign: a lattice that fits the device has
+// less than 2^32 cells (88 bytes each), but may have more than 2^31.
+struct Run {
+    unsigned N, first, end;
+    __device__ __forceinline__ Run(int2 run, int nx, int ny)
+        : N((unsigned)nx * (unsigned)ny), first((unsigned)run.y * kRunCells), end(first + min(kRunCells, N - first)) {}
+};
 
 // f = f^eq(rho0, u = 0) of every lattice from its initial densities on the device.
 __global__ void __launch_bounds__(256)
     batch_init_kernel(const BatchLattice* __restrict__ lats, const int2* __restrict__ runs) {
     const int2 run = runs[blockIdx.x];
     const BatchLattice& L = lats[run.x];
-    const int nx = L.P.nx, ny = L.P.ny, end = min(run.y + kRunCells, nx * ny);
-    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x)
+    const int nx = L.P.nx, ny = L.P.ny;
+    const Run R(run, nx, ny);
+    for (long long c = R.first + threadIdx.x; c < R.end; c += blockDim.x)
         init_cell(L.rho0, L.buf[0], LBM_PSEUDOPOTENTIAL, nx, ny, L.P.pitch, L.P.rest_inv, c);
 }
 
@@ -370,14 +378,17 @@ __global__ void __launch_bounds__(256)
     const int2 run = runs[blockIdx.x];
     const BatchLattice& L = lats[run.x];
     const StepParams<float> P = L.P;
-    const int nx = P.nx, ny = P.ny, N = nx * ny, end = min(run.y + kRunCells, N);
+    const int nx = P.nx, ny = P.ny;
+    const Run R(run, nx, ny);
     const float* f = L.buf[L.nsteps & 1];
-    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x) {
+    float* psi = L.scratch + R.N;
+    for (unsigned k = threadIdx.x; k < R.end - R.first; k += blockDim.x) {
+        const unsigned c = R.first + k;
         float v[9];
-        pull_cell(f, P.pitch, c % nx, c / nx, nx, ny, v);
+        pull_cell(f, P.pitch, (int)(c % nx), (int)(c / nx), nx, ny, v);
         const float r = sum9_rest(v, rest_lo_plane(f, P.pitch)[c], P);
         L.scratch[c] = r;
-        L.scratch[N + c] = pseudo_psi(r, P);
+        psi[c] = pseudo_psi(r, P);
     }
 }
 
@@ -387,13 +398,15 @@ __global__ void __launch_bounds__(256)
     const int2 run = runs[blockIdx.x];
     const BatchLattice& L = lats[run.x];
     const StepParams<float> P = L.P;
-    const int nx = P.nx, ny = P.ny, N = nx * ny, end = min(run.y + kRunCells, N);
+    const int nx = P.nx, ny = P.ny;
+    const Run R(run, nx, ny);
     const float* f = L.buf[L.nsteps & 1];
     const float* rho = L.scratch;
-    const float* ps = L.scratch + N;
+    const float* ps = L.scratch + R.N;
     double m = 0.0, u2 = 0.0, bad = 0.0, liq = 0.0, vap = 0.0, dmax = 0.0;
-    for (int c = run.y + threadIdx.x; c < end; c += blockDim.x) {
-        const int x = c % nx, y = c / nx;
+    for (unsigned k = threadIdx.x; k < R.end - R.first; k += blockDim.x) {
+        const unsigned c = R.first + k;
+        const int x = (int)(c % nx), y = (int)(c / nx);
         float v[9], an[9];
         pull_cell(f, P.pitch, x, y, nx, ny, v);
         gather8(ps, x, y, nx, ny, an);
@@ -419,7 +432,8 @@ __global__ void __launch_bounds__(256)
         }
         const int prow = L.geometry == 0 ? 0 : ny / 2;
         if (y == prow) {
-            const double a = rho[y * nx + (x == nx - 1 ? 0 : x + 1)], b = rho[y * nx + (x == 0 ? nx - 1 : x - 1)];
+            const float* row = rho + (size_t)y * nx;
+            const double a = row[x == nx - 1 ? 0 : x + 1], b = row[x == 0 ? nx - 1 : x - 1];
             dmax = fmax(dmax, fabs(a - b) * 0.5);
         }
     }
@@ -455,7 +469,8 @@ __global__ void __launch_bounds__(32)
     batch_obs_kernel(const BatchLattice* __restrict__ lats, const int* __restrict__ first,
                      const double* __restrict__ sums, double* __restrict__ out) {
     const BatchLattice& L = lats[blockIdx.x];
-    const int nx = L.P.nx, ny = L.P.ny, N = nx * ny, lane = threadIdx.x;
+    const int nx = L.P.nx, ny = L.P.ny, lane = threadIdx.x;
+    const unsigned N = (unsigned)nx * (unsigned)ny;
     double s[kRunSums] = {0, 0, 0, 0, 0, 0};
     for (int r = first[blockIdx.x] + lane; r < first[blockIdx.x + 1]; r += 32)
         for (int j = 0; j < kRunSums; ++j) {
@@ -526,7 +541,7 @@ struct lbm_batch {
     cudaStream_t s_tile;
     cudaGraphExec_t chunk[2];            // kChunk steps with strips, with tiles
     bool ran;
-    std::vector<int2> runs;                 // cells in runs of kRunCells: lattice, first cell
+    std::vector<int2> runs;                 // cells in runs of kRunCells: lattice, run of it
     int2* d_runs;
     int* d_first;                           // each lattice's first run (n + 1)
     double* d_sums;                         // kRunSums per run
@@ -563,11 +578,11 @@ int batch_init_state(lbm_batch* b) {
 int upload_state(lbm_batch* b, const double* const* rho0) {
     std::vector<int> first;
     for (int i = 0; i < b->n; ++i) {
-        const int cells = b->lat[i].P.nx * b->lat[i].P.ny;
+        const size_t cells = (size_t)b->lat[i].P.nx * b->lat[i].P.ny;
         first.push_back((int)b->runs.size());
-        for (int c = 0; c < cells; c += lbmk::kRunCells) b->runs.push_back(make_int2(i, c));
+        for (size_t c = 0; c < cells; c += lbmk::kRunCells) b->runs.push_back(make_int2(i, (int)(c / lbmk::kRunCells)));
         if (b->rho0.empty())
-            BCK(cudaMemcpyAsync(b->lat[i].rho0, rho0[i], sizeof(double) * (size_t)cells, cudaMemcpyHostToDevice, b->s_tile));
+            BCK(cudaMemcpyAsync(b->lat[i].rho0, rho0[i], sizeof(double) * cells, cudaMemcpyHostToDevice, b->s_tile));
     }
     first.push_back((int)b->runs.size());
     BCK(cudaMalloc(&b->d_runs, sizeof(int2) * b->runs.size()));
@@ -609,8 +624,9 @@ int build_groups(lbm_batch* b) {
         g.even = cls % 2 == 0;
         const int hi = 1152 << cls / 2, lo = cls < 2 ? 0 : hi / 2;
         for (int i = 0; i < b->n; ++i) {
+            if (!b->lat[i].resident) continue;
             const int nx = b->lat[i].P.nx, cells = nx * b->lat[i].P.ny;
-            if (b->lat[i].resident && (nx % 2 == 0) == g.even && cells > lo && cells <= hi) {
+            if ((nx % 2 == 0) == g.even && cells > lo && cells <= hi) {
                 g.ids.push_back(i);
                 g.max_cells = std::max(g.max_cells, cells);
             }
