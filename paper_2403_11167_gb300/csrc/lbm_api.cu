@@ -104,7 +104,8 @@ struct lbm_ctx {
     double* partials;    // kRedBlocks x 3
     double* d_obs;       // 8 doubles
     int* d_err;          // device error word of the TMA kernels (bounded waits)
-    bool use_tma;
+    bool use_tma;        // the strip kernels can run (strip_step says where they do)
+    bool strips;         // ... and run whatever the size (LBM_STRIPS set: route comparisons)
     bool walls;          // no-slip walls on rows 0 and ny-1 (mirrored or one-sided)
     bool onesided;       // free-energy walls with the one-sided normal mu gradient (LBM_BC_WALL_ZOUHE_ONESIDED)
     void* wall;          // 14 nx reals: the wall rows' J_y and solve scratch (fe_wall_solve_kernel)
@@ -523,6 +524,7 @@ extern "C" int lbm_create(const lbm_params* p, int nx, int ny, int bc_x, int bc_
     // walls: the periodic strip kernels serve the interior when both wall bands fit
     c->use_tma = (!walls || ny >= 2 * kWallBandFE) && c->prec == LBM_F32 && nx % 4 == 0 && nx >= 8 && ny >= 4 &&
                  std::getenv("LBM_NO_TMA") == nullptr;
+    c->strips = std::getenv("LBM_STRIPS") != nullptr;
     cudaError_t e = cudaMallocHost(&c->h_pinned, 8 * sizeof(double));
     if (e != cudaSuccess) {
         if (c->own_ws) cudaFree(c->ws);
@@ -718,7 +720,7 @@ static int launch_tile_step(lbm_ctx* c, int src, bool driven, int chain, int ban
 //   drive (FE)             1664^2  59.1, 61.3   1792^2  67.3, 65.2
 static bool strip_step(const lbm_ctx* c, bool driven) {
     if (!c->use_tma) return false;
-    const long long cells = (long long)c->nx * c->ny;
+    const long long cells = c->strips ? 1LL << 31 : (long long)c->nx * c->ny;
     if (uses_iwb(c)) return cells >= 2800000 && !c->walls && !driven && (!c->grav || c->rho_g == 0.0);
     const bool pp = c->prm.model == LBM_PSEUDOPOTENTIAL;
     if (driven) return cells >= (pp ? 2500000 : 3100000);
