@@ -150,8 +150,9 @@ int lbm_resolve_params_many(int n, const lbm_params* in, lbm_params* out, lbm_th
 
 /* Bytes of device workspace a context of this size and precision needs: two population
  * buffers (nine planes, plus the rest-population extension plane for FP32), four fields for
- * the observables, reduction partials, the one-sided walls' row solve (14 nx reals) and one
- * double per strip warp or tile row for the droplet-collision drive's stored mass (Sec. 5.4). */
+ * the observables, reduction partials, the one-sided walls' row solve (14 nx reals) and the
+ * droplet-collision drive's stored mass (Sec. 5.4): three sets of 96 integers of 8 bytes, or one
+ * double per strip warp where that is more (FP32 with nx a multiple of 4). */
 size_t lbm_workspace_bytes(int precision, int nx, int ny);
 
 /* Create a context for an nx x ny lattice (nx, ny >= 1).  Boundaries: bc_x must be

@@ -109,7 +109,7 @@ struct lbm_ctx {
     bool walls;          // no-slip walls on rows 0 and ny-1 (mirrored or one-sided)
     bool onesided;       // free-energy walls with the one-sided normal mu gradient (LBM_BC_WALL_ZOUHE_ONESIDED)
     void* wall;          // 14 nx reals: the wall rows' J_y and solve scratch (fe_wall_solve_kernel)
-    double* dmass;       // stored mass of the driven steps by warp (drive_mass_slots)
+    double* dmass;       // stored mass of the driven steps: by strip warp, or the tiles' accumulators (drive_mass_slots)
     bool drive;          // droplet-collision drive configured (lbm_set_drive)
     bool grav;           // gravity configured (lbm_set_gravity; free-energy model)
     double g, rho_g, y_ref;
@@ -332,12 +332,19 @@ static size_t buffer_bytes(int precision, int nx, int ny) {
     return align256((precision == LBM_F64 ? 9 : 10) * (size_t)plane_pitch(nx, ny) * esz);
 }
 
-// Slots of the driven steps' stored mass: strip kernels, one per consumer warp of every strip CTA
-// (strips of at least one row); tile kernel, three sets of accumulators (kDriveSet).
-static size_t drive_mass_slots(int nx, int ny) {
+// Lattices whose rows the strip kernels can copy (FP32; the TMA's 16-byte rule).
+static bool strip_rows_copyable(int precision, int nx, int ny) {
+    return precision == LBM_F32 && nx % 4 == 0 && nx >= 8 && ny >= 4;
+}
+
+// 8-byte slots of the driven steps' stored mass: tile kernel, three sets of accumulators (kDriveSet); strip
+// kernels, where they can run, one per consumer warp of every strip CTA (strips of at least one row).
+static size_t drive_mass_slots(int precision, int nx, int ny) {
+    const size_t tiles = 3 * lbmk::kDriveSet;
+    if (!strip_rows_copyable(precision, nx, ny)) return tiles;
     const size_t pp = (size_t)((nx + kPPPTX - 1) / kPPPTX) * kPPPWarps;
     const size_t fe = (size_t)((nx + kFEPTX - 1) / kFEPTX) * kFEPWarps;
-    return std::max(std::max(pp, fe) * (size_t)ny, (size_t)3 * lbmk::kDriveSet);
+    return std::max(std::max(pp, fe) * (size_t)ny, tiles);
 }
 
 extern "C" size_t lbm_workspace_bytes(int precision, int nx, int ny) {
@@ -348,7 +355,7 @@ extern "C" size_t lbm_workspace_bytes(int precision, int nx, int ny) {
     const size_t fields = align256(4 * n * esz);
     // ... + the one-sided walls' row solve (14 nx reals) + the drive's mass slots
     return 2 * fbytes + fields + align256(kRedBlocks * 3 * sizeof(double)) + align256(8 * sizeof(double)) + 256 +
-           align256(14 * (size_t)nx * esz) + align256(drive_mass_slots(nx, ny) * sizeof(double));
+           align256(14 * (size_t)nx * esz) + align256(drive_mass_slots(precision, nx, ny) * sizeof(double));
 }
 
 template <typename real>
@@ -522,7 +529,7 @@ extern "C" int lbm_create(const lbm_params* p, int nx, int ny, int bc_x, int bc_
     c->walls = walls;
     c->onesided = bc_y == LBM_BC_WALL_ZOUHE_ONESIDED && p->model == LBM_FREE_ENERGY;
     // walls: the periodic strip kernels serve the interior when both wall bands fit
-    c->use_tma = (!walls || ny >= 2 * kWallBandFE) && c->prec == LBM_F32 && nx % 4 == 0 && nx >= 8 && ny >= 4 &&
+    c->use_tma = (!walls || ny >= 2 * kWallBandFE) && strip_rows_copyable(c->prec, nx, ny) &&
                  std::getenv("LBM_NO_TMA") == nullptr;
     c->strips = std::getenv("LBM_STRIPS") != nullptr;
     cudaError_t e = cudaMallocHost(&c->h_pinned, 8 * sizeof(double));
