@@ -188,7 +188,7 @@ __device__ __forceinline__ F2 fmav(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 
 // Reciprocal: the hardware approximation and one Newton step r + r (1 - x r) in fused
 // multiply-adds (Markstein 1990), which for a normal x with a normal reciprocal is the correctly
-// rounded 1/x (checked against __frcp_rn for every mantissa and exponents -40 .. 40).  The library
+// rounded 1/x (every mantissa and exponents -40 .. 40 in tests/test_gpu_math.py).  The library
 // function adds a range test, a branch and a slow path per lane; here both cells of a lane share
 // the packed step.  With sqrt_v below: P step at 4096^2 239 -> 232 us, FE 263 -> 251 us, full FE
 // at 1024^2 46 -> 42 us, the same bits.  0, infinities and subnormal values give NaN or infinity.
@@ -380,7 +380,7 @@ __device__ __forceinline__ F cs_pressure_v(F rho, const StepParams<float>& P) {
     return fmav(rho * F::c(P.RT) * num, r * r * r, -(F::c(P.a) * rho * rho));
 }
 // Square root g = x r, g + (x - g^2) r / 2 from the hardware's r ~ 1/sqrt(x) (Markstein 1990): for a
-// normal x the correctly rounded root (checked as rcp_v).  The 1e-37 that keeps r finite at x = 0
+// normal x the correctly rounded root (tested as rcp_v).  The 1e-37 that keeps r finite at x = 0
 // (root 0) is below half an ulp of every radicand above 2^-98; a negative x gives NaN.
 __device__ __forceinline__ float rsqrt_approx(float x) {
     float r;

@@ -19,8 +19,10 @@ __device__ __forceinline__ double fmav(double a, double b, double c) { return fm
 __device__ __forceinline__ double abs_v(double a) { return fabs(a); }
 __device__ __forceinline__ double sum9_v(const double v[9]) { return sum9(v); }
 
-// 1/x: the hardware's approximation (relative error e < 2^-20) and one cubic step r (1 + e + e^2),
-// accurate to an ulp for a normal x with a normal reciprocal.
+// 1/x: the hardware's approximation (relative error e < 2^-20) and one step of the third-order iteration
+// r (1 + e + e^2), e = 1 - x r (Chebyshev's, the geometric series cut after two terms), for a normal x with a
+// normal reciprocal: 2^-60 before the last rounding, so correctly rounded but for 3 in 10,000 arguments, and
+// these to an ulp (tests/test_gpu_math.py).
 __device__ __forceinline__ double rcp_d(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -28,11 +30,12 @@ __device__ __forceinline__ double rcp_d(double x) {
     return fma(r, fma(e, e, e), r);
 }
 
-// sqrt(x) by two coupled (Goldschmidt) steps and a residual correction; 0 gives 0, x < 0 NaN.
+// sqrt(x) from the hardware's 1/sqrt(x) by one coupled step (Goldschmidt 1964) and Markstein's (1990) correction
+// by the residual x - g^2; correctly rounded for a normal x.  0 and subnormal numbers give 0, x < 0 NaN.
 __device__ __forceinline__ double sqrt_d(double x) {
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    if (__double2hiint(x) == 0) r = 0.0;  // x = 0 (or subnormal): r is infinite
+    if ((unsigned)__double2hiint(x) < 0x00100000u) r = 0.0;  // below the normal numbers r is infinite
     double g = x * r, h = 0.5 * r;
     const double e = fma(-g, h, 0.5);
     g = fma(g, e, g);
