@@ -209,7 +209,8 @@ int lbm_set_gravity(lbm_ctx* ctx, double g, double rho_ref, double y_ref);
  * Sec. 5.4 uses ax_lo = 5e-6, ax_hi = -5e-6, x_split = 100, t_on = 2000 on a 200 x 100 lattice.
  * Driven steps also sum the populations they store, which is the next state's mass; the
  * reduction over the populations runs only at the first step of each captured 64-step graph and
- * at single steps.  The step kernels differ only in the summation order of rho_ave.  Errors: LBM_ERR_ARG for a non-finite value, LBM_ERR_UNSUPPORTED with walls (the
+ * at single steps.  The step kernels differ only in the rounding of rho_ave.
+ * Errors: LBM_ERR_ARG for a non-finite value, LBM_ERR_UNSUPPORTED with walls (the
  * reduction sums the stored populations of a periodic lattice).  Synchronises the stream. */
 int lbm_set_drive(lbm_ctx* ctx, double ax_lo, double ax_hi, double x_split, long long t_on);
 
@@ -296,8 +297,8 @@ typedef struct lbm_batch lbm_batch;
  * (copied; f starts at f^eq(rho0, u = 0)).  Lattices of up to 4452 cells (11 nx ny floats and nx ny
  * int16 <= 200 KB) run resident: one CTA each, all steps in shared memory and registers, in one
  * persistent launch per size class.  The others run as strips or tiles of a work table, one launch per
- * step for all of them, replayed as 64-step CUDA graphs on a further stream concurrently.  An autotuner picks the resident block size and the strip
- * height by timing short trials (cached per shape class); the state is re-initialised
+ * step for all of them, replayed as 64-step CUDA graphs on a further stream concurrently.  An autotuner
+ * picks the resident block size and the strip height by timing short trials (cached per shape class); the state is re-initialised
  * afterwards.  The library allocates the device memory (one pooled cudaMalloc).
  * Errors: LBM_ERR_ARG (sizes, densities), LBM_ERR_UNSUPPORTED (other model or precision,
  * a tiled lattice with nx % 4 != 0 or nx < 8 or ny < 4), LBM_ERR_CUDA. */

@@ -101,8 +101,9 @@ namespace lbmk {
 
 // ------------------------------------------------------------------------------------
 // Resident lattice: all steps on one SM.  A thread keeps PAIRS pairs of cells for the whole run: their
-// rest populations and extensions stay in its registers, the eight moving populations in shared memory
-// in the stored layout S_i(x) (post-collision at the source cell).  Per step: (A) pull every cell's
+// rest populations and extensions are its own (in registers with one pair; with two 8 to 80 bytes a thread
+// spill to local memory, with four, which lattices above 2048 cells need, 196 to 788), the eight moving
+// populations are in shared memory in the stored layout S_i(x) (post-collision at the source cell).  Per step: (A) pull every cell's
 // populations into registers and write psi; barrier; (B) collide from the neighbours' psi and write f*
 // over S, which every thread has read by then; barrier.  So no population moves through global memory
 // and each step has two barriers.  A pair is two cells of one row when nx is even, so that reads of
