@@ -1018,8 +1018,7 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     return LBM_OK;
 }
 
-extern "C" int lbm_batch_run(lbm_batch* b) {
-    if (!b) return LBM_ERR_ARG;
+static int run_batch(lbm_batch* b) {
     if (b->ran) {
         int rc = batch_init_state(b);
         if (rc) return rc;
@@ -1044,6 +1043,16 @@ extern "C" int lbm_batch_run(lbm_batch* b) {
         BCK(cudaStreamWaitEvent(b->s_tile, g.done, 0));
     }
     return LBM_OK;
+}
+
+extern "C" int lbm_batch_run(lbm_batch* b) {
+    if (!b) return LBM_ERR_ARG;
+    const int rc = run_batch(b);
+    // after a failure on the way the groups already launched are not joined to s_tile: a further run's initial
+    // state must not be written before they have stored their last
+    if (rc)
+        for (const ResidentGroup& g : b->groups) cudaStreamSynchronize(g.stream);
+    return rc;
 }
 
 extern "C" int lbm_batch_observables(lbm_batch* b, lbm_obs* out) {

@@ -1,4 +1,5 @@
 """Batches at the edges of what a process and a device hold: several host threads, device memory."""
+import ctypes
 import threading
 
 import numpy as np
@@ -81,3 +82,32 @@ def test_batch_that_fills_the_device(lbm):
     for g, w in zip(got, want):
         assert repr(g[0]) == repr(w[0])
         assert np.array_equal(g[1], w[1]) and np.array_equal(g[2], w[2])
+
+
+def test_run_after_a_failed_run(lbm):
+    """A run that fails between the resident launch and the tiled one (the caller has left the batch's stream in
+    capture, so its graph cannot be captured) does not spoil the next: the resident kernel of the failed run,
+    20,000 steps long, stores its last state before the next run's initial state is written."""
+    specs, rhos = zip(_spec(lbm, 64, 64, 20000, seed=1), _spec(lbm, 100, 60, 10, seed=2))
+    want = []
+    for s, r in zip(specs, rhos):
+        ctx = lbm.Context(s["params"], s["nx"], s["ny"])
+        ctx.set_density(r)
+        ctx.step(s["nsteps"])
+        want.append(ctx.populations())
+        ctx.close()
+    b = lbm.Batch(specs, rhos)
+    cudart = ctypes.CDLL("libcudart.so.13")
+    stream = ctypes.c_void_p(lbm._lib().lbm_batch_stream(b.h))
+    assert cudart.cudaStreamBeginCapture(stream, 2) == 0  # relaxed
+    with pytest.raises(lbm.LBMError):
+        b.run()
+    graph = ctypes.c_void_p()
+    cudart.cudaStreamEndCapture(stream, ctypes.byref(graph))
+    if graph:
+        cudart.cudaGraphDestroy(graph)
+    cudart.cudaGetLastError()
+    b.run()
+    for i, w in enumerate(want):
+        assert np.array_equal(b.populations(i), w), i
+    b.close()
