@@ -976,8 +976,11 @@ extern "C" int lbm_batch_create(int n, const lbm_batch_lattice* specs, const dou
     cudaError_t e = allocate(true);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();  // (not an error of the calls below)
-        for (int i = 0; i < n; ++i) b->rho0.emplace_back(rho0[i], rho0[i] + (size_t)specs[i].nx * specs[i].ny);
-        e = allocate(false);
+        try {
+            for (int i = 0; i < n; ++i) b->rho0.emplace_back(rho0[i], rho0[i] + (size_t)specs[i].nx * specs[i].ny);
+            e = allocate(false);
+        } catch (const std::bad_alloc&) {  // no room on the host either: the device's error stands
+        }
     }
     if (e != cudaSuccess) {
         delete b;
